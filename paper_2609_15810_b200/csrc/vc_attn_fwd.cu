@@ -287,8 +287,6 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
     mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
     sh->abort = 0;
-    sh->wait_limit = a.wait_limit;
-    sh->wait_hint_ns = a.wait_hint_ns;
     mbar_fence_init();
     tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_mu);
   }
@@ -318,7 +316,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       for (; j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         unsigned char* base = sStage + st * kStageBytes;
-        if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.status, 11)) break;
+        if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.wait, 11)) break;
         if (elect_one()) {
           mbar_expect_tx(&sh->kv_full[st], kKBytes + kVBytes + kMuBytes);
           tma_load_3d(base, &tm_k, &sh->kv_full[st], 0, j * 128, bh);
@@ -337,16 +335,16 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // that neither kind of MMA ever waits behind a barrier that only the other kind needs.)
       const uint32_t idesc_qk = INT8 ? idesc_s8(128, 128) : idesc_e4m3(128, 128);
       const uint64_t dq0 = smem_desc_kmajor(smem_u32(sQ), D), dq1 = smem_desc_kmajor(smem_u32(sQ + kQBytes), D);
-      bool ok = warp_wait2(&sh->q_full, 0, sh, a.status, 20);
+      bool ok = warp_wait2(&sh->q_full, 0, sh, a.wait, 20);
       for (int j = 0; ok && j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
-        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.status, 21))) break;
+        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.wait, 21))) break;
         const uint64_t dk = smem_desc_kmajor(smem_u32(sStage + st * kStageBytes), D);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           // S_0(j) waits for the read of S_1(j-1), S_1(j) for the read of S_0(j)
           if (t == 0 ? j > 0 : true) {
-            if (!(ok = warp_wait2(&sh->s_free[1 - t], (t == 0 ? j - 1 : j) & 1, sh, a.status, 22))) break;
+            if (!(ok = warp_wait2(&sh->s_free[1 - t], (t == 0 ? j - 1 : j) & 1, sh, a.wait, 22))) break;
           }
           if (elect_one()) {
             tc_fence_after();
@@ -373,12 +371,12 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       for (int j = 0; ok && j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         const int stp = (j + kStages2 - 1) % kStages2;    // stage of tile j-1
-        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.status, 25))) break;
+        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.wait, 25))) break;
         const uint64_t dv = smem_desc_kmajor(smem_u32(sStage + st * kStageBytes + kKBytes), 128);
         const uint64_t dm = smem_desc_kmajor(smem_u32(sStage + stp * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-          if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.status, 23))) break;
+          if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 23))) break;
           if (elect_one()) {
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
@@ -394,7 +392,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const uint64_t dml = smem_desc_kmajor(smem_u32(sStage + ((nb - 1) % kStages2) * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {                       // mean term of the last tile
-        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.status, 27))) break;
+        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
         if (elect_one()) {
           tc_fence_after();
           mma_tf32_ss(tmem + O_COL + O_STRIDE * t, dam[t], dml, idesc_mu, 1);
@@ -419,7 +417,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const int ph = j & 1;
       const float cs = (sq * sk_next) * a.sl;             // code units -> log2 domain
       if (j + 1 < nb) sk_next = __ldg(&a.k_scale[(size_t)bh * nb + j + 1]);
-      if (!warp_wait2(&sh->s_full[t], ph, sh, a.status, 30)) break;
+      if (!warp_wait2(&sh->s_full[t], ph, sh, a.wait, 30)) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
       tmem_ld32(lane_base, s0); tmem_ld32(lane_base + 32, s1); tmem_ld32(lane_base + 64, s2); tmem_ld32(lane_base + 96, s3);
@@ -473,7 +471,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       mbar_arrive(&sh->a_full[t][j & 1]);
       m_run = m_new;
       // the previous code tile must have been consumed before it is overwritten
-      if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.status, 31)) break;
+      if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31)) break;
 
       const float fa = cs * 0.0625f, fb = (a.code_off - 8.0f * m_new) * 0.0078125f, nm = 8.0f - m_new;
       const uint64_t fa2 = pack_f32x2(fa, fa), fb2 = pack_f32x2(fb, fb);
@@ -527,10 +525,10 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
-      if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.status, 40))) break;
+      if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 40))) break;
       const float alpha = sh->alpha[t][row];
       if (j > 0) {
-        if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.status, 41))) break;
+        if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 41))) break;
         tc_fence_after();
         l_now = __uint_as_float(tmem_ld1(o_base + L_COL));   // l after tile j-1
         tmem_wait_ld();
@@ -556,14 +554,14 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
     // ---- last tile's mean term, then the epilogue: O = s_V * A / l
-    if (ok && (ok = warp_wait2(&sh->o_done[t], (nb - 1) & 1, sh, a.status, 42))) {
+    if (ok && (ok = warp_wait2(&sh->o_done[t], (nb - 1) & 1, sh, a.wait, 42))) {
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
       tmem_wait_ld();
       put_pair(l_now - l_resc);
       mbar_arrive(&sh->fin_full[t]);
     }
-    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.status, 43)) {
+    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43)) {
       tc_fence_after();
       const int grow = qblk * 128 + row;
       const float inv_l = 1.0f / l_now;
@@ -827,8 +825,7 @@ cudaError_t run8(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   a.N = pr.N; a.n_pad = pr.n_pad; a.nb = pr.nb; a.p_format = pr.p_format;
   a.sl = pr.softmax_scale * 1.4426950408889634f;
   a.code_off = 120.0f + pr.beta;
-  a.wait_limit = attn_wait_limit();
-  a.wait_hint_ns = attn_wait_hint_ns();
+  a.wait = {a.status, attn_wait_limit(), attn_wait_hint_ns()};
   cudaError_t e;
   if (pr.kernel_variant == 1) {     // serial reference kernel
     const size_t smem = 1024 + 2 * 128 * D + D * 128 + D * 4 + 64;

@@ -87,8 +87,7 @@ struct Attn4Args {
   int N, n_pad, nb;
   float sl;                        // softmax_scale * log2(e)
   float code_off;                  // 120 + beta  (Eq. 7; hybrid arrangement only)
-  uint32_t wait_limit;             // polls after which a wait gives up
-  uint32_t wait_hint_ns;
+  WaitArgs wait;
 };
 
 // Value of a non-negative E4M3 byte.
@@ -150,8 +149,6 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
     sh->abort = 0;
-    sh->wait_limit = a.wait_limit;
-    sh->wait_hint_ns = a.wait_hint_ns;
     mbar_fence_init();
     tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_mu);
   }
@@ -190,7 +187,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       for (; j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         unsigned char* base = sStage + st * kStageBytes;
-        if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.status, 11)) break;
+        if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.wait, 11)) break;
         if (elect_one()) {
           mbar_expect_tx(&sh->kv_full[st], kKBytes + kVTx + kMuBytes + kSfBytes);
           tma_load_3d(base, &tm_k, &sh->kv_full[st], 0, j * 128, bh);
@@ -206,7 +203,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // ------------------------------------------------------------------ score issuer
       const uint32_t idesc_qk = idesc_nvfp4(128, 128);
       const uint64_t dq0 = smem_desc_kmajor(smem_u32(sQ), kRowB), dq1 = smem_desc_kmajor(smem_u32(sQ + kQBytes), kRowB);
-      bool ok = warp_wait2(&sh->q_full, 0, sh, a.status, 20);
+      bool ok = warp_wait2(&sh->q_full, 0, sh, a.wait, 20);
       if (ok && elect_one()) {
         for (int t = 0; t < 2; ++t)
           for (int kb = 0; kb < KB; ++kb)
@@ -215,14 +212,14 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       __syncwarp();
       for (int j = 0; ok && j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
-        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.status, 21))) break;
+        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.wait, 21))) break;
         const unsigned char* base = sStage + st * kStageBytes;
         const uint64_t dk = smem_desc_kmajor(smem_u32(base), kRowB);
         const uint32_t sf_smem = smem_u32(base + kKBytes + kVBytes + kOnesBytes + kMuPad);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           if (t == 0 ? j > 0 : true) {
-            if (!(ok = warp_wait2(&sh->s_free[1 - t], (t == 0 ? j - 1 : j) & 1, sh, a.status, 22))) break;
+            if (!(ok = warp_wait2(&sh->s_free[1 - t], (t == 0 ? j - 1 : j) & 1, sh, a.wait, 22))) break;
           }
           if (elect_one()) {
             tc_fence_after();
@@ -258,14 +255,14 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       for (int j = 0; ok && j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         const int stp = (j + kStages2 - 1) % kStages2;    // stage of tile j-1
-        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.status, 25))) break;
+        if (!(ok = warp_wait2(&sh->kv_full[st], it & 1, sh, a.wait, 25))) break;
         const unsigned char* base = sStage + st * kStageBytes;
         const uint64_t dv = smem_desc_kmajor(smem_u32(base + kKBytes), kVRow);
         const uint64_t dm = smem_desc_kmajor(smem_u32(sStage + stp * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
         const uint32_t sfv_smem = smem_u32(base + kKBytes + kVBytes + kOnesBytes + kMuPad + KB * 512);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-          if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.status, 23))) break;
+          if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 23))) break;
           if (elect_one()) {
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
@@ -297,7 +294,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const uint64_t dml = smem_desc_kmajor(smem_u32(sStage + ((nb - 1) % kStages2) * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {                       // mean term of the last tile
-        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.status, 27))) break;
+        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
         if (elect_one()) {
           tc_fence_after();
           mma_tf32_ss(tmem + O_COL + O_STRIDE * t, dam[t], dml, idesc_mu, 1);
@@ -321,7 +318,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     float m_run = -INFINITY;
     for (int j = 0; j < nb; ++j) {
       const int ph = j & 1;
-      if (!warp_wait2(&sh->s_full[t], ph, sh, a.status, 30)) break;
+      if (!warp_wait2(&sh->s_full[t], ph, sh, a.wait, 30)) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
       tmem_ld32(lane_base, s0); tmem_ld32(lane_base + 32, s1); tmem_ld32(lane_base + 64, s2); tmem_ld32(lane_base + 96, s3);
@@ -365,7 +362,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if constexpr (HYB) {
         // ExpCast-FP8 (Eq. 7): t = (8 u + 120 + beta) / 128, code = round-to-nearest-even(128 t)
         // clipped at 0 (two packed FP32 instructions and a saturating pack per two scores)
-        if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.status, 31)) break;
+        if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31)) break;
         const float fa = cs * 0.0625f, fb = (a.code_off - 8.0f * m_new) * 0.0078125f;
         const uint64_t fa2 = pack_f32x2(fa, fa), fb2 = pack_f32x2(fb, fb);
         auto code4 = [&](const uint32_t (&sv)[32], int w) -> uint32_t {
@@ -396,7 +393,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         off[g] = sb ? c0 - lg2_approx(decode_ue4m3(sb)) : -INFINITY;
       }
       // the previous code tile must have been consumed before it is overwritten
-      if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.status, 31)) break;
+      if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31)) break;
 
       const uint64_t cs2 = pack_f32x2(cs, cs);
       auto quant16 = [&](const uint32_t (&sv)[32], int half, int g) -> uint2 {   // keys 16 g .. 16 g + 15
@@ -439,10 +436,10 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
-      if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.status, 40))) break;
+      if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 40))) break;
       const float alpha = sh->alpha[t][row];
       if (j > 0) {
-        if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.status, 41))) break;
+        if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 41))) break;
         tc_fence_after();
         l_now = __uint_as_float(tmem_ld1(o_base + L_COL));   // l after tile j-1
         tmem_wait_ld();
@@ -468,14 +465,14 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
     // ---- last tile's mean term, then the epilogue: O = A / l (means are unscaled at 4 bits, App. B)
-    if (ok && (ok = warp_wait2(&sh->o_done[t], (nb - 1) & 1, sh, a.status, 42))) {
+    if (ok && (ok = warp_wait2(&sh->o_done[t], (nb - 1) & 1, sh, a.wait, 42))) {
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
       tmem_wait_ld();
       put_pair(l_now - l_resc);
       mbar_arrive(&sh->fin_full[t]);
     }
-    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.status, 43)) {
+    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43)) {
       tc_fence_after();
       const int grow = qblk * 128 + row;
       const float inv_l = 1.0f / l_now;
@@ -530,8 +527,7 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   a.N = pr.N; a.n_pad = pr.n_pad; a.nb = pr.nb;
   a.sl = pr.softmax_scale * 1.4426950408889634f;
   a.code_off = 120.0f + pr.beta;
-  a.wait_limit = attn_wait_limit();
-  a.wait_hint_ns = attn_wait_hint_ns();
+  a.wait = {a.status, attn_wait_limit(), attn_wait_hint_ns()};
   constexpr size_t stage = 128 * (D / 2) + (D + 16) * kVRow + ((D * 32 + 1023) / 1024) * 1024 + (((KB + NVC) * 512 + 1023) / 1024) * 1024;
   constexpr size_t smem = 1024 + 2 * 128 * (D / 2) + 2 * 128 * kVRow + 2 * 128 * 32 + 2 * 1024 + 2 * 1024 + 1024 + kStages2 * stage + sizeof(FaSmem);
   static_assert(smem <= 227 * 1024, "shared memory of the 4-bit kernel exceeds the SM");

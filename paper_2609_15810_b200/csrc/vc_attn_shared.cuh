@@ -16,6 +16,12 @@ using namespace sm100;
 
 constexpr uint32_t kErrTimeout = kStatusTimeout;
 
+// Where a wait that gives up says so, the polls after which it does, and how long one may sleep.
+struct WaitArgs {
+  uint32_t* status;
+  uint32_t limit, hint_ns;
+};
+
 // Arguments of the 8-bit attention kernels.
 struct AttnArgs {
   const float *q_scale, *k_scale, *v_scale;
@@ -25,8 +31,7 @@ struct AttnArgs {
   int N, n_pad, nb, p_format;
   float sl;        // softmax_scale * log2(e)
   float code_off;  // 120 + beta  (Eq. 7)
-  uint32_t wait_limit;   // polls after which a wait gives up
-  uint32_t wait_hint_ns;
+  WaitArgs wait;
 };
 
 constexpr int kStages2 = 4;
@@ -50,31 +55,34 @@ struct FaSmem {
   uint64_t drain[2];      // exit: "every MMA this issuer warp issued has completed"
   float alpha[2][128];
   uint32_t tmem_base;
-  uint32_t wait_limit;    // polls of a wait ...
-  uint32_t wait_hint_ns;  // ... each of which may sleep this long in hardware
   volatile int abort;
 };
 
-__device__ __forceinline__ bool wait2(uint64_t* bar, uint32_t parity, FaSmem* sh, uint32_t* status, uint32_t code) {
-  const uint32_t limit = sh->wait_limit, hint = sh->wait_hint_ns;
-  if (hint) {
-    if (mbar_try_wait(bar, parity)) return true;
-    for (uint32_t i = 0; i < limit; ++i) {
-      if (mbar_try_wait_hint(bar, parity, hint)) return true;
-      if ((i & 63u) == 63u && sh->abort) return false;
+// Bounded wait of a whole warp.  A key tile's critical chain holds a dozen of these and many find
+// their phase complete, so a wait starts with a bare non-blocking test and a vote (about 30 cycles);
+// behind it the loop that sleeps in hardware wakes up through one vote as well, and its limits are
+// kernel arguments, not loads.  (With the limits read from shared memory in front of the first test
+// and the vote behind the loop a completed wait took 170 cycles.  8-bit kernel at B1 H12 N32760 d128:
+// 3.52 -> 3.34 ms, at B2 H16 N16384 d64: 2.21 -> 1.94 ms; hybrid 3.40 -> 3.26, NVFP4 5.66 -> 5.28 ms.)
+// hint_ns = 0 (test hook): the polls never sleep.
+__device__ __forceinline__ bool warp_wait2(uint64_t* bar, uint32_t parity, FaSmem* sh, const WaitArgs& w, uint32_t code) {
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+  if (w.hint_ns) {
+#pragma unroll 1
+    for (uint32_t i = 0; i < w.limit; ++i) {
+      if (__all_sync(0xffffffffu, mbar_try_wait_hint(bar, parity, w.hint_ns))) return true;
+      if ((i & 63u) == 63u && __any_sync(0xffffffffu, sh->abort)) return false;
     }
-  } else {                                     // test hook: polls that never sleep
-    for (uint32_t i = 0; i < limit; ++i) {
-      if (mbar_test_wait(bar, parity)) return true;
-      if ((i & 63u) == 63u && sh->abort) return false;
+  } else {
+#pragma unroll 1
+    for (uint32_t i = 0; i < w.limit; ++i) {
+      if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+      if ((i & 63u) == 63u && __any_sync(0xffffffffu, sh->abort)) return false;
     }
   }
   sh->abort = 1;
-  atomicExch(status, kErrTimeout | code);
+  atomicExch(w.status, kErrTimeout | code);
   return false;
-}
-__device__ __forceinline__ bool warp_wait2(uint64_t* bar, uint32_t parity, FaSmem* sh, uint32_t* status, uint32_t code) {
-  return __all_sync(0xffffffffu, wait2(bar, parity, sh, status, code));
 }
 
 // Exit protocol of the pipelined kernels.  A CTA may leave early (a wait gave up and set `abort`),
