@@ -125,9 +125,7 @@ WorkLayout work_layout(const Problem& pr) {
   W.amax = place(W.amax_bytes);
   W.perm_bits_bytes = (pr.flags & VC_FLAG_CHECK_PERM) ? BH * (((size_t)pr.N + 31) / 32) * 4 : 0;
   W.perm_bits = place(W.perm_bits_bytes);
-  W.mu_mma = place(BH * nb * d * 32);
-  W.sf_q = place(pr.bits == 4 ? BH * nb * (d / 64) * 512 : 0);
-  W.sf_kv = place(pr.bits == 4 ? BH * nb * (d / 64 + 2) * 512 : 0);
+  W.prep_end = off;
   W.expand = place(pr.bits == 4 && pr.kernel_variant == 1 ? 3 * BH * (size_t)pr.n_pad * d * 2 : 0);
   W.total = off;
   return W;

@@ -251,11 +251,13 @@ __device__ __forceinline__ float exp2_poly(float x) {
   return __uint_as_float(__float_as_uint(p) + (__float_as_uint(t) << 23));
 }
 
-template <int D, int PF, bool INT8>
+// SMOOTH = false: value smoothing is off, every block mean is zero and the mean term falls away (no mean
+// operand, no TF32 product, no per-tile read of l).  A launch argument instead of a template
+// parameter costs 1 % of the kernel with smoothing on.
+template <int D, int PF, bool INT8, bool SMOOTH>
 __global__ void __launch_bounds__(640, 1)
 attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_mu,
-                   const AttnArgs a) {
+                   const __grid_constant__ CUtensorMap tm_v, const AttnArgs a) {
   constexpr int kTmemCols = 512;
   constexpr uint32_t O_COL = 128, O_STRIDE = 144, L_COL = D;   // A_t at O_COL + t * O_STRIDE; l in its column d
   // Register re-partition (setmaxnreg): the CTA owns 640 x 96 registers; a warpgroup that asks for
@@ -288,9 +290,11 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
     sh->abort = 0;
     mbar_fence_init();
-    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_mu);
+    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
   }
   for (int i = tid; i < 2 * (int)kAmBytes / 16; i += 640) reinterpret_cast<uint4*>(sAm)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < kStages2 * (int)kMuBytes / 16; i += 640)
+    reinterpret_cast<uint4*>(sStage + (i / (kMuBytes / 16)) * kStageBytes + kKBytes + kVBytes + kOnesBytes)[i % (kMuBytes / 16)] = make_uint4(0, 0, 0, 0);
   // 16 rows of E4M3 1.0 behind every value tile (the rows are uniform, so the swizzle is moot)
   for (int i = tid; i < kStages2 * (int)kOnesBytes / 4; i += 640)
     reinterpret_cast<uint32_t*>(sStage + (i / (kOnesBytes / 4)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 4)] = 0x38383838u;
@@ -306,7 +310,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     reg_dec<kRegCtl>();
     if (warp == 0) {
       // ------------------------------------------------------------------ TMA producer
-      // (the whole warp runs the loop; one elected lane issues the copies)
+      // (the whole warp runs the loop: one elected lane issues the copies, all write the block means)
       if (elect_one()) {
         mbar_expect_tx(&sh->q_full, 2 * kQBytes);
         tma_load_3d(sQ, &tm_q, &sh->q_full, 0, (2 * qpair) * 128, bh);
@@ -316,13 +320,20 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       for (; j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         unsigned char* base = sStage + st * kStageBytes;
+        MeanRows<D> mu;
+        if (SMOOTH) mu.fetch(a.v_means + ((size_t)bh * nb + j) * D, lane);
         if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.wait, 11)) break;
         if (elect_one()) {
-          mbar_expect_tx(&sh->kv_full[st], kKBytes + kVBytes + kMuBytes);
+          mbar_expect_tx_only(&sh->kv_full[st], kKBytes + kVBytes);
           tma_load_3d(base, &tm_k, &sh->kv_full[st], 0, j * 128, bh);
           tma_load_3d(base + kKBytes, &tm_v, &sh->kv_full[st], j * 128, 0, bh);
-          tma_load_3d(base + kKBytes + kVBytes + kOnesBytes, &tm_mu, &sh->kv_full[st], 0, 0, bh * nb + j);
         }
+        if (SMOOTH) {
+          mu.store(base + kKBytes + kVBytes + kOnesBytes, lane);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the stores -> tensor-core reads
+        }
+        __syncwarp();
+        if (elect_one()) mbar_arrive(&sh->kv_full[st]);
         __syncwarp();
       }
       drain_loads(sh, j);                                 // (returns at once on a normal run)
@@ -382,7 +393,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
 #pragma unroll
             for (int k = 0; k < 4; ++k) mma_f8_ss(o_col, dp[t] + 2 * k, dv + 2 * k, idesc_pv, (j > 0) | (k > 0));
-            if (j > 0) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
+            if (j > 0 && SMOOTH) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
             mma_commit(&sh->o_done[t]);
             if (j > 0) mma_commit(&sh->kv_empty[stp]);    // this tile is done with stage j-1
           }
@@ -392,7 +403,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const uint64_t dml = smem_desc_kmajor(smem_u32(sStage + ((nb - 1) % kStages2) * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {                       // mean term of the last tile
-        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
+        if (!SMOOTH || !ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
         if (elect_one()) {
           tc_fence_after();
           mma_tf32_ss(tmem + O_COL + O_STRIDE * t, dam[t], dml, idesc_mu, 1);
@@ -409,8 +420,9 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int row = (warp & 3) * 32 + lane;
     const int qblk = 2 * qpair + t;
     // my row of the swizzled code tile: 16-byte chunk c sits at chunk position c ^ (row % 8)
-    unsigned char* p_row = sP + t * kPBytes + (row >> 3) * 1024 + (row & 7) * 128;
+    const uint32_t p_row = smem_u32(sP + t * kPBytes + row * 128) + ((row & 7) << 4);
     const float sq = qblk < nb ? a.q_scale[(size_t)bh * nb + qblk] : 1.0f;
+    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
     float m_run = -INFINITY;
     float sk_next = __ldg(&a.k_scale[(size_t)bh * nb]);   // fetched one tile ahead: an L2 round trip
     for (int j = 0; j < nb; ++j) {
@@ -467,7 +479,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       }
       const float mxa = max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
       const float m_new = fmaxf(m_run, mxa * cs);         // m' = max(m, rowmax S_ij)
-      sh->alpha[t][row] = ex2_approx(m_run - m_new);      // alpha; 0 on the first tile
+      sts32(alpha_at, ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
       mbar_arrive(&sh->a_full[t][j & 1]);
       m_run = m_new;
       // the previous code tile must have been consumed before it is overwritten
@@ -499,8 +511,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         }
       };
       auto store16 = [&](const uint32_t (&sv)[32], int half, int chunk) {   // keys 16*chunk .. +15
-        const uint4 v = make_uint4(code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
-        *reinterpret_cast<uint4*>(p_row + ((chunk ^ (row & 7)) << 4)) = v;
+        sts128(p_row ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
       };
       store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
       store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
@@ -515,32 +526,35 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int qblk = 2 * qpair + t;
     const uint32_t o_base = lane_base + O_COL + O_STRIDE * t;
     // my row of the row-sum operand: 32-byte rows, the two 16-byte chunks swap when (row / 4) is odd
-    uint4* am_row = reinterpret_cast<uint4*>(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
+    const uint32_t am_row = smem_u32(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
+    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
     float l_resc = 0.f;       // l as it stands in column d after the latest rescale, before the tile's own sum
     float l_now = 0.f;
     bool ok = true;
     auto put_pair = [&](float rho) {                      // (rho_hi, rho_lo, 0, 0) for the mean MMA
       const uint32_t hi = (__float_as_uint(rho) + 0x1000u) & 0xffffe000u;   // nearest TF32
-      *am_row = make_uint4(hi, __float_as_uint(rho - __uint_as_float(hi)), 0u, 0u);
+      sts128(am_row, hi, __float_as_uint(rho - __uint_as_float(hi)), 0u, 0u);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
       if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 40))) break;
-      const float alpha = sh->alpha[t][row];
-      if (j > 0) {
+      const float alpha = lds32(alpha_at);
+      const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);   // a row maximum of the warp moved
+      // (without block means nothing needs l tile by tile: a warp whose maxima stand still passes on)
+      if (j > 0 && (SMOOTH || moved)) {
         if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 41))) break;
         tc_fence_after();
         l_now = __uint_as_float(tmem_ld1(o_base + L_COL));   // l after tile j-1
         tmem_wait_ld();
         const float r_prev = l_now - l_resc;                 // r_{j-1} = P~ 1 over the decoded codes
-        if (__any_sync(0xffffffffu, alpha != 1.0f)) {        // a row maximum moved: A <- alpha A (l included)
+        if (moved) {                                         // A <- alpha A (l included)
           uint32_t r[16];
 #pragma unroll 1
           for (int c = 0; c < D / 16; ++c) {
             tmem_ld16(o_base + 16 * c, r);
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+            for (int i = 0; i < 16; i += 2) unpack_b32x2(mul2(pack_b32x2(r[i], r[i + 1]), pack_f32x2(alpha, alpha)), r[i], r[i + 1]);
             tmem_st16(o_base + 16 * c, r);
           }
           // of the 16 row-sum columns only column d is ever read, and its value is at hand
@@ -549,7 +563,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tc_fence_before();
         }
         l_resc = l_now * alpha;
-        put_pair(r_prev * alpha);                            // added after the rescale, so referenced to m_j
+        if (SMOOTH) put_pair(r_prev * alpha);              // added after the rescale, so referenced to m_j
       }
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
@@ -558,10 +572,12 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
       tmem_wait_ld();
-      put_pair(l_now - l_resc);
-      mbar_arrive(&sh->fin_full[t]);
+      if (SMOOTH) {
+        put_pair(l_now - l_resc);
+        mbar_arrive(&sh->fin_full[t]);
+      }
     }
-    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43)) {
+    if (ok && (!SMOOTH || warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43))) {
       tc_fence_after();
       const int grow = qblk * 128 + row;
       const float inv_l = 1.0f / l_now;
@@ -825,7 +841,7 @@ cudaError_t run8(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   a.N = pr.N; a.n_pad = pr.n_pad; a.nb = pr.nb; a.p_format = pr.p_format;
   a.sl = pr.softmax_scale * 1.4426950408889634f;
   a.code_off = 120.0f + pr.beta;
-  a.wait = {a.status, attn_wait_limit(), attn_wait_hint_ns()};
+  a.wait = {a.status, attn_wait_limit(), attn_wait_nonblocking()};
   cudaError_t e;
   if (pr.kernel_variant == 1) {     // serial reference kernel
     const size_t smem = 1024 + 2 * 128 * D + D * 128 + D * 4 + 64;
@@ -835,34 +851,29 @@ cudaError_t run8(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
     return cudaGetLastError();
   }
   if (pr.kernel_variant == 0) {     // two query tiles per CTA (default)
-    alignas(64) CUtensorMap tmt;
-    if (!make_map(&tmt, work + wl.mu_mma, 32, D, (uint64_t)pr.BH * pr.nb, 32, D)) return cudaErrorUnknown;
-    const size_t n = (size_t)pr.BH * pr.nb * D;
-    means_tile_layout_kernel<D><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a.v_means, (float*)(work + wl.mu_mma), n);
     const size_t stage = 2 * 128 * D + 2048 + ((D * 32 + 1023) / 1024) * 1024;
     const size_t smem2 = 1024 + 2 * 128 * D + 2 * 128 * 128 + 2 * 128 * 32 + kStages2 * stage + sizeof(FaSmem);
     const dim3 grid((pr.nb + 1) / 2, pr.BH);
     const bool int8 = pr.flags & VC_FLAG_INT8_QK;
-#define VC_LAUNCH_2Q(EC, I8)                                                                                             \
-  {                                                                                                                      \
-    if ((e = cudaFuncSetAttribute(attn_fwd_2q_kernel<D, EC, I8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2)) != cudaSuccess) return e; \
-    attn_fwd_2q_kernel<D, EC, I8><<<grid, 640, smem2, s>>>(tq, tk, tv, tmt, a);                                           \
-  }
+    auto launch = [&](auto kernel) {
+      if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2)) == cudaSuccess)
+        kernel<<<grid, 640, smem2, s>>>(tq, tk, tv, a);
+    };
+    const bool smooth = pr.flags & VC_FLAG_V_SMOOTH;
     const int pf = pr.p_format == VC_P_EXPCAST_E4M3 ? kPfExpCast
                    : pr.p_format == VC_P_EXP_E4M3   ? kPfExp
                    : pr.p_format == VC_P_EXP_POLY_E4M3 ? kPfExpPoly : kPfExpMix;
-    if (int8) {
-      if (pf == kPfExpCast) VC_LAUNCH_2Q(kPfExpCast, true)
-      else if (pf == kPfExp) VC_LAUNCH_2Q(kPfExp, true)
-      else return cudaErrorNotSupported;
-    } else {
-      if (pf == kPfExpCast) VC_LAUNCH_2Q(kPfExpCast, false)
-      else if (pf == kPfExp) VC_LAUNCH_2Q(kPfExp, false)
-      else if (pf == kPfExpPoly) VC_LAUNCH_2Q(kPfExpPoly, false)
-      else VC_LAUNCH_2Q(kPfExpMix, false)
+    if (int8 && pf > kPfExp) return cudaErrorNotSupported;
+    if (pf == kPfExpCast) {
+      if (smooth) int8 ? launch(attn_fwd_2q_kernel<D, kPfExpCast, true, true>) : launch(attn_fwd_2q_kernel<D, kPfExpCast, false, true>);
+      else int8 ? launch(attn_fwd_2q_kernel<D, kPfExpCast, true, false>) : launch(attn_fwd_2q_kernel<D, kPfExpCast, false, false>);
     }
-#undef VC_LAUNCH_2Q
-    count_launches(2);
+    // (the other formats exist for comparison: they add means of zero)
+    else if (pf == kPfExp) int8 ? launch(attn_fwd_2q_kernel<D, kPfExp, true, true>) : launch(attn_fwd_2q_kernel<D, kPfExp, false, true>);
+    else if (pf == kPfExpPoly) launch(attn_fwd_2q_kernel<D, kPfExpPoly, false, true>);
+    else launch(attn_fwd_2q_kernel<D, kPfExpMix, false, true>);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
     return cudaGetLastError();
   }
   return cudaErrorNotSupported;

@@ -5,8 +5,8 @@
 // under an unsigned E4M3 factor per 16 elements along the contraction axis - and both products
 // run as tcgen05.mma kind::mxf4nvf4 (K = 64 per instruction), which multiplies each 16-element
 // partial sum by the two factors.  The factors live in tensor memory; tcgen05.cp brings them
-// there from shared memory in 512-byte chunks (128 operand rows x 4 groups).  A small pre-pass
-// rewrites the bundle's row-major factor arrays into that chunk order, per 128-row tile.
+// there from shared memory in 512-byte chunks (128 operand rows x 4 groups).  The producer warp
+// reads a tile's factors from the bundle's row-major arrays and writes them in chunk order.
 //
 // The pipeline is the one of the 8-bit kernel (two query tiles per CTA, one shared score
 // buffer, probability codes through shared memory, the row sums l from 16 rows of ones behind
@@ -36,52 +36,46 @@ namespace {
 using namespace sm100;
 using namespace attn;
 
-// Factor arrays -> MMA chunk order.  One CTA per (b, h, 128-row tile), thread r = operand row.
-//   sf_q  [BH*nb][D/64][512]          Q^ factors of query tile
-//   sf_kv [BH*nb][D/64 + 2][512]      K^ factors of key tile, then the R^ factors of the same
-//                                     tile (operand rows = channels, groups = 16 tokens);
-//                                     HYB: [D/64 + 1] chunks, the last one holding the four
-//                                     power-of-two factors (32 tokens each) of every channel
-// Chunk byte 16 (r % 32) + 4 (r / 32) + k  <-  factor of row r, group 4 kb + k.
-template <int D, bool HYB>
-__global__ void __launch_bounds__(128)
-nvfp4_sf_tiles_kernel(const uint8_t* __restrict__ q_micro, const uint8_t* __restrict__ k_micro,
-                      const uint8_t* __restrict__ v_micro, uint8_t* __restrict__ sf_q, uint8_t* __restrict__ sf_kv,
-                      int nb, int n_pad) {
-  constexpr int KB = D / 64, NVC = HYB ? 1 : 2;
-  const int tile = blockIdx.x, bh = blockIdx.y, r = threadIdx.x;
-  const size_t t_idx = (size_t)bh * nb + tile;
-  const uint32_t pos = (r & 31) * 16 + (r >> 5) * 4;
-  const size_t row = (size_t)bh * n_pad + (size_t)tile * 128 + r;
-  const uint32_t* qm = reinterpret_cast<const uint32_t*>(q_micro + row * (D / 16));
-  const uint32_t* km = reinterpret_cast<const uint32_t*>(k_micro + row * (D / 16));
+// Factors in MMA chunk order: chunk byte 16 (r % 32) + 4 (r / 32) + k is the factor of operand row r,
+// group 4 kb + k.  A lane takes rows lane, lane + 32, lane + 64, lane + 96 of the 128: their four
+// words are 16 consecutive bytes of the chunk, one store.  (A launch that rewrote the arrays into
+// chunks for bulk copies cost 7 us and 2 x 9 MB at B1 H12 N32760 d128.)
+template <int W> struct FactorRows {   // W words (of four factors) per row
+  uint32_t w[4][W];
+  __device__ __forceinline__ void fetch_row(int i, const uint8_t* src) {
+    if constexpr (W == 2) {
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
+      w[i][0] = v.x; w[i][1] = v.y;
+    } else {
+      w[i][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+    }
+  }
+  // 128 rows of consecutive bytes (Q^ and K^: rows are tokens, groups run along channels)
+  __device__ __forceinline__ void fetch_tokens(const uint8_t* tile, int lane) {
 #pragma unroll
-  for (int kb = 0; kb < KB; ++kb) {
-    *reinterpret_cast<uint32_t*>(sf_q + t_idx * (KB * 512) + kb * 512 + pos) = qm[kb];
-    *reinterpret_cast<uint32_t*>(sf_kv + t_idx * ((KB + NVC) * 512) + kb * 512 + pos) = km[kb];
+    for (int i = 0; i < 4; ++i) fetch_row(i, tile + (size_t)(lane + 32 * i) * (4 * W));
   }
-  if constexpr (HYB) {
-    uint32_t w = 0;
-    if (r < D) w = *reinterpret_cast<const uint32_t*>(v_micro + ((size_t)bh * D + r) * (n_pad / 32) + (size_t)tile * 4);
-    else if (r < D + 16) w = 0x7f7f7f7fu;   // the rows of ones: factor 2^0
-    *reinterpret_cast<uint32_t*>(sf_kv + t_idx * ((KB + NVC) * 512) + KB * 512 + pos) = w;
-    return;
+  // rows are channels, groups run along tokens; the 16 rows behind the channels are the rows of ones
+  template <int D> __device__ __forceinline__ void fetch_channels(const uint8_t* first, size_t pitch, uint32_t one, int lane) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (32 * i < D) fetch_row(i, first + (size_t)(lane + 32 * i) * pitch);
+      else {
+#pragma unroll
+        for (int k = 0; k < W; ++k) w[i][k] = 32 * i == D && lane < 16 ? one : 0u;
+      }
+    }
   }
-  uint32_t w0 = 0, w1 = 0;
-  if (r < D) {
-    const uint2 vm = *reinterpret_cast<const uint2*>(v_micro + ((size_t)bh * D + r) * (n_pad / 16) + (size_t)tile * 8);
-    w0 = vm.x; w1 = vm.y;
-  } else if (r < D + 16) {
-    w0 = w1 = 0x38383838u;   // the rows of ones behind the value tile carry the factor 1.0
+  __device__ __forceinline__ void store(unsigned char* chunks, int lane) const {
+#pragma unroll
+    for (int k = 0; k < W; ++k) *reinterpret_cast<uint4*>(chunks + 512 * k + 16 * lane) = make_uint4(w[0][k], w[1][k], w[2][k], w[3][k]);
   }
-  uint8_t* dst = sf_kv + t_idx * ((KB + 2) * 512) + KB * 512 + pos;
-  *reinterpret_cast<uint32_t*>(dst) = w0;
-  *reinterpret_cast<uint32_t*>(dst + 512) = w1;
-}
+};
 
 struct Attn4Args {
   const float *q_g, *k_g;          // NVFP4 outer scales per (b, h)
-  const uint8_t *sf_q, *sf_kv;     // factor chunks (see nvfp4_sf_tiles_kernel)
+  const uint8_t *q_micro, *k_micro, *v_micro;
+  const __nv_bfloat16* v_means;
   __nv_bfloat16* o;
   uint32_t* status;
   int N, n_pad, nb;
@@ -103,11 +97,10 @@ __device__ __forceinline__ float decode_ue4m3(uint32_t code) {
 //   warps 4-11    softmax warpgroups (tile 0, tile 1), one thread per query row
 //   warps 12-19   correction warpgroups, one thread per query row
 // Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16) | scale factors (56 columns).
-template <int D, bool HYB>
+template <int D, bool HYB, bool SMOOTH>
 __global__ void __launch_bounds__(640, 1)
 attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_mu,
-                    const Attn4Args a) {
+                    const __grid_constant__ CUtensorMap tm_v, const Attn4Args a) {
   constexpr int kTmemCols = 512;
   constexpr int KB = D / 64;                        // K = 64 steps of the score product
   constexpr int kRowB = D / 2;                      // bytes per Q^/K^ row
@@ -121,7 +114,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   constexpr uint32_t kQBytes = 128 * kRowB, kKBytes = 128 * kRowB, kVBytes = D * kVRow, kOnesBytes = 16 * kVRow;
   constexpr uint32_t kVTx = D * 64;                 // bytes the value copy reports (the packed ones)
   constexpr uint32_t kMuBytes = D * 32, kMuPad = ((kMuBytes + 1023) / 1024) * 1024;
-  constexpr uint32_t kSfqBytes = KB * 512, kSfBytes = (KB + NVC) * 512, kSfPad = ((kSfBytes + 1023) / 1024) * 1024;
+  constexpr uint32_t kSfBytes = (KB + NVC) * 512, kSfPad = ((kSfBytes + 1023) / 1024) * 1024;
   constexpr uint32_t kStageBytes = kKBytes + kVBytes + kOnesBytes + kMuPad + kSfPad;
   constexpr uint32_t kPBytes = 128 * kVRow, kSfpBytes = 1024, kAmBytes = 128 * 32;
   extern __shared__ unsigned char smem_raw[];
@@ -150,9 +143,11 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
     sh->abort = 0;
     mbar_fence_init();
-    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); tma_prefetch_desc(&tm_mu);
+    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
   }
   for (int i = tid; i < 2 * (int)kAmBytes / 16; i += 640) reinterpret_cast<uint4*>(sAm)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < kStages2 * (int)kMuBytes / 16; i += 640)
+    reinterpret_cast<uint4*>(sStage + (i / (kMuBytes / 16)) * kStageBytes + kKBytes + kVBytes + kOnesBytes)[i % (kMuBytes / 16)] = make_uint4(0, 0, 0, 0);
   // 16 rows of E2M1 1.0 (two per byte) behind every value tile; their factor chunk: 1.0 for
   // rows 0..15 of the second 128-row half, group bytes 0..3
   // (HYB: the same bytes, of which the product reads the low 8 of every 16; factor code 127 = 2^0,
@@ -175,27 +170,43 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     reg_dec<kRegCtl>();
     if (warp == 0) {
       // ------------------------------------------------------------------ TMA producer
-      if (elect_one()) {
-        mbar_expect_tx(&sh->q_full, 2 * kQBytes + 2 * kSfqBytes);
-        for (int t = 0; t < 2; ++t) {
-          const int qb = 2 * qpair + t;                    // past the end: zero codes, any factors
-          tma_load_3d(sQ + t * kQBytes, &tm_q, &sh->q_full, 0, qb * 128, bh);
-          bulk_load(sSfq + t * 1024, a.sf_q + ((size_t)bh * nb + min(qb, nb - 1)) * kSfqBytes, kSfqBytes, &sh->q_full);
-        }
+      // (the whole warp runs the loop: one elected lane issues the copies, all write factors and means)
+      FactorRows<KB> fq;
+      if (elect_one()) mbar_expect_tx_only(&sh->q_full, 2 * kQBytes);
+#pragma unroll 1
+      for (int t = 0; t < 2; ++t) {
+        const int qb = 2 * qpair + t;                      // past the end: zero codes, any factors
+        if (elect_one()) tma_load_3d(sQ + t * kQBytes, &tm_q, &sh->q_full, 0, qb * 128, bh);
+        fq.fetch_tokens(a.q_micro + ((size_t)bh * a.n_pad + min(qb, nb - 1) * 128) * (D / 16), lane);
+        fq.store(sSfq + t * 1024, lane);
       }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // the stores -> tensor-core reads
+      __syncwarp();
+      if (elect_one()) mbar_arrive(&sh->q_full);
       int j = 0;
       for (; j < nb; ++j) {
         const int st = j % kStages2, it = j / kStages2;
         unsigned char* base = sStage + st * kStageBytes;
+        unsigned char* extra = base + kKBytes + kVBytes + kOnesBytes;       // block mean, then the factor chunks
+        FactorRows<KB> fk;
+        FactorRows<NVC> fv;
+        MeanRows<D> mu;
+        fk.fetch_tokens(a.k_micro + ((size_t)bh * a.n_pad + j * 128) * (D / 16), lane);
+        if (HYB) fv.template fetch_channels<D>(a.v_micro + (size_t)bh * D * (a.n_pad / 32) + j * 4, a.n_pad / 32, 0x7f7f7f7fu, lane);
+        else fv.template fetch_channels<D>(a.v_micro + (size_t)bh * D * (a.n_pad / 16) + j * 8, a.n_pad / 16, 0x38383838u, lane);
+        if (SMOOTH) mu.fetch(a.v_means + ((size_t)bh * nb + j) * D, lane);
         if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.wait, 11)) break;
         if (elect_one()) {
-          mbar_expect_tx(&sh->kv_full[st], kKBytes + kVTx + kMuBytes + kSfBytes);
+          mbar_expect_tx_only(&sh->kv_full[st], kKBytes + kVTx);
           tma_load_3d(base, &tm_k, &sh->kv_full[st], 0, j * 128, bh);
           tma_load_3d(base + kKBytes, &tm_v, &sh->kv_full[st], HYB ? j * 128 : j * 64, 0, bh);   // elements resp. bytes
-          tma_load_3d(base + kKBytes + kVBytes + kOnesBytes, &tm_mu, &sh->kv_full[st], 0, 0, bh * nb + j);
-          bulk_load(base + kKBytes + kVBytes + kOnesBytes + kMuPad, a.sf_kv + ((size_t)bh * nb + j) * kSfBytes, kSfBytes,
-                    &sh->kv_full[st]);
         }
+        fk.store(extra + kMuPad, lane);
+        fv.store(extra + kMuPad + KB * 512, lane);
+        if (SMOOTH) mu.store(extra, lane);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // the stores -> tensor-core reads
+        __syncwarp();
+        if (elect_one()) mbar_arrive(&sh->kv_full[st]);
         __syncwarp();
       }
       drain_loads(sh, j);                                 // (returns at once on a normal run)
@@ -284,7 +295,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 mma_nvfp4_ss(o_col, dp[t] + 2 * kb, dv + 2 * kb, idesc_pv, (j > 0) | (kb > 0), tmem + SFP_COL + t * 8 + kb * 4,
                              tmem + SFV_COL + kb * 8);
             }
-            if (j > 0) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
+            if (j > 0 && SMOOTH) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
             mma_commit(&sh->o_done[t]);
             if (j > 0) mma_commit(&sh->kv_empty[stp]);    // this tile is done with stage j-1
           }
@@ -294,7 +305,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const uint64_t dml = smem_desc_kmajor(smem_u32(sStage + ((nb - 1) % kStages2) * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
       for (int t = 0; t < 2; ++t) {                       // mean term of the last tile
-        if (!ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
+        if (!SMOOTH || !ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
         if (elect_one()) {
           tc_fence_after();
           mma_tf32_ss(tmem + O_COL + O_STRIDE * t, dam[t], dml, idesc_mu, 1);
@@ -311,10 +322,10 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int row = (warp & 3) * 32 + lane;
     // my row of the swizzled code tile: 64-byte rows, chunk c sits at chunk position c ^ ((row / 2) % 4)
     // (HYB: 128-byte rows, chunk c at position c ^ (row % 8))
-    unsigned char* p_row = sP + t * kPBytes + row * kVRow;
-    const int p_xor = (row >> 1) & 3;
-    uint32_t* sfp_row = reinterpret_cast<uint32_t*>(sSfp + t * kSfpBytes + (row & 31) * 16 + (row >> 5) * 4);
+    const uint32_t p_row = smem_u32(sP + t * kPBytes + row * kVRow) + ((HYB ? row & 7 : (row >> 1) & 3) << 4);
+    const uint32_t sfp_row = smem_u32(sSfp + t * kSfpBytes + (row & 31) * 16 + (row >> 5) * 4);
     const float cs = (a.q_g[bh] * a.k_g[bh]) * a.sl;       // code units -> log2 domain
+    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
     float m_run = -INFINITY;
     for (int j = 0; j < nb; ++j) {
       const int ph = j & 1;
@@ -356,7 +367,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       const float mxa = max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
       const float m_new = fmaxf(m_run, mxa * cs);         // m' = max(m, rowmax S_ij)
-      sh->alpha[t][row] = ex2_approx(m_run - m_new);      // alpha; 0 on the first tile
+      sts32(alpha_at, ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
       mbar_arrive(&sh->a_full[t][j & 1]);
       m_run = m_new;
       if constexpr (HYB) {
@@ -369,8 +380,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           return expcast_codes4(sv[4 * w], sv[4 * w + 1], sv[4 * w + 2], sv[4 * w + 3], fa2, fb2);
         };
         auto store16 = [&](const uint32_t (&sv)[32], int half, int chunk) {   // keys 16 chunk .. +15
-          const uint4 v = make_uint4(code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
-          *reinterpret_cast<uint4*>(p_row + ((chunk ^ (row & 7)) << 4)) = v;
+          sts128(p_row ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
         };
         store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
         store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
@@ -411,11 +421,11 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       };
       auto store32 = [&](const uint32_t (&sv)[32], int chunk) {   // keys 32 chunk .. +31 -> 16 bytes
         const uint2 lo = quant16(sv, 0, 2 * chunk), hi = quant16(sv, 1, 2 * chunk + 1);
-        *reinterpret_cast<uint4*>(p_row + ((chunk ^ p_xor) << 4)) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+        sts128(p_row ^ (chunk << 4), lo.x, lo.y, hi.x, hi.y);
       };
       store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
-      sfp_row[0] = sfw[0];
-      sfp_row[128] = sfw[1];                               // the chunk of keys 64..127
+      sts32(sfp_row, __uint_as_float(sfw[0]));
+      sts32(sfp_row + 512, __uint_as_float(sfw[1]));                               // the chunk of keys 64..127
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
@@ -426,32 +436,35 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int row = (warp & 3) * 32 + lane;
     const int qblk = 2 * qpair + t;
     const uint32_t o_base = lane_base + O_COL + O_STRIDE * t;
-    uint4* am_row = reinterpret_cast<uint4*>(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
+    const uint32_t am_row = smem_u32(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
+    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
     float l_resc = 0.f;       // l as it stands in column d after the latest rescale, before the tile's own sum
     float l_now = 0.f;
     bool ok = true;
     auto put_pair = [&](float rho) {                      // (rho_hi, rho_lo, 0, 0) for the mean MMA
       const uint32_t hi = (__float_as_uint(rho) + 0x1000u) & 0xffffe000u;   // nearest TF32
-      *am_row = make_uint4(hi, __float_as_uint(rho - __uint_as_float(hi)), 0u, 0u);
+      sts128(am_row, hi, __float_as_uint(rho - __uint_as_float(hi)), 0u, 0u);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
       if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 40))) break;
-      const float alpha = sh->alpha[t][row];
-      if (j > 0) {
+      const float alpha = lds32(alpha_at);
+      const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);   // a row maximum of the warp moved
+      // (without block means nothing needs l tile by tile: a warp whose maxima stand still passes on)
+      if (j > 0 && (SMOOTH || moved)) {
         if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 41))) break;
         tc_fence_after();
         l_now = __uint_as_float(tmem_ld1(o_base + L_COL));   // l after tile j-1
         tmem_wait_ld();
         const float r_prev = l_now - l_resc;                 // r_{j-1}: sum of the decoded codes
-        if (__any_sync(0xffffffffu, alpha != 1.0f)) {        // a row maximum moved: A <- alpha A (l included)
+        if (moved) {                                         // A <- alpha A (l included)
           uint32_t r[16];
 #pragma unroll 1
           for (int c = 0; c < D / 16; ++c) {
             tmem_ld16(o_base + 16 * c, r);
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
+            for (int i = 0; i < 16; i += 2) unpack_b32x2(mul2(pack_b32x2(r[i], r[i + 1]), pack_f32x2(alpha, alpha)), r[i], r[i + 1]);
             tmem_st16(o_base + 16 * c, r);
           }
           // of the 16 row-sum columns only column d is ever read, and its value is at hand
@@ -460,7 +473,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           tc_fence_before();
         }
         l_resc = l_now * alpha;
-        put_pair(r_prev * alpha);
+        if (SMOOTH) put_pair(r_prev * alpha);
       }
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
@@ -469,10 +482,12 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
       tmem_wait_ld();
-      put_pair(l_now - l_resc);
-      mbar_arrive(&sh->fin_full[t]);
+      if (SMOOTH) {
+        put_pair(l_now - l_resc);
+        mbar_arrive(&sh->fin_full[t]);
+      }
     }
-    if (ok && warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43)) {
+    if (ok && (!SMOOTH || warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43))) {
       tc_fence_after();
       const int grow = qblk * 128 + row;
       const float inv_l = 1.0f / l_now;
@@ -505,36 +520,31 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
                  void* o, uint8_t* work, cudaStream_t s) {
   constexpr int KB = D / 64, NVC = HYB ? 1 : 2;
   constexpr size_t kVRow = HYB ? 128 : 64;
-  alignas(64) CUtensorMap tq, tk, tv, tmt;
+  alignas(64) CUtensorMap tq, tk, tv;
   if (!make_map(&tq, quant + ql.q_codes, D / 2, pr.n_pad, pr.BH, D / 2, 128) ||
       !make_map(&tk, quant + ql.k_codes, D / 2, pr.n_pad, pr.BH, D / 2, 128) ||
       !(HYB ? make_map_u4(&tv, quant + ql.v_codes, (uint64_t)pr.n_pad, D, pr.BH, D)
-            : make_map(&tv, quant + ql.v_codes, (uint64_t)pr.n_pad / 2, D, pr.BH, 64, D)) ||
-      !make_map(&tmt, work + wl.mu_mma, 32, D, (uint64_t)pr.BH * pr.nb, 32, D))
+            : make_map(&tv, quant + ql.v_codes, (uint64_t)pr.n_pad / 2, D, pr.BH, 64, D)))
     return cudaErrorUnknown;
-  const size_t n = (size_t)pr.BH * pr.nb * D;
-  means_tile_layout_kernel<D><<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const __nv_bfloat16*)(quant + ql.v_means),
-                                                                        (float*)(work + wl.mu_mma), n);
-  nvfp4_sf_tiles_kernel<D, HYB><<<dim3(pr.nb, pr.BH), 128, 0, s>>>(quant + ql.q_micro, quant + ql.k_micro, quant + ql.v_micro,
-                                                                  work + wl.sf_q, work + wl.sf_kv, pr.nb, pr.n_pad);
   Attn4Args a{};
   a.q_g = (const float*)(quant + ql.q_scale);
   a.k_g = (const float*)(quant + ql.k_scale);
-  a.sf_q = work + wl.sf_q;
-  a.sf_kv = work + wl.sf_kv;
+  a.q_micro = quant + ql.q_micro; a.k_micro = quant + ql.k_micro; a.v_micro = quant + ql.v_micro;
+  a.v_means = (const __nv_bfloat16*)(quant + ql.v_means);
   a.o = (__nv_bfloat16*)o;
   a.status = (uint32_t*)(work + wl.status);
   a.N = pr.N; a.n_pad = pr.n_pad; a.nb = pr.nb;
   a.sl = pr.softmax_scale * 1.4426950408889634f;
   a.code_off = 120.0f + pr.beta;
-  a.wait = {a.status, attn_wait_limit(), attn_wait_hint_ns()};
+  a.wait = {a.status, attn_wait_limit(), attn_wait_nonblocking()};
   constexpr size_t stage = 128 * (D / 2) + (D + 16) * kVRow + ((D * 32 + 1023) / 1024) * 1024 + (((KB + NVC) * 512 + 1023) / 1024) * 1024;
   constexpr size_t smem = 1024 + 2 * 128 * (D / 2) + 2 * 128 * kVRow + 2 * 128 * 32 + 2 * 1024 + 2 * 1024 + 1024 + kStages2 * stage + sizeof(FaSmem);
   static_assert(smem <= 227 * 1024, "shared memory of the 4-bit kernel exceeds the SM");
-  cudaError_t e = cudaFuncSetAttribute(attn4_fwd_2q_kernel<D, HYB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kernel = (pr.flags & VC_FLAG_V_SMOOTH) ? attn4_fwd_2q_kernel<D, HYB, true> : attn4_fwd_2q_kernel<D, HYB, false>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  attn4_fwd_2q_kernel<D, HYB><<<dim3((pr.nb + 1) / 2, pr.BH), 640, smem, s>>>(tq, tk, tv, tmt, a);
-  count_launches(3);
+  kernel<<<dim3((pr.nb + 1) / 2, pr.BH), 640, smem, s>>>(tq, tk, tv, a);
+  count_launches(1);
   return cudaGetLastError();
 }
 

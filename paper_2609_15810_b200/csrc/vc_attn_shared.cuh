@@ -16,10 +16,10 @@ using namespace sm100;
 
 constexpr uint32_t kErrTimeout = kStatusTimeout;
 
-// Where a wait that gives up says so, the polls after which it does, and how long one may sleep.
+// Where a wait that gives up says so, the polls after which it does, and (test hook) whether these may sleep.
 struct WaitArgs {
   uint32_t* status;
-  uint32_t limit, hint_ns;
+  uint32_t limit, nonblocking;
 };
 
 // Arguments of the 8-bit attention kernels.
@@ -42,9 +42,8 @@ inline uint32_t attn_wait_limit() {
   const uint32_t lim = wait_limit_override();
   return lim ? lim : kWaitLimit2;
 }
-// with the test override a poll never sleeps (hint 0 selects non-blocking tests of the barrier),
-// so that a tiny limit really is a short wait
-inline uint32_t attn_wait_hint_ns() { return wait_limit_override() ? 0u : 4000u; }
+// with the test override a poll never sleeps, so that a tiny limit really is a short wait
+inline uint32_t attn_wait_nonblocking() { return wait_limit_override() ? 1u : 0u; }
 
 struct FaSmem {
   uint64_t q_full, kv_full[kStages2], kv_empty[kStages2];
@@ -64,13 +63,12 @@ struct FaSmem {
 // kernel arguments, not loads.  (With the limits read from shared memory in front of the first test
 // and the vote behind the loop a completed wait took 170 cycles.  8-bit kernel at B1 H12 N32760 d128:
 // 3.52 -> 3.34 ms, at B2 H16 N16384 d64: 2.21 -> 1.94 ms; hybrid 3.40 -> 3.26, NVFP4 5.66 -> 5.28 ms.)
-// hint_ns = 0 (test hook): the polls never sleep.
 __device__ __forceinline__ bool warp_wait2(uint64_t* bar, uint32_t parity, FaSmem* sh, const WaitArgs& w, uint32_t code) {
   if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-  if (w.hint_ns) {
+  if (!w.nonblocking) {
 #pragma unroll 1
     for (uint32_t i = 0; i < w.limit; ++i) {
-      if (__all_sync(0xffffffffu, mbar_try_wait_hint(bar, parity, w.hint_ns))) return true;
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
       if ((i & 63u) == 63u && __any_sync(0xffffffffu, sh->abort)) return false;
     }
   } else {
@@ -104,17 +102,29 @@ __device__ __forceinline__ void drain_mmas(FaSmem* sh, int which) {
   mbar_wait(&sh->drain[which], 0, kDrainLimit);
 }
 
-// Block means as the B operand of the per-tile mean-restoration MMA: per (b, h, key tile) a
-// [d][8] fp32 tile with entry [c][0] = [c][1] = mu~[c] (for r_hi and r_lo) and zeros elsewhere.
+// Block means as the B operand of the per-tile mean-restoration MMA: a [d][8] fp32 tile with entry
+// [c][0] = [c][1] = mu~[c] (for r_hi and r_lo) and zeros elsewhere, in 32-byte rows whose two 16-byte
+// chunks swap when (row / 4) is odd.  The producer warp writes the two live words of every row into
+// the key tile's stage, next to the copies it issues; the zeros are written once per CTA.  (As a
+// tensor in global memory, expanded by a launch of its own and fetched by TMA, the same operand was
+// 32 bytes per mean: 42 MB written and 4 of the 37 KB a key tile moves into shared memory at B1 H40
+// N32760 d128.)
 template <int D>
-__global__ void means_tile_layout_kernel(const __nv_bfloat16* __restrict__ means, float* __restrict__ out, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // (bh * nb + tile) * D + c
-  if (i >= n) return;
-  const float v = __bfloat162float(means[i]);
-  float4* dst = reinterpret_cast<float4*>(out + i * 8);
-  dst[0] = make_float4(v, v, 0.f, 0.f);
-  dst[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
+struct MeanRows {
+  uint16_t v[D / 32];
+  // bf16 bits of the means of channels lane, lane + 32, ...
+  __device__ __forceinline__ void fetch(const __nv_bfloat16* means, int lane) {
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) v[i] = __ldg(reinterpret_cast<const unsigned short*>(means) + lane + 32 * i);
+  }
+  __device__ __forceinline__ void store(unsigned char* tile, int lane) const {
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) {
+      const int row = lane + 32 * i;
+      *reinterpret_cast<uint2*>(tile + row * 32 + 16 * ((row >> 2) & 1)) = make_uint2((uint32_t)v[i] << 16, (uint32_t)v[i] << 16);
+    }
+  }
+};
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,

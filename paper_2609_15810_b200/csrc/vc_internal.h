@@ -47,9 +47,7 @@ struct WorkLayout {
   size_t amax_bytes;
   size_t perm_bits;  // uint32 [BH][ceil(N / 32)]: bitmap of the permutation validator (VC_FLAG_CHECK_PERM)
   size_t perm_bits_bytes;
-  size_t mu_mma;     // fp32 [BH][nb][d][8]: block means as the B operand of the mean-restoration MMA
-  size_t sf_q;       // bytes [BH][nb][d/64][512]: Q^ NVFP4 factors in MMA chunk order (4 bits)
-  size_t sf_kv;      // bytes [BH][nb][d/64 + 2][512]: K^ and R^ factors per key tile (4 bits)
+  size_t prep_end;   // end of the sections the preprocessing pass uses
   size_t expand;     // bf16 [3][BH][N_pad][d]: NVFP4 operands expanded to bf16, serial 4-bit kernel only
   size_t total;
   int rope_off[3];   // entry offset of each axis table

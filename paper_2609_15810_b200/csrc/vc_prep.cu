@@ -1399,8 +1399,7 @@ extern "C" vc_status vc_prep_noalloc(const vc_params* p, const void* q, const vo
   if (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)quant | (uintptr_t)perm) & 15) return VC_ERR_INVALID_ARG;
   const vc::QuantLayout ql = vc::quant_layout(pr);
   const vc::WorkLayout wl = vc::work_layout(pr);
-  // the pass uses the workspace sections in front of the attention kernel's mean table
-  if (wl.mu_mma > (size_t)VC_NOALLOC_SCRATCH_BYTES) return VC_ERR_SCRATCH_LIMIT;
+  if (wl.prep_end > (size_t)VC_NOALLOC_SCRATCH_BYTES) return VC_ERR_SCRATCH_LIMIT;
   unsigned char* scratch = nullptr;
   if (scratch_address(&scratch) != cudaSuccess) return VC_ERR_CUDA;
   // launch_prep clears the words that must start at zero (status, amax) on the stream itself
