@@ -9,12 +9,14 @@ without a GPU driver (symbol checks) as well as on the B200 machine.
 import os
 import subprocess
 import sys
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libvc.so")
-SOURCES = ["vc_api.cu", "vc_prep.cu", "vc_perm_check.cu", "vc_attn_fwd.cu", "vc_attn_fwd4.cu", "vc_group.cu", "vc_mma_peak.cu", "vc_test_hooks.cu"]
+SOURCES = ["vc_api.cu", "vc_prep.cu", "vc_perm_check.cu", "vc_attn_fwd.cu", "vc_attn_fwd_2q_d128.cu", "vc_attn_fwd_2q_d64.cu",
+           "vc_attn_fwd4.cu", "vc_group.cu", "vc_mma_peak.cu", "vc_test_hooks.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -30,11 +32,10 @@ def _newer(target, deps):
 def build(force=False, verbose=False):
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(ROOT, "include", "vc_attn.h"))
-    objs = []
-    for src in SOURCES:
+
+    def compile_one(src):
         s = os.path.join(CSRC, src)
         o = os.path.join(CSRC, src.replace(".cu", ".o"))
-        objs.append(o)
         if force or not _newer(o, [s] + headers):
             cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", s, "-o", o]
             r = subprocess.run(cmd, capture_output=True, text=True)
@@ -42,6 +43,10 @@ def build(force=False, verbose=False):
                 sys.stderr.write(r.stdout + r.stderr)
             if r.returncode:
                 raise RuntimeError("nvcc failed for " + src)
+        return o
+
+    with ThreadPoolExecutor(max_workers=os.cpu_count() or 1) as pool:
+        objs = list(pool.map(compile_one, SOURCES))
     if force or not _newer(LIB, objs):
         cmd = [NVCC, "-shared", "-o", LIB] + objs + ["-cudart", "static"]
         r = subprocess.run(cmd, capture_output=True, text=True)

@@ -14,6 +14,16 @@ void count_launches(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order
 static std::atomic<uint32_t> g_wait_limit{0};
 uint32_t wait_limit_override() { return g_wait_limit.load(std::memory_order_relaxed); }
 
+int sm_count() {
+  static std::atomic<int> cache[64];             // per device: a process may drive GPUs of different sizes
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 148;
+  if (dev < 64 && (sms = cache[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+  if (dev < 64) cache[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 vc_status resolve(const vc_params* p, Problem* out) {

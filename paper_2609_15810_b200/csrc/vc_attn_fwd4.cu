@@ -79,6 +79,7 @@ struct Attn4Args {
   __nv_bfloat16* o;
   uint32_t* status;
   int N, n_pad, nb;
+  Tiles tiles;
   float sl;                        // softmax_scale * log2(e)
   float code_off;                  // 120 + beta  (Eq. 7; hybrid arrangement only)
   WaitArgs wait;
@@ -97,14 +98,13 @@ __device__ __forceinline__ float decode_ue4m3(uint32_t code) {
 //   warps 4-11    softmax warpgroups (tile 0, tile 1), one thread per query row
 //   warps 12-19   correction warpgroups, one thread per query row
 // Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16) | scale factors (56 columns).
-template <int D, bool HYB, bool SMOOTH>
-__global__ void __launch_bounds__(640, 1)
-attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                    const __grid_constant__ CUtensorMap tm_v, const Attn4Args a) {
+template <int D, bool HYB, bool SMOOTH, bool TWO>
+__device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                                              const Attn4Args& a, const int q0, const int bh) {
   constexpr int kTmemCols = 512;
   constexpr int KB = D / 64;                        // K = 64 steps of the score product
   constexpr int kRowB = D / 2;                      // bytes per Q^/K^ row
-  constexpr uint32_t O_COL = 128, O_STRIDE = 144, L_COL = D;
+  constexpr uint32_t O_COL = 128, O_STRIDE = 144, L_COL = D, S1_COL = O_COL + O_STRIDE;
   constexpr uint32_t SF_COL = 416;
   constexpr uint32_t SFQ_COL = SF_COL, SFK_COL = SF_COL + 16, SFP_COL = SF_COL + 24, SFV_COL = SF_COL + 40;
   constexpr int kRegCtl = 48, kRegSoftmax = 160, kRegCorr = 56;
@@ -129,21 +129,26 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   FaSmem* sh = reinterpret_cast<FaSmem*>(sStage + kStages2 * kStageBytes);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int qpair = blockIdx.x, bh = blockIdx.y;
   const int nb = a.nb;
+  // (one tile: double buffers, as in the 8-bit kernel)
+  // buffer (and barrier) of scores, codes and products of key tile j, and the parity of its phase
+  auto buf = [](int t, int j) { return TWO ? t : j & 1; };
+  auto par = [](int j) { return TWO ? j & 1 : (j >> 1) & 1; };
+  // alpha hand-off: tile t's two slots alternate; four slots when there is one tile
+  auto a_slot = [](int t, int j) { return TWO ? 2 * t + (j & 1) : j & 3; };
+  auto a_par = [](int j) { return TWO ? (j >> 1) & 1 : (j >> 2) & 1; };
 
+  const int early = min(kStages2, nb);      // key tiles whose copies are issued before anything else happens
   if (tid == 0) {
-    mbar_init(&sh->q_full, 1);
-    for (int i = 0; i < kStages2; ++i) { mbar_init(&sh->kv_full[i], 1); mbar_init(&sh->kv_empty[i], 2); }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&sh->s_full[i], 1); mbar_init(&sh->s_free[i], 128); mbar_init(&sh->o_done[i], 1);
-      mbar_init(&sh->fin_full[i], 128); mbar_init(&sh->o_final[i], 1);
-      for (int b = 0; b < 2; ++b) { mbar_init(&sh->a_full[i][b], 128); mbar_init(&sh->pc_full[i][b], 256); }
+    init_barriers(sh, TWO);
+    mbar_expect_tx_only(&sh->q_full, (TWO ? 2 : 1) * kQBytes);
+    tma_load_3d(sQ, &tm_q, &sh->q_full, 0, q0 * 128, bh);
+    if (TWO) tma_load_3d(sQ + kQBytes, &tm_q, &sh->q_full, 0, (q0 + 1) * 128, bh);   // past the end: zero fill
+    for (int j = 0; j < early; ++j) {
+      mbar_expect_tx_only(&sh->kv_full[j], kKBytes + kVTx);
+      tma_load_3d(sStage + j * kStageBytes, &tm_k, &sh->kv_full[j], 0, j * 128, bh);
+      tma_load_3d(sStage + j * kStageBytes + kKBytes, &tm_v, &sh->kv_full[j], HYB ? j * 128 : j * 64, 0, bh);   // elements resp. bytes
     }
-    mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
-    sh->abort = 0;
-    mbar_fence_init();
-    tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v);
   }
   for (int i = tid; i < 2 * (int)kAmBytes / 16; i += 640) reinterpret_cast<uint4*>(sAm)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < kStages2 * (int)kMuBytes / 16; i += 640)
@@ -152,8 +157,8 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // rows 0..15 of the second 128-row half, group bytes 0..3
   // (HYB: the same bytes, of which the product reads the low 8 of every 16; factor code 127 = 2^0,
   // and a chunk of that code for every row of P^)
-  for (int i = tid; i < kStages2 * (int)kOnesBytes / 4; i += 640)
-    reinterpret_cast<uint32_t*>(sStage + (i / (kOnesBytes / 4)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 4)] = 0x22222222u;
+  for (int i = tid; i < kStages2 * (int)kOnesBytes / 16; i += 640)
+    reinterpret_cast<uint4*>(sStage + (i / (kOnesBytes / 16)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 16)] = make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
   for (int i = tid; i < 128; i += 640)
     reinterpret_cast<uint32_t*>(sSfOnes)[i] = ((i & 3) == 0 && i < 64) ? (HYB ? 0x7f7f7f7fu : 0x38383838u) : 0u;
   if constexpr (HYB)
@@ -172,12 +177,9 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // ------------------------------------------------------------------ TMA producer
       // (the whole warp runs the loop: one elected lane issues the copies, all write factors and means)
       FactorRows<KB> fq;
-      if (elect_one()) mbar_expect_tx_only(&sh->q_full, 2 * kQBytes);
 #pragma unroll 1
-      for (int t = 0; t < 2; ++t) {
-        const int qb = 2 * qpair + t;                      // past the end: zero codes, any factors
-        if (elect_one()) tma_load_3d(sQ + t * kQBytes, &tm_q, &sh->q_full, 0, qb * 128, bh);
-        fq.fetch_tokens(a.q_micro + ((size_t)bh * a.n_pad + min(qb, nb - 1) * 128) * (D / 16), lane);
+      for (int t = 0; t < (TWO ? 2 : 1); ++t) {            // (past the end: zero codes, any factors)
+        fq.fetch_tokens(a.q_micro + ((size_t)bh * a.n_pad + min(q0 + t, nb - 1) * 128) * (D / 16), lane);
         fq.store(sSfq + t * 1024, lane);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // the stores -> tensor-core reads
@@ -196,7 +198,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         else fv.template fetch_channels<D>(a.v_micro + (size_t)bh * D * (a.n_pad / 16) + j * 8, a.n_pad / 16, 0x38383838u, lane);
         if (SMOOTH) mu.fetch(a.v_means + ((size_t)bh * nb + j) * D, lane);
         if (!warp_wait2(&sh->kv_empty[st], (it & 1) ^ 1, sh, a.wait, 11)) break;
-        if (elect_one()) {
+        if (j >= early && elect_one()) {
           mbar_expect_tx_only(&sh->kv_full[st], kKBytes + kVTx);
           tma_load_3d(base, &tm_k, &sh->kv_full[st], 0, j * 128, bh);
           tma_load_3d(base + kKBytes, &tm_v, &sh->kv_full[st], HYB ? j * 128 : j * 64, 0, bh);   // elements resp. bytes
@@ -216,7 +218,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const uint64_t dq0 = smem_desc_kmajor(smem_u32(sQ), kRowB), dq1 = smem_desc_kmajor(smem_u32(sQ + kQBytes), kRowB);
       bool ok = warp_wait2(&sh->q_full, 0, sh, a.wait, 20);
       if (ok && elect_one()) {
-        for (int t = 0; t < 2; ++t)
+        for (int t = 0; t < (TWO ? 2 : 1); ++t)
           for (int kb = 0; kb < KB; ++kb)
             tmem_cp_sf(tmem + SFQ_COL + (t * KB + kb) * 4, smem_desc_sf_chunk(smem_u32(sSfq + t * 1024 + kb * 512)));
       }
@@ -228,9 +230,9 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint64_t dk = smem_desc_kmajor(smem_u32(base), kRowB);
         const uint32_t sf_smem = smem_u32(base + kKBytes + kVBytes + kOnesBytes + kMuPad);
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          if (t == 0 ? j > 0 : true) {
-            if (!(ok = warp_wait2(&sh->s_free[1 - t], (t == 0 ? j - 1 : j) & 1, sh, a.wait, 22))) break;
+        for (int t = 0; t < (TWO ? 2 : 1); ++t) {
+          if (TWO ? (t == 0 ? j > 0 : true) : j > 1) {
+            if (!(ok = warp_wait2(&sh->s_free[TWO ? 1 - t : j & 1], TWO ? (t == 0 ? j - 1 : j) & 1 : par(j) ^ 1, sh, a.wait, 22))) break;
           }
           if (elect_one()) {
             tc_fence_after();
@@ -241,9 +243,9 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             const uint64_t dq = t == 0 ? dq0 : dq1;
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb)
-              mma_nvfp4_ss(tmem, dq + 2 * kb, dk + 2 * kb, idesc_qk, kb > 0, tmem + SFQ_COL + (t * KB + kb) * 4,
+              mma_nvfp4_ss(tmem + (TWO ? 0 : (j & 1) * S1_COL), dq + 2 * kb, dk + 2 * kb, idesc_qk, kb > 0, tmem + SFQ_COL + (t * KB + kb) * 4,
                            tmem + SFK_COL + kb * 4);
-            mma_commit(&sh->s_full[t]);
+            mma_commit(&sh->s_full[buf(t, j)]);
           }
           __syncwarp();
         }
@@ -272,31 +274,33 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint64_t dm = smem_desc_kmajor(smem_u32(sStage + stp * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
         const uint32_t sfv_smem = smem_u32(base + kKBytes + kVBytes + kOnesBytes + kMuPad + KB * 512);
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < (TWO ? 2 : 1); ++t) {
           if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 23))) break;
           if (elect_one()) {
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
+            const int b = buf(t, j);
+            const uint64_t dpt = b ? dp[1] : dp[0];
             if constexpr (HYB) {
               if (t == 0) tmem_cp_sf(tmem + SFV_COL, smem_desc_sf_chunk(sfv_smem));
 #pragma unroll
               for (int k = 0; k < 4; ++k)                  // 32 keys each; factor byte k of the value rows
-                mma_mxf8_ss(o_col, dp[t] + 2 * k, dv + 2 * k, idesc_mxf8_e4m3_e2m1(128, D + 16, k), (j > 0) | (k > 0),
+                mma_mxf8_ss(o_col, dpt + 2 * k, dv + 2 * k, idesc_mxf8_e4m3_e2m1(128, D + 16, k), (j > 0) | (k > 0),
                             tmem + SFP_COL, tmem + SFV_COL);
             } else {
               if (t == 0) {
                 tmem_cp_sf(tmem + SFV_COL, smem_desc_sf_chunk(sfv_smem));
                 tmem_cp_sf(tmem + SFV_COL + 8, smem_desc_sf_chunk(sfv_smem + 512));
               }
-              tmem_cp_sf(tmem + SFP_COL + t * 8, smem_desc_sf_chunk(smem_u32(sSfp + t * kSfpBytes)));
-              tmem_cp_sf(tmem + SFP_COL + t * 8 + 4, smem_desc_sf_chunk(smem_u32(sSfp + t * kSfpBytes + 512)));
+              tmem_cp_sf(tmem + SFP_COL + b * 8, smem_desc_sf_chunk(smem_u32(sSfp + b * kSfpBytes)));
+              tmem_cp_sf(tmem + SFP_COL + b * 8 + 4, smem_desc_sf_chunk(smem_u32(sSfp + b * kSfpBytes + 512)));
 #pragma unroll
               for (int kb = 0; kb < 2; ++kb)
-                mma_nvfp4_ss(o_col, dp[t] + 2 * kb, dv + 2 * kb, idesc_pv, (j > 0) | (kb > 0), tmem + SFP_COL + t * 8 + kb * 4,
+                mma_nvfp4_ss(o_col, dpt + 2 * kb, dv + 2 * kb, idesc_pv, (j > 0) | (kb > 0), tmem + SFP_COL + b * 8 + kb * 4,
                              tmem + SFV_COL + kb * 8);
             }
             if (j > 0 && SMOOTH) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
-            mma_commit(&sh->o_done[t]);
+            mma_commit(&sh->o_done[b]);
             if (j > 0) mma_commit(&sh->kv_empty[stp]);    // this tile is done with stage j-1
           }
           __syncwarp();
@@ -304,7 +308,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       const uint64_t dml = smem_desc_kmajor(smem_u32(sStage + ((nb - 1) % kStages2) * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {                       // mean term of the last tile
+      for (int t = 0; t < (TWO ? 2 : 1); ++t) {           // mean term of the last tile
         if (!SMOOTH || !ok || !(ok = warp_wait2(&sh->fin_full[t], 0, sh, a.wait, 27))) break;
         if (elect_one()) {
           tc_fence_after();
@@ -315,27 +319,27 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       drain_mmas(sh, 1);
     }
-  } else if (warp < 12) {
+  } else if (warp < (TWO ? 12 : 8)) {
     // -------------------------------------------------------------------- softmax warpgroups
     reg_inc<kRegSoftmax>();
-    const int t = (warp - 4) >> 2;                         // query tile of this warpgroup
+    const int t = TWO ? (warp - 4) >> 2 : 0;               // query tile of this warpgroup
     const int row = (warp & 3) * 32 + lane;
     // my row of the swizzled code tile: 64-byte rows, chunk c sits at chunk position c ^ ((row / 2) % 4)
     // (HYB: 128-byte rows, chunk c at position c ^ (row % 8))
     const uint32_t p_row = smem_u32(sP + t * kPBytes + row * kVRow) + ((HYB ? row & 7 : (row >> 1) & 3) << 4);
     const uint32_t sfp_row = smem_u32(sSfp + t * kSfpBytes + (row & 31) * 16 + (row >> 5) * 4);
     const float cs = (a.q_g[bh] * a.k_g[bh]) * a.sl;       // code units -> log2 domain
-    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
+    const uint32_t alpha_at = smem_u32(&sh->alpha[0][row]);
     float m_run = -INFINITY;
     for (int j = 0; j < nb; ++j) {
-      const int ph = j & 1;
-      if (!warp_wait2(&sh->s_full[t], ph, sh, a.wait, 30)) break;
+      if (!warp_wait2(&sh->s_full[buf(t, j)], par(j), sh, a.wait, 30)) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
-      tmem_ld32(lane_base, s0); tmem_ld32(lane_base + 32, s1); tmem_ld32(lane_base + 64, s2); tmem_ld32(lane_base + 96, s3);
+      const uint32_t s_col = lane_base + (TWO ? 0 : (j & 1) * S1_COL);
+      tmem_ld32(s_col, s0); tmem_ld32(s_col + 32, s1); tmem_ld32(s_col + 64, s2); tmem_ld32(s_col + 96, s3);
       tmem_wait_ld();
       tc_fence_before();
-      mbar_arrive(&sh->s_free[t]);                        // the score buffer may be overwritten
+      mbar_arrive(&sh->s_free[buf(t, j)]);                 // the score buffer may be overwritten
       const int nv = a.N - j * 128;                       // >= 128 except on the ragged last tile
       if (nv < 128) {                                     // padded keys: probability zero
 #pragma unroll
@@ -367,20 +371,20 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       const float mxa = max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
       const float m_new = fmaxf(m_run, mxa * cs);         // m' = max(m, rowmax S_ij)
-      sts32(alpha_at, ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
-      mbar_arrive(&sh->a_full[t][j & 1]);
+      sts32(alpha_at + 512 * a_slot(t, j), ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
+      mbar_arrive(&sh->a_full[a_slot(t, j)]);
       m_run = m_new;
       if constexpr (HYB) {
         // ExpCast-FP8 (Eq. 7): t = (8 u + 120 + beta) / 128, code = round-to-nearest-even(128 t)
         // clipped at 0 (two packed FP32 instructions and a saturating pack per two scores)
-        if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31)) break;
+        if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
         const float fa = cs * 0.0625f, fb = (a.code_off - 8.0f * m_new) * 0.0078125f;
         const uint64_t fa2 = pack_f32x2(fa, fa), fb2 = pack_f32x2(fb, fb);
         auto code4 = [&](const uint32_t (&sv)[32], int w) -> uint32_t {
           return expcast_codes4(sv[4 * w], sv[4 * w + 1], sv[4 * w + 2], sv[4 * w + 3], fa2, fb2);
         };
         auto store16 = [&](const uint32_t (&sv)[32], int half, int chunk) {   // keys 16 chunk .. +15
-          sts128(p_row ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
+          sts128((p_row + (TWO ? 0 : (j & 1) * kPBytes)) ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
         };
         store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
         store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
@@ -403,7 +407,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         off[g] = sb ? c0 - lg2_approx(decode_ue4m3(sb)) : -INFINITY;
       }
       // the previous code tile must have been consumed before it is overwritten
-      if (j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31)) break;
+      if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
 
       const uint64_t cs2 = pack_f32x2(cs, cs);
       auto quant16 = [&](const uint32_t (&sv)[32], int half, int g) -> uint2 {   // keys 16 g .. 16 g + 15
@@ -421,23 +425,23 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       };
       auto store32 = [&](const uint32_t (&sv)[32], int chunk) {   // keys 32 chunk .. +31 -> 16 bytes
         const uint2 lo = quant16(sv, 0, 2 * chunk), hi = quant16(sv, 1, 2 * chunk + 1);
-        sts128(p_row ^ (chunk << 4), lo.x, lo.y, hi.x, hi.y);
+        sts128((p_row + (TWO ? 0 : (j & 1) * kPBytes)) ^ (chunk << 4), lo.x, lo.y, hi.x, hi.y);
       };
       store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
-      sts32(sfp_row, __uint_as_float(sfw[0]));
-      sts32(sfp_row + 512, __uint_as_float(sfw[1]));                               // the chunk of keys 64..127
+      sts32(sfp_row + (TWO ? 0 : (j & 1) * kSfpBytes), __uint_as_float(sfw[0]));
+      sts32(sfp_row + (TWO ? 0 : (j & 1) * kSfpBytes) + 512, __uint_as_float(sfw[1]));                               // the chunk of keys 64..127
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
-  } else {
+  } else if (TWO ? warp >= 12 : warp >= 12 && warp < 16) {
     // -------------------------------------------------------------------- correction warpgroups
     reg_dec<kRegCorr>();
-    const int t = (warp - 12) >> 2;
+    const int t = TWO ? (warp - 12) >> 2 : 0;
     const int row = (warp & 3) * 32 + lane;
-    const int qblk = 2 * qpair + t;
+    const int qblk = q0 + t;
     const uint32_t o_base = lane_base + O_COL + O_STRIDE * t;
     const uint32_t am_row = smem_u32(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
-    const uint32_t alpha_at = smem_u32(&sh->alpha[t][row]);
+    const uint32_t alpha_at = smem_u32(&sh->alpha[0][row]);
     float l_resc = 0.f;       // l as it stands in column d after the latest rescale, before the tile's own sum
     float l_now = 0.f;
     bool ok = true;
@@ -447,12 +451,12 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
-      if (!(ok = warp_wait2(&sh->a_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 40))) break;
-      const float alpha = lds32(alpha_at);
+      if (!(ok = warp_wait2(&sh->a_full[a_slot(t, j)], a_par(j), sh, a.wait, 40))) break;
+      const float alpha = lds32(alpha_at + 512 * a_slot(t, j));
       const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);   // a row maximum of the warp moved
       // (without block means nothing needs l tile by tile: a warp whose maxima stand still passes on)
       if (j > 0 && (SMOOTH || moved)) {
-        if (!(ok = warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 41))) break;
+        if (!(ok = warp_wait2(&sh->o_done[buf(t, j - 1)], par(j - 1), sh, a.wait, 41))) break;
         tc_fence_after();
         l_now = __uint_as_float(tmem_ld1(o_base + L_COL));   // l after tile j-1
         tmem_wait_ld();
@@ -478,7 +482,7 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
     // ---- last tile's mean term, then the epilogue: O = A / l (means are unscaled at 4 bits, App. B)
-    if (ok && (ok = warp_wait2(&sh->o_done[t], (nb - 1) & 1, sh, a.wait, 42))) {
+    if (ok && (ok = warp_wait2(&sh->o_done[buf(t, nb - 1)], par(nb - 1), sh, a.wait, 42))) {
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
       tmem_wait_ld();
@@ -515,6 +519,17 @@ attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   if (warp == 2) tmem_dealloc<kTmemCols>(tmem);
 }
 
+// CTAs with a pair of query tiles, and behind them CTAs with one (see split_tiles).
+template <int D, bool HYB, bool SMOOTH>
+__global__ void __launch_bounds__(640, 1)
+attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                    const __grid_constant__ CUtensorMap tm_v, const Attn4Args a) {
+  const TileOf w = tile_of(a.tiles, a.nb);
+  if (w.q0 >= a.nb) return;                 // the missing second tile of a head's last pair
+  if (w.two) attn4_2q_body<D, HYB, SMOOTH, true>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
+  else attn4_2q_body<D, HYB, SMOOTH, false>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
+}
+
 template <int D, bool HYB>
 cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl, const uint8_t* quant,
                  void* o, uint8_t* work, cudaStream_t s) {
@@ -543,7 +558,9 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   auto kernel = (pr.flags & VC_FLAG_V_SMOOTH) ? attn4_fwd_2q_kernel<D, HYB, true> : attn4_fwd_2q_kernel<D, HYB, false>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kernel<<<dim3((pr.nb + 1) / 2, pr.BH), 640, smem, s>>>(tq, tk, tv, a);
+  unsigned grid;
+  a.tiles = split_tiles(pr, true, &grid);
+  kernel<<<grid, 640, smem, s>>>(tq, tk, tv, a);
   count_launches(1);
   return cudaGetLastError();
 }

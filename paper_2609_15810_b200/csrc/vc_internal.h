@@ -54,6 +54,9 @@ struct WorkLayout {
   int rope_entries;
 };
 
+// SM count of the current device (asked for once per device).
+int sm_count();
+
 vc_status resolve(const vc_params* p, Problem* out);
 QuantLayout quant_layout(const Problem& pr);
 WorkLayout work_layout(const Problem& pr);
@@ -67,6 +70,11 @@ cudaError_t launch_prep(const Problem& pr, const QuantLayout& ql, const WorkLayo
 cudaError_t launch_attn_fwd(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
                             const uint8_t* quant, void* o, uint8_t* work, cudaStream_t stream, bool clear_status);
 
+// the two-query-tile kernels of the 8-bit path, one translation unit per head dimension
+cudaError_t launch_2q_d128(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl, const uint8_t* quant, void* o,
+                           uint8_t* work, cudaStream_t s);
+cudaError_t launch_2q_d64(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl, const uint8_t* quant, void* o,
+                          uint8_t* work, cudaStream_t s);
 cudaError_t launch_attn_fwd4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
                              const uint8_t* quant, void* o, uint8_t* work, cudaStream_t stream);
 

@@ -1212,16 +1212,7 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
 }
 
 int persistent_grid(int n_items, int per_sm = 2) {
-  // SM count of the CURRENT device (cached per device: a process may drive GPUs of different sizes)
-  static int cache[64] = {};
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-  if (dev >= 0 && dev < 64 && cache[dev] > 0) sms = cache[dev];
-  else {
-    if (dev < 0 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-    if (dev >= 0 && dev < 64) cache[dev] = sms;
-  }
-  const int g = per_sm * sms;
+  const int g = per_sm * sm_count();
   return n_items < g ? n_items : g;
 }
 

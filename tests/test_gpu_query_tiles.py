@@ -1,0 +1,40 @@
+"""CTAs with one query tile against CTAs with two: the same arithmetic in the same order, so a head's
+output does not depend on how many heads share the launch (which decides who gets a pair), bit for bit."""
+import pytest
+import torch
+
+import paper_2609_15810_b200 as vc
+from paper_2609_15810_b200.binding import Params, alloc_buffers
+
+pytestmark = pytest.mark.gpu
+
+FORMATS = {"fp8": (8, vc.VC_P_DEFAULT, 0), "int8qk": (8, vc.VC_P_DEFAULT, vc.VC_FLAG_INT8_QK),
+           "nvfp4": (4, vc.VC_P_DEFAULT, 0), "hybrid": (4, vc.VC_P_EXPCAST_E4M3, 0)}
+
+
+def _attn(q, k, v, grid, fmt, smooth):
+    bits, pf, flags = FORMATS[fmt]
+    flags |= vc.VC_FLAG_ALL if smooth else vc.VC_FLAG_ALL & ~vc.VC_FLAG_V_SMOOTH
+    B, H, N, d = q.shape
+    p = Params.make(B, H, N, d, grid, bits=bits, p_format=pf, flags=flags)
+    quant, work = alloc_buffers(p)
+    o = torch.empty_like(q)
+    vc.vc_attn(p, q, k, v, None, o, quant, work)
+    vc.vc_poll_status(work)
+    return o
+
+
+@pytest.mark.parametrize("smooth", [True, False])
+@pytest.mark.parametrize("fmt", list(FORMATS))
+@pytest.mark.parametrize("N,grid,d,H", [(300, (3, 10, 10), 128, 160),    # 3 tiles: every second pair is half empty
+                                        (512, (2, 16, 16), 64, 84),      # 168 pairs: whole waves and 20 pairs behind
+                                        (129, (1, 3, 43), 128, 75),      # 2 tiles, the last wave more than half full
+                                        (1153, (1, 1, 1153), 64, 20)])   # 10 tiles: every buffer several times
+def test_output_does_not_depend_on_the_split(N, grid, d, H, fmt, smooth):
+    g = torch.Generator(device="cuda").manual_seed(N + H)
+    q, k, v = [torch.randn(1, H, N, d, generator=g, device="cuda").bfloat16() for _ in range(3)]
+    k += 2 * torch.randn(1, H, 1, d, generator=g, device="cuda").bfloat16()
+    many = _attn(q, k, v, grid, fmt, smooth)
+    for h in (0, H // 2, H - 2, H - 1):
+        alone = _attn(*[t[:, h:h + 1].contiguous() for t in (q, k, v)], grid, fmt, smooth)
+        assert torch.equal(many[:, h:h + 1], alone), h
