@@ -336,20 +336,18 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
       const uint32_t s_col = lane_base + (TWO ? 0 : (j & 1) * S1_COL);
+      if (j == nb - 1 && (a.N & 127)) {                   // ragged last tile: padded keys score -inf
+#pragma unroll 1
+        for (int c = a.N & 127; c < 128; ++c) tmem_st1(s_col + c, 0xff800000u);
+        tmem_wait_st();
+      }
       tmem_ld32(s_col, s0); tmem_ld32(s_col + 32, s1); tmem_ld32(s_col + 64, s2); tmem_ld32(s_col + 96, s3);
       tmem_wait_ld();
       tc_fence_before();
       mbar_arrive(&sh->s_free[buf(t, j)]);                 // the score buffer may be overwritten
-      const int nv = a.N - j * 128;                       // >= 128 except on the ragged last tile
-      if (nv < 128) {                                     // padded keys: probability zero
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i >= nv) s0[i] = 0xff800000u;
-          if (32 + i >= nv) s1[i] = 0xff800000u;
-          if (64 + i >= nv) s2[i] = 0xff800000u;
-          if (96 + i >= nv) s3[i] = 0xff800000u;
-        }
-      }
+      // (never taken: the end of a basic block here keeps the compiler from moving the maxima in front of
+      // the release of the score buffer, which costs 4 to 14 percent of the kernel)
+      if (a.n_pad < 0) break;
       float mx[8];                                        // maxima of the eight 16-key groups
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
