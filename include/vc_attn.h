@@ -265,8 +265,7 @@ int32_t vc_group_schedule(int32_t step, int32_t n_steps, int32_t reuse);
  *     without ordering between their streams) race on the array: serialize them.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current; make that first call outside any
- *     stream capture.  Later calls only set the kernels' shared-memory attribute (a host-side
- *     call that allocates nothing), launch kernels and issue two small memsets on `stream`.
+ *     stream capture.  Later calls only launch kernels on `stream`.
  * It calls no cudaMalloc / cudaFree and no allocating library routine.  The output is
  * the same bundle vc_prep writes. */
 #define VC_NOALLOC_SCRATCH_BYTES (4u << 20)

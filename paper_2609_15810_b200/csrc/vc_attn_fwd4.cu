@@ -28,6 +28,7 @@
 
 #include "vc_attn_shared.cuh"
 #include "vc_internal.h"
+#include "vc_launch.h"
 #include "vc_sm100.cuh"
 
 namespace vc {
@@ -141,6 +142,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   const int early = min(kStages2, nb);      // key tiles whose copies are issued before anything else happens
   if (tid == 0) {
     init_barriers(sh, TWO);
+    pdl_wait();                             // the bundle is complete from here on
     mbar_expect_tx_only(&sh->q_full, (TWO ? 2 : 1) * kQBytes);
     tma_load_3d(sQ, &tm_q, &sh->q_full, 0, q0 * 128, bh);
     if (TWO) tma_load_3d(sQ + kQBytes, &tm_q, &sh->q_full, 0, (q0 + 1) * 128, bh);   // past the end: zero fill
@@ -163,6 +165,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
     reinterpret_cast<uint32_t*>(sSfOnes)[i] = ((i & 3) == 0 && i < 64) ? (HYB ? 0x7f7f7f7fu : 0x38383838u) : 0u;
   if constexpr (HYB)
     for (int i = tid; i < 128; i += 640) reinterpret_cast<uint32_t*>(sSfp)[i] = 0x7f7f7f7fu;
+  pdl_wait();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor-core reads
   if (warp == 2) { tmem_alloc<kTmemCols>(&sh->tmem_base); tmem_relinquish(); }
   tc_fence_before();
@@ -522,6 +525,7 @@ template <int D, bool HYB, bool SMOOTH>
 __global__ void __launch_bounds__(640, 1)
 attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const Attn4Args a) {
+  pdl_allow();
   const TileOf w = tile_of(a.tiles, a.nb);
   if (w.q0 >= a.nb) return;                 // the missing second tile of a head's last pair
   if (w.two) attn4_2q_body<D, HYB, SMOOTH, true>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
@@ -553,12 +557,17 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   constexpr size_t stage = 128 * (D / 2) + (D + 16) * kVRow + ((D * 32 + 1023) / 1024) * 1024 + (((KB + NVC) * 512 + 1023) / 1024) * 1024;
   constexpr size_t smem = 1024 + 2 * 128 * (D / 2) + 2 * 128 * kVRow + 2 * 128 * 32 + 2 * 1024 + 2 * 1024 + 1024 + kStages2 * stage + sizeof(FaSmem);
   static_assert(smem <= 227 * 1024, "shared memory of the 4-bit kernel exceeds the SM");
-  auto kernel = (pr.flags & VC_FLAG_V_SMOOTH) ? attn4_fwd_2q_kernel<D, HYB, true> : attn4_fwd_2q_kernel<D, HYB, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   unsigned grid;
   a.tiles = split_tiles(pr, true, &grid);
-  kernel<<<grid, 640, smem, s>>>(tq, tk, tv, a);
+  cudaError_t e;
+  if (pr.flags & VC_FLAG_V_SMOOTH) {
+    if ((e = allow_smem<attn4_fwd_2q_kernel<D, HYB, true>>()) == cudaSuccess)
+      e = launch_overlapped(attn4_fwd_2q_kernel<D, HYB, true>, dim3(grid), 640, smem, s, tq, tk, tv, a);
+  } else {
+    if ((e = allow_smem<attn4_fwd_2q_kernel<D, HYB, false>>()) == cudaSuccess)
+      e = launch_overlapped(attn4_fwd_2q_kernel<D, HYB, false>, dim3(grid), 640, smem, s, tq, tk, tv, a);
+  }
+  if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();
 }

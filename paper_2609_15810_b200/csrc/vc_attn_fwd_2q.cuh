@@ -6,6 +6,7 @@
 
 #include "vc_attn_shared.cuh"
 #include "vc_internal.h"
+#include "vc_launch.h"
 #include "vc_sm100.cuh"
 
 namespace vc {
@@ -102,6 +103,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   const int early = min(kStages2, nb);      // key tiles whose copies are issued before anything else happens
   if (tid == 0) {
     init_barriers(sh, TWO);
+    pdl_wait();                             // the bundle is complete from here on
     mbar_expect_tx(&sh->q_full, (TWO ? 2 : 1) * kQBytes);
     tma_load_3d(sQ, &tm_q, &sh->q_full, 0, q0 * 128, bh);
     if (TWO) tma_load_3d(sQ + kQBytes, &tm_q, &sh->q_full, 0, (q0 + 1) * 128, bh);   // past the end: zero fill
@@ -117,6 +119,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   // 16 rows of E4M3 1.0 behind every value tile (the rows are uniform, so the swizzle is moot)
   for (int i = tid; i < kStages2 * (int)kOnesBytes / 16; i += 640)
     reinterpret_cast<uint4*>(sStage + (i / (kOnesBytes / 16)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 16)] = make_uint4(0x38383838u, 0x38383838u, 0x38383838u, 0x38383838u);
+  pdl_wait();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor-core reads
   if (warp == 2) { tmem_alloc<kTmemCols>(&sh->tmem_base); tmem_relinquish(); }
   tc_fence_before();
@@ -430,6 +433,7 @@ template <int D, int PF, bool INT8, bool SMOOTH, bool ONE>
 __global__ void __launch_bounds__(640, 1)
 attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const AttnArgs a) {
+  pdl_allow();
   const TileOf w = tile_of(a.tiles, a.nb);
   if (w.q0 >= a.nb) return;                 // the missing second tile of a head's last pair
   if constexpr (ONE) {
@@ -457,19 +461,20 @@ cudaError_t run_2q(const Problem& pr, const QuantLayout& ql, const WorkLayout& w
   if (int8 && pf > kPfExp) return cudaErrorNotSupported;
   unsigned grid;
   a.tiles = split_tiles(pr, pf == kPfExpCast, &grid);
+#define VC_LAUNCH_2Q(...)                                                                                      \
+  ((e = allow_smem<attn_fwd_2q_kernel<D, __VA_ARGS__>>()) == cudaSuccess                                       \
+       ? (e = launch_overlapped(attn_fwd_2q_kernel<D, __VA_ARGS__>, dim3(grid), 640, smem, s, tq, tk, tv, a)) \
+       : e)
   cudaError_t e = cudaSuccess;
-  auto launch = [&](auto kernel) {
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) == cudaSuccess)
-      kernel<<<grid, 640, smem, s>>>(tq, tk, tv, a);
-  };
   if (pf == kPfExpCast) {
-    if (smooth) int8 ? launch(attn_fwd_2q_kernel<D, kPfExpCast, true, true, true>) : launch(attn_fwd_2q_kernel<D, kPfExpCast, false, true, true>);
-    else int8 ? launch(attn_fwd_2q_kernel<D, kPfExpCast, true, false, true>) : launch(attn_fwd_2q_kernel<D, kPfExpCast, false, false, true>);
+    if (smooth) int8 ? VC_LAUNCH_2Q(kPfExpCast, true, true, true) : VC_LAUNCH_2Q(kPfExpCast, false, true, true);
+    else int8 ? VC_LAUNCH_2Q(kPfExpCast, true, false, true) : VC_LAUNCH_2Q(kPfExpCast, false, false, true);
   }
   // (the other formats exist for comparison: always pairs, and means of zero are added)
-  else if (pf == kPfExp) int8 ? launch(attn_fwd_2q_kernel<D, kPfExp, true, true, false>) : launch(attn_fwd_2q_kernel<D, kPfExp, false, true, false>);
-  else if (pf == kPfExpPoly) launch(attn_fwd_2q_kernel<D, kPfExpPoly, false, true, false>);
-  else launch(attn_fwd_2q_kernel<D, kPfExpMix, false, true, false>);
+  else if (pf == kPfExp) int8 ? VC_LAUNCH_2Q(kPfExp, true, true, false) : VC_LAUNCH_2Q(kPfExp, false, true, false);
+  else if (pf == kPfExpPoly) VC_LAUNCH_2Q(kPfExpPoly, false, true, false);
+  else VC_LAUNCH_2Q(kPfExpMix, false, true, false);
+#undef VC_LAUNCH_2Q
   if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();

@@ -13,6 +13,7 @@
 // can be processed in groups so that the second read of K and V may hit L2.  All passes are
 // persistent kernels that prefetch the next row blocks with cp.async while they transform
 // the current one.
+#include "vc_launch.h"
 #include "vc_prep_common.cuh"
 
 namespace vc {
@@ -21,8 +22,27 @@ namespace {
 // ---------------------------------------------------------------------------------------
 // RoPE tables: per axis a, entry [pos][i] = (cos, sin)(pos * theta^(-2 i / d_a)), evaluated
 // in double and rounded once to fp32.
-__global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
+// The same launch clears the words that must start at zero (the status word, the maxima) and, when
+// the caller supplies the statistics, turns them into the K mean and the value scales of the bundle.
+struct SetUp {
+  unsigned int *status, *zero;
+  int n_zero;                       // words behind `zero`
+  int n_ext;                        // B H d with supplied statistics, else 0
+  const float *ext_k_mean, *ext_v_amax;   // ext_k_mean: null = a mean of zero (K smoothing off)
+  float *k_mean, *v_scale;
+};
+__device__ __forceinline__ float value_scale(float amax) { return amax > 0.f ? amax / 448.0f : 1.0f; }
+
+__global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta, const SetUp u) {
+  pdl_wait();
+  pdl_allow();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+  if (e == 0) *u.status = 0u;
+  for (int i = e; i < u.n_zero; i += all) u.zero[i] = 0u;
+  for (int i = e; i < u.n_ext; i += all) {
+    u.k_mean[i] = u.ext_k_mean ? u.ext_k_mean[i] : 0.f;
+    u.v_scale[i] = value_scale(u.ext_v_amax[i]);
+  }
   if (e >= rd.entries) return;
   int a = e >= rd.off[2] ? 2 : (e >= rd.off[1] ? 1 : 0);
   int r = e - rd.off[a];
@@ -30,7 +50,8 @@ __global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta) {
   int i = r - pos * rd.pairs[a];
   double freq = pow(theta, -2.0 * (double)i / (double)(2 * rd.pairs[a]));
   double phi = (double)pos * freq;
-  const double c = cos(phi), sn = sin(phi);
+  double c, sn;
+  sincos(phi, &sn, &c);
   tab[e] = make_float2((float)c, (float)sn);
   // second table: the rotation folded into the first Hadamard level, u = x0 (c + s) + x1 (c - s),
   // v = x0 (c - s) - x1 (c + s), each coefficient rounded once
@@ -50,26 +71,21 @@ __global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta) {
 // block kept the copy engine, not HBM, busy.)
 constexpr int kThreads = 256;      // threads of the column-sum and V passes
 constexpr int kRowThreads = 128;   // rows of a Q/K item (threads of the pass = rows x threads per row)
-#ifndef VC_PREP_TPR
-#define VC_PREP_TPR 2
-#endif
-#ifndef VC_PREP_TPR_FAST
-#define VC_PREP_TPR_FAST VC_PREP_TPR      // threads per row of the packed row transform
-#endif
+constexpr int kTpr = 2;            // threads per Q/K row
 
 template <int D> struct Geo {
   static constexpr int pitch = 2 * D + 16;          // row pitch of the thread-per-row layout
   static constexpr int stage_bytes = kBlock * pitch;
 };
 
-// Items are numbered block-fastest, then head, then tensor.  A CTA visits items blockIdx.x + k *
-// gridDim.x: the position is divided out once and then advanced by the grid stride with carries
+// Items are numbered block-fastest, then head, then tensor.  The CTA with number `rank` of a pass visits
+// items rank + k * stride: the position is divided out once and then advanced by the grid stride with carries
 // (the divisions are not free at 64 elements per thread and item).
 struct Cursor {
   int blk, hh, z;            // block, head within the launch's group, tensor
 };
 struct CursorStep {
-  int dblk, dhh;             // gridDim.x = dhh * nb + dblk
+  int dblk, dhh;             // stride = dhh * nb + dblk
 };
 __device__ __forceinline__ Cursor cursor_at(int item, int nb, int nh) {
   Cursor c;
@@ -79,10 +95,10 @@ __device__ __forceinline__ Cursor cursor_at(int item, int nb, int nh) {
   c.z = r / nh;
   return c;
 }
-__device__ __forceinline__ CursorStep cursor_step(int nb) {
+__device__ __forceinline__ CursorStep cursor_step(int stride, int nb) {
   CursorStep s;
-  s.dhh = (int)gridDim.x / nb;
-  s.dblk = (int)gridDim.x - s.dhh * nb;
+  s.dhh = stride / nb;
+  s.dblk = stride - s.dhh * nb;
   return s;
 }
 __device__ __forceinline__ void advance(Cursor& c, const CursorStep& s, int nb, int nh) {
@@ -952,20 +968,23 @@ __device__ __forceinline__ RopeTab stage_rope_table(const PrepArgs& a, unsigned 
   return tab;
 }
 
-// Launch 1a: column sums of RoPE(K) per block (the channel mean is taken after the rotation).
+// Where a CTA stands in a pass: CTA `rank` of `stride`, n items.
+struct Slot {
+  int rank, stride, n_items;
+};
+
+// Column sums of RoPE(K) per block (the channel mean is taken after the rotation).
 // Shared memory: [2 stages x 32 KB][red: 8 D floats][RoPE table].
 template <int D>
-__global__ void __launch_bounds__(kThreads, 2) prep_kcolsum_kernel(const PrepArgs a, int n_items, int nh) {
+__device__ __forceinline__ void kcolsum_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh) {
   constexpr int LPR = D / 8, RPL = LPR / 2, kStage = kThreads * RPL * 16;
-  extern __shared__ __align__(128) unsigned char smem[];
   float* red = reinterpret_cast<float*>(smem + 2 * kStage);
-  const RopeTab tab = stage_rope_table(a, smem + 2 * kStage + 8 * D * 4);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lr = lane % LPR, hb = lane / LPR;
   const PairSlots ps = pair_slots(a.rd, 4 * lr);
-  const CursorStep step = cursor_step(a.nb);
+  const CursorStep step = cursor_step(sl.stride, a.nb);
   auto issue = [&](int item, const Cursor& c, int st) {
-    if (item < n_items) {
+    if (item < sl.n_items) {
       const char* base = reinterpret_cast<const char*>(a.k) + head_offset_bytes(a, a.bh0 + c.hh) + 16 * lr;
       const int t0 = c.blk * kBlock + 16 * warp + RPL * hb;
       unsigned char* dst = smem + st * kStage + tid * 16;
@@ -975,12 +994,14 @@ __global__ void __launch_bounds__(kThreads, 2) prep_kcolsum_kernel(const PrepArg
     }
     cp_async_commit();
   };
-  Cursor cur = cursor_at(blockIdx.x, a.nb, nh), nxt = cur;
+  Cursor cur = cursor_at(sl.rank, a.nb, nh), nxt = cur;
   advance(nxt, step, a.nb, nh);
-  issue(blockIdx.x, cur, 0);
+  issue(sl.rank, cur, 0);
+  pdl_wait();
+  const RopeTab tab = stage_rope_table(a, smem + 2 * kStage + 8 * D * 4);
   int i = 0;
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++i) {
-    issue(item + gridDim.x, nxt, (i + 1) & 1);
+  for (int item = sl.rank; item < sl.n_items; item += sl.stride, ++i) {
+    issue(item + sl.stride, nxt, (i + 1) & 1);
     cp_async_wait<1>();                       // this thread's chunks of item i have landed
     k_colsum_item<D>(a, smem + (i & 1) * kStage, red, tab, ps, a.bh0 + cur.hh, cur.blk);
     cur = nxt;
@@ -988,25 +1009,24 @@ __global__ void __launch_bounds__(kThreads, 2) prep_kcolsum_kernel(const PrepArg
   }
 }
 
-// V pass: STAGE = block means + residual amax (launch 1b) or quantization of the residual.
+// V pass: STAGE = block means + residual amax, or quantization of the residual.
 // Shared memory: [3 stages x (128 x 2 D)][red: 16 D floats][source rows: 2 x 128].
 template <int D, int STAGE>
-__global__ void __launch_bounds__(kThreads, 2) prep_v_kernel(const PrepArgs a, int n_items, int nh) {
+__device__ __forceinline__ void v_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh) {
   constexpr int LPR = D / 8, kStage = kBlock * 2 * D, NL = kBlock * LPR / kThreads;
-  extern __shared__ __align__(128) unsigned char smem[];
   float* red = reinterpret_cast<float*>(smem + 3 * kStage);
   int* src_ring = reinterpret_cast<int*>(red + 16 * D);                // [2][128]
   const int tid = threadIdx.x;
-  const CursorStep step = cursor_step(a.nb);
+  const CursorStep step = cursor_step(sl.stride, a.nb);
   // source row of row `tid` of an item (the gather by pi), -1 if there is none
   auto fetch = [&](int item, const Cursor& c) -> int {
-    if (item >= n_items || tid >= kBlock) return -1;
+    if (item >= sl.n_items || tid >= kBlock) return -1;
     const int t = c.blk * kBlock + tid;
     if (t >= a.N) return -1;
     return a.perm ? min(max(__ldg(a.perm + (size_t)(a.bh0 + c.hh) * a.N + t), 0), a.N - 1) : t;   // clamped: never a bad address
   };
   auto issue = [&](int item, const Cursor& c, int st, const int* src) {
-    if (item < n_items) {
+    if (item < sl.n_items) {
       const char* base = reinterpret_cast<const char*>(a.v) + head_offset_bytes(a, a.bh0 + c.hh) + 16 * (tid % LPR);
       unsigned char* dst = smem + st * kStage + tid * 16;
 #pragma unroll
@@ -1020,31 +1040,32 @@ __global__ void __launch_bounds__(kThreads, 2) prep_v_kernel(const PrepArgs a, i
   // per-item scalars of the quantizing stage, fetched one item ahead
   const int cp = tid % (D / 2);
   auto fetch_mu = [&](int item, const Cursor& c) -> float2 {
-    if (STAGE == kVStats || STAGE == kVQuant4 || STAGE == kVQuant4M || item >= n_items) return make_float2(0.f, 0.f);
+    if (STAGE == kVStats || STAGE == kVQuant4 || STAGE == kVQuant4M || item >= sl.n_items) return make_float2(0.f, 0.f);
     return *reinterpret_cast<const float2*>(a.v_mu + ((size_t)(a.bh0 + c.hh) * a.nb + c.blk) * D + 2 * cp);
   };
   // cursors of items i, i+1, i+2 and i+4 of this CTA
-  const int g = gridDim.x;
-  Cursor c0 = cursor_at(blockIdx.x, a.nb, nh), c1 = c0;
+  const int g = sl.stride;
+  Cursor c0 = cursor_at(sl.rank, a.nb, nh), c1 = c0;
   advance(c1, step, a.nb, nh);
   Cursor c2 = c1;
   advance(c2, step, a.nb, nh);
   Cursor c4 = c2;
   advance(c4, step, a.nb, nh);
   if (tid < kBlock) {
-    src_ring[tid] = fetch(blockIdx.x, c0);
-    src_ring[kBlock + tid] = fetch(blockIdx.x + g, c1);
+    src_ring[tid] = fetch(sl.rank, c0);
+    src_ring[kBlock + tid] = fetch(sl.rank + g, c1);
   }
   __syncthreads();
-  issue(blockIdx.x, c0, 0, src_ring);
-  issue(blockIdx.x + g, c1, 1, src_ring + kBlock);
+  issue(sl.rank, c0, 0, src_ring);
+  issue(sl.rank + g, c1, 1, src_ring + kBlock);
   __syncthreads();                            // the two slices have been read
-  if (tid < kBlock) src_ring[tid] = fetch(blockIdx.x + 2 * g, c2);
-  int nxt = fetch(blockIdx.x + 3 * g, c4);    // (c4 still stands at item 3 here)
+  if (tid < kBlock) src_ring[tid] = fetch(sl.rank + 2 * g, c2);
+  int nxt = fetch(sl.rank + 3 * g, c4);    // (c4 still stands at item 3 here)
   advance(c4, step, a.nb, nh);
-  float2 mu = fetch_mu(blockIdx.x, c0), am = make_float2(0.f, 0.f);
+  pdl_wait();                                 // (the inputs are in flight; the statistics may be read from here on)
+  float2 mu = fetch_mu(sl.rank, c0), am = make_float2(0.f, 0.f);
   int i = 0, last_hh = -1;
-  for (int item = blockIdx.x; item < n_items; item += g, ++i) {
+  for (int item = sl.rank; item < sl.n_items; item += g, ++i) {
     cp_async_wait<1>();                       // my chunks of item i have landed ...
     __syncthreads();                          // ... and everyone's; all are done with item i-1
     if (tid < kBlock) src_ring[((i + 1) & 1) * kBlock + tid] = nxt;     // source rows of item i+3
@@ -1072,35 +1093,29 @@ __global__ void __launch_bounds__(kThreads, 2) prep_v_kernel(const PrepArgs a, i
   }
 }
 
-// Launch 2: per-head finalization: K channel mean, V scale, g_Q.
+// Per-head finalization: K channel mean, V scale, g_Q.
 template <int D, int BITS>
 __global__ void prep_finalize_kernel(const PrepArgs a, int which) {
-  // which 0 / 2: a block of 8 D threads per head; the block partial sums are added in double, in
-  // eight interleaved slices that are then added in a fixed order
+  // which 0: a block of 8 D threads per head; the block partial sums are added in double, in eight
+  // interleaved slices that are then added in a fixed order.  which 1 (4 bits): the outer scale of K.
   __shared__ double part[8][D];
   const int bh = a.bh0 + blockIdx.x, c = threadIdx.x % D, slice = threadIdx.x / D;
-  if (which == 0 || which == 2) {
-    if (which == 0 && (a.flags & VC_FLAG_K_SMOOTH)) {
+  pdl_wait();
+  pdl_allow();
+  if (which == 0) {
+    if (a.flags & VC_FLAG_K_SMOOTH) {
       double s = 0.0;
+#pragma unroll 8
       for (int j = slice; j < a.nb; j += 8) s += (double)a.k_part[((size_t)bh * a.nb + j) * D + c];
       part[slice][c] = s;
       __syncthreads();
     }
     if (slice == 0) {
-      if (which == 2) {        // statistics from the caller: the mean as given (zero if K smoothing is off)
-        a.k_mean[(size_t)bh * D + c] = (a.flags & VC_FLAG_K_SMOOTH) ? a.ext_k_mean[(size_t)bh * D + c] : 0.f;
-      } else {
-        double s = 0.0;
-        if (a.flags & VC_FLAG_K_SMOOTH)
-          for (int k = 0; k < 8; ++k) s += part[k][c];
-        a.k_mean[(size_t)bh * D + c] = (float)(s / (double)a.N);
-      }
-      float vs = 1.0f;
-      if (BITS == 8) {
-        const float am = __uint_as_float(a.v_amax[(size_t)bh * D + c]);
-        vs = am > 0.f ? am / 448.0f : 1.0f;
-      }
-      a.v_scale[(size_t)bh * D + c] = vs;
+      double s = 0.0;
+      if (a.flags & VC_FLAG_K_SMOOTH)
+        for (int k = 0; k < 8; ++k) s += part[k][c];
+      a.k_mean[(size_t)bh * D + c] = (float)(s / (double)a.N);
+      a.v_scale[(size_t)bh * D + c] = BITS == 8 ? value_scale(__uint_as_float(a.v_amax[(size_t)bh * D + c])) : 1.0f;
     }
     if (BITS == 4 && threadIdx.x == 0) {
       const float am = __uint_as_float(a.qk_amax[bh]);
@@ -1121,15 +1136,15 @@ __global__ void prep_finalize_kernel(const PrepArgs a, int which) {
 // of the block maximum.
 // Shared memory: [2 stages x 128 x pitch][out tile 128 x D][src ring 3 x 128][scratch][RoPE table].
 // FAST: the packed row transform (standard configuration), see qk_row_item_fast.
-template <int D, int STAGE, int TPR, bool FAST = false>
-__global__ void __launch_bounds__(kRowThreads * TPR, 2) prep_qk_kernel(const PrepArgs a, int n_items, int nh, int z0) {
+template <int D, int STAGE, bool FAST>
+__device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
+  constexpr int TPR = kTpr;
   constexpr int NT = kRowThreads * TPR;
   constexpr int kRowBytes = STAGE == kStageQuant4 ? D / 2 : D;      // code bytes per row
   constexpr int CPR = kRowBytes / 16;                                // 16-byte chunks per code row
   constexpr int RW = 32 / TPR;                                       // rows of a warp
   constexpr int LPR = D / 8;                                         // lanes on one input row
   constexpr int RPI = 32 / LPR;                                      // input rows per warp instruction
-  extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* out_tile = smem + 2 * Geo<D>::stage_bytes;
   int* src_ring = reinterpret_cast<int*>(out_tile + kBlock * D);     // [3][128]
   float* red = reinterpret_cast<float*>(src_ring + 3 * kBlock);      // [2][16]
@@ -1138,11 +1153,10 @@ __global__ void __launch_bounds__(kRowThreads * TPR, 2) prep_qk_kernel(const Pre
   if (FAST) {
     for (int c = tid; c < D; c += NT) kmean_s[c] = 0.f;    // (m+, m-) pairs: zeros until a smoothed K head arrives
   }
-  const RopeTab tab = stage_rope_table(a, reinterpret_cast<unsigned char*>(kmean_s + D), FAST);
   const int my_row = qk_row_of<TPR>(tid);
-  const CursorStep step = cursor_step(a.nb);
+  const CursorStep step = cursor_step(sl.stride, a.nb);
   auto fetch = [&](int item, const Cursor& c) -> int {   // input row behind row `row0 + lane` of the item, -1 if none
-    if (item >= n_items || lane >= RW) return -1;
+    if (item >= sl.n_items || lane >= RW) return -1;
     const int t = c.blk * kBlock + row0 + lane;
     if (t >= a.N) return -1;
     // the head amax is a maximum over all rows: that stage reads the rows in place
@@ -1150,7 +1164,7 @@ __global__ void __launch_bounds__(kRowThreads * TPR, 2) prep_qk_kernel(const Pre
     return gather ? min(max(__ldg(&a.perm[(size_t)(a.bh0 + c.hh) * a.N + t]), 0), a.N - 1) : t;   // clamped: never a bad address
   };
   auto issue = [&](int item, const Cursor& c, int st, const int* src) {
-    if (item < n_items) {
+    if (item < sl.n_items) {
       const char* base = reinterpret_cast<const char*>((c.z + z0) == 0 ? a.q : a.k) + head_offset_bytes(a, a.bh0 + c.hh) + 16 * (lane % LPR);
       unsigned char* dst = smem + st * Geo<D>::stage_bytes + 16 * (lane % LPR) + (row0 + lane / LPR) * Geo<D>::pitch;
 #pragma unroll
@@ -1162,21 +1176,23 @@ __global__ void __launch_bounds__(kRowThreads * TPR, 2) prep_qk_kernel(const Pre
     cp_async_commit();
   };
   // cursors of items i, i+1 and i+3 of this CTA
-  const int g = gridDim.x;
-  Cursor c0 = cursor_at(blockIdx.x, a.nb, nh), c1 = c0;
+  const int g = sl.stride;
+  Cursor c0 = cursor_at(sl.rank, a.nb, nh), c1 = c0;
   advance(c1, step, a.nb, nh);
   Cursor c3 = c1;
   advance(c3, step, a.nb, nh);
   if (lane < RW) {
-    src_ring[row0 + lane] = fetch(blockIdx.x, c0);
-    src_ring[kBlock + row0 + lane] = fetch(blockIdx.x + g, c1);
+    src_ring[row0 + lane] = fetch(sl.rank, c0);
+    src_ring[kBlock + row0 + lane] = fetch(sl.rank + g, c1);
   }
-  int nxt = fetch(blockIdx.x + 2 * g, c3);    // (c3 still stands at item 2 here)
+  int nxt = fetch(sl.rank + 2 * g, c3);    // (c3 still stands at item 2 here)
   advance(c3, step, a.nb, nh);
   __syncwarp();
-  issue(blockIdx.x, c0, 0, src_ring);
+  issue(sl.rank, c0, 0, src_ring);
+  pdl_wait();                                 // (the first rows are in flight)
+  const RopeTab tab = stage_rope_table(a, reinterpret_cast<unsigned char*>(kmean_s + D), FAST);
   int i = 0, last_hh = -1;
-  for (int item = blockIdx.x; item < n_items; item += g, ++i) {
+  for (int item = sl.rank; item < sl.n_items; item += g, ++i) {
     cp_async_wait<0>();                       // my chunks of item i have landed ...
     __syncwarp();                             // ... and the warp's; the warp is done with item i-1
     if (lane < RW) src_ring[((i + 2) % 3) * kBlock + row0 + lane] = nxt;
@@ -1206,86 +1222,118 @@ __global__ void __launch_bounds__(kRowThreads * TPR, 2) prep_qk_kernel(const Pre
   }
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+// ---------------------------------------------------------------------------------------
+// Launches.  Passes that do not depend on one another share one: the statistics passes wait on their
+// copies, the Q/K row transform on instruction issue and the shared-memory pipe, so CTAs of both kinds
+// on an SM overlap where either kind alone leaves the other resource idle.  Each pass gets a share of
+// the CTAs (2 per SM) in proportion to what it costs alone.
+//   8 bits  1: K column sums | V statistics | Q codes      2: K codes | V codes
+//   4 bits  1: K column sums | Q head maximum | V codes    2: K head maximum | Q codes    3: K codes
+// with the per-head finalization in between.
+enum { kPhase1 = 1, kPhase2 = 2, kPhase3 = 3 };
+
+// Time of 128 rows of each pass relative to the Q/K quantizing pass (measured alone at B1 H40 N32760).
+constexpr float kCostRows = 1.0f, kCostAmax = 0.9f, kCostSums = 0.53f, kCostVStats = 0.47f, kCostV8 = 0.7f, kCostV4 = 1.0f;
+
+struct Share {
+  int n0, n1, n2;            // CTAs of the launch's passes, in order of their CTA numbers
+  int i0, i1, i2;            // their items
+  int z0;                    // first tensor of the Q/K quantizing pass (0 = Q, 1 = K)
+};
+
+template <int D, int BITS, int PHASE, bool FAST, int VARIANT>   // VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits)
+__global__ void __launch_bounds__(kThreads, 2) prep_kernel(const PrepArgs a, const Share s, int nh) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  pdl_allow();
+  constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
+  const int b = blockIdx.x;
+  if (BITS == 8 && PHASE == kPhase1) {
+    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
+    else if (b < s.n0 + s.n1) kcolsum_pass<D>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
+    else v_pass<D, kVStats>(a, smem, Slot{b - s.n0 - s.n1, s.n2, s.i2}, nh);
+  } else if (BITS == 8) {
+    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, s.z0);
+    else v_pass<D, kVQuant8>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
+  } else if (PHASE == kPhase1) {
+    if (b < s.n0) qk_pass<D, kStageAmax, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
+    else if (b < s.n0 + s.n1) kcolsum_pass<D>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
+    else v_pass<D, VARIANT ? kVQuant4M : kVQuant4>(a, smem, Slot{b - s.n0 - s.n1, s.n2, s.i2}, nh);
+  } else if (PHASE == kPhase2) {
+    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
+    else qk_pass<D, kStageAmax, FAST>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh, 1);
+  } else {
+    qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 1);
+  }
 }
 
-int persistent_grid(int n_items, int per_sm = 2) {
-  const int g = per_sm * sm_count();
-  return n_items < g ? n_items : g;
+// CTAs of each pass: all of them while they fit two per SM, else in proportion to items x cost.
+inline Share share_ctas(int i0, float c0, int i1, float c1, int i2, float c2, int z0) {
+  Share s{i0, i1, i2, i0, i1, i2, z0};
+  const int total = 2 * sm_count();
+  if (i0 + i1 + i2 <= total) return s;
+  const float w0 = i0 * c0, w1 = i1 * c1, w2 = i2 * c2, w = w0 + w1 + w2;
+  auto part = [&](float x, int items) { return items == 0 ? 0 : (int)(x / w * total) < 1 ? 1 : (int)(x / w * total) > items ? items : (int)(x / w * total); };
+  s.n1 = part(w1, i1);
+  s.n2 = part(w2, i2);
+  s.n0 = total - s.n1 - s.n2 < i0 ? total - s.n1 - s.n2 : i0;
+  return s;
 }
 
-template <int D, int BITS>
-cudaError_t run(const Problem& pr, PrepArgs a, const WorkLayout& wl, uint8_t* work, cudaStream_t s) {
+template <auto KERNEL>
+cudaError_t launch_phase(const PrepArgs& a, const Share& sh, int nh, size_t smem, cudaStream_t s) {
+  cudaError_t e = allow_smem<KERNEL>();
+  if (e == cudaSuccess) e = launch_overlapped(KERNEL, dim3((unsigned)(sh.n0 + sh.n1 + sh.n2)), kThreads, smem, s, a, sh, nh);
+  count_launches(1);
+  return e;
+}
+
+template <int D, int BITS, bool FAST, int VARIANT>
+cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
+  static_assert(kRowThreads * kTpr == kThreads, "the passes of a launch have the same block size");
   const size_t rope_bytes = ((a.flags & VC_FLAG_ROPE) && a.rope_in_smem) ? (size_t)a.rd.entries * 8 : 0;
   const size_t colsum_smem = 2 * (size_t)kThreads * (D / 16) * 16 + 8 * D * 4 + rope_bytes;
   const size_t row_smem = 2 * (size_t)Geo<D>::stage_bytes + (size_t)kBlock * D + 3 * kBlock * 4 + 128 + D * 4 + rope_bytes;
   const size_t v_smem = 3 * (size_t)kBlock * 2 * D + 16 * D * 4 + 2 * kBlock * 4;
-  constexpr int kQuant = BITS == 8 ? kStageQuant8 : kStageQuant4;
-  constexpr int kTpr = VC_PREP_TPR;            // threads per Q/K row
-  constexpr int kTprF = D == 128 ? VC_PREP_TPR_FAST : VC_PREP_TPR;   // ... of the packed row transform
-  constexpr int kVQuant = BITS == 8 ? kVQuant8 : kVQuant4;
-  cudaError_t e;
-  if ((e = allow_smem(prep_kcolsum_kernel<D>, colsum_smem)) != cudaSuccess) return e;
-  if ((e = allow_smem(prep_v_kernel<D, kVStats>, v_smem)) != cudaSuccess) return e;
-  if ((e = allow_smem(prep_v_kernel<D, kVQuant>, v_smem)) != cudaSuccess) return e;
-  if (BITS == 4 && (e = allow_smem(prep_v_kernel<D, kVQuant4M>, v_smem)) != cudaSuccess) return e;
-  const bool v_pow2 = hybrid4(pr);           // 4-bit values under power-of-two factors per 32 tokens
-  if ((e = allow_smem(prep_qk_kernel<D, kQuant, kTpr>, row_smem)) != cudaSuccess) return e;
-  if (BITS == 8 && (e = allow_smem(prep_qk_kernel<D, kStageQuant8I, kTpr>, row_smem)) != cudaSuccess) return e;
-  if (BITS == 8 && (e = allow_smem(prep_qk_kernel<D, kStageQuant8, kTprF, true>, row_smem)) != cudaSuccess) return e;
-  if (BITS == 8 && (e = allow_smem(prep_qk_kernel<D, kStageQuant8I, kTprF, true>, row_smem)) != cudaSuccess) return e;
-  // the packed row transform serves the standard configuration
-  const bool fast = (a.flags & VC_FLAG_ROPE) && (a.flags & VC_FLAG_HADAMARD) && a.rope_default && a.rope_in_smem;
-  if (BITS == 4 && (e = allow_smem(prep_qk_kernel<D, kStageAmax, kTpr>, row_smem)) != cudaSuccess) return e;
-  if (BITS == 4 && (e = allow_smem(prep_qk_kernel<D, kStageAmax, kTprF, true>, row_smem)) != cudaSuccess) return e;
-  if (BITS == 4 && (e = allow_smem(prep_qk_kernel<D, kStageQuant4, kTprF, true>, row_smem)) != cudaSuccess) return e;
+  const size_t smem = row_smem > v_smem ? row_smem : v_smem;
+  static_assert(2 * kThreads * (D / 16) * 16 + 8 * D * 4 <= 2 * Geo<D>::stage_bytes + kBlock * D, "the column sums fit the row pass's share");
+  (void)colsum_smem;
+  cudaError_t e = cudaSuccess;
   int group = pr.heads_per_pass > 0 ? pr.heads_per_pass : pr.BH;
   if (group > 32768) group = 32768;
-  for (int bh0 = 0; bh0 < pr.BH; bh0 += group) {
+  for (int bh0 = 0; bh0 < pr.BH && e == cudaSuccess; bh0 += group) {
     const int nh = pr.BH - bh0 < group ? pr.BH - bh0 : group;
     const int per = pr.nb * nh;
     a.bh0 = bh0;
-    const bool ext = a.ext_k_mean != nullptr;     // the caller supplied the statistics: no statistics launches
-    if ((a.flags & VC_FLAG_K_SMOOTH) && !ext) {
-      prep_kcolsum_kernel<D><<<persistent_grid(per), kThreads, colsum_smem, s>>>(a, per, nh);
-      count_launches(1);
-    }
-    if (BITS == 8 && !ext) { prep_v_kernel<D, kVStats><<<persistent_grid(per), kThreads, v_smem, s>>>(a, per, nh); count_launches(1); }
-    auto amax_pass = [&](int z0) {
-      if (fast) prep_qk_kernel<D, kStageAmax, kTprF, true><<<persistent_grid(per), kRowThreads * kTprF, row_smem, s>>>(a, per, nh, z0);
-      else prep_qk_kernel<D, kStageAmax, kTpr><<<persistent_grid(per), kRowThreads * kTpr, row_smem, s>>>(a, per, nh, z0);
+    const bool ext = a.ext_k_mean != nullptr;     // the caller supplied the statistics: no statistics passes
+    const int sums = a.flags & VC_FLAG_K_SMOOTH ? per : 0;
+    auto finalize = [&](int which, int threads) {
+      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
       count_launches(1);
     };
-    if (BITS == 4) amax_pass(0);
-    prep_finalize_kernel<D, BITS><<<nh, 8 * D, 0, s>>>(a, ext ? 2 : 0);
-    count_launches(1);
-    if (BITS == 4) {
-      amax_pass(1);
-      prep_finalize_kernel<D, BITS><<<nh, 32, 0, s>>>(a, 1);
-      count_launches(1);
-    }
     if constexpr (BITS == 8) {
-      if (fast && (a.flags & VC_FLAG_INT8_QK))
-        prep_qk_kernel<D, kStageQuant8I, kTprF, true><<<persistent_grid(2 * per), kRowThreads * kTprF, row_smem, s>>>(a, 2 * per, nh, 0);
-      else if (fast)
-        prep_qk_kernel<D, kStageQuant8, kTprF, true><<<persistent_grid(2 * per), kRowThreads * kTprF, row_smem, s>>>(a, 2 * per, nh, 0);
-      else if (a.flags & VC_FLAG_INT8_QK)
-        prep_qk_kernel<D, kStageQuant8I, kTpr><<<persistent_grid(2 * per), kRowThreads * kTpr, row_smem, s>>>(a, 2 * per, nh, 0);
-      else
-        prep_qk_kernel<D, kStageQuant8, kTpr><<<persistent_grid(2 * per), kRowThreads * kTpr, row_smem, s>>>(a, 2 * per, nh, 0);
+      if (!ext) e = launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT>>(a, share_ctas(per, kCostRows, sums, kCostSums, per, kCostVStats, 0), nh, smem, s);
+      if (!ext) finalize(0, 8 * D);
+      // (with supplied statistics Q has no launch of its own to share)
+      const Share sh = ext ? share_ctas(2 * per, kCostRows, per, kCostV8, 0, 0.f, 0) : share_ctas(per, kCostRows, per, kCostV8, 0, 0.f, 1);
+      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT>>(a, sh, nh, smem, s);
     } else {
-      if (fast) prep_qk_kernel<D, kStageQuant4, kTprF, true><<<persistent_grid(2 * per), kRowThreads * kTprF, row_smem, s>>>(a, 2 * per, nh, 0);
-      else prep_qk_kernel<D, kStageQuant4, kTpr><<<persistent_grid(2 * per), kRowThreads * kTpr, row_smem, s>>>(a, 2 * per, nh, 0);
+      e = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT>>(a, share_ctas(per, kCostAmax, sums, kCostSums, per, kCostV4, 0), nh, smem, s);
+      finalize(0, 8 * D);
+      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0>>(a, share_ctas(per, kCostRows, per, kCostAmax, 0, 0.f, 0), nh, smem, s);
+      finalize(1, 32);
+      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0>>(a, share_ctas(per, kCostRows, 0, 0.f, 0, 0.f, 1), nh, smem, s);
     }
-    if (BITS == 4 && v_pow2)
-      prep_v_kernel<D, kVQuant4M><<<persistent_grid(per), kThreads, v_smem, s>>>(a, per, nh);
-    else
-      prep_v_kernel<D, kVQuant><<<persistent_grid(per), kThreads, v_smem, s>>>(a, per, nh);
-    count_launches(2);
   }
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <int D, int BITS>
+cudaError_t run(const Problem& pr, const PrepArgs& a, cudaStream_t s) {
+  // the packed row transform serves the standard configuration
+  const bool fast = (a.flags & VC_FLAG_ROPE) && (a.flags & VC_FLAG_HADAMARD) && a.rope_default && a.rope_in_smem;
+  const bool variant = BITS == 8 ? (a.flags & VC_FLAG_INT8_QK) != 0 : hybrid4(pr);
+  if (fast) return variant ? run_phases<D, BITS, true, 1>(pr, a, s) : run_phases<D, BITS, true, 0>(pr, a, s);
+  return variant ? run_phases<D, BITS, false, 1>(pr, a, s) : run_phases<D, BITS, false, 0>(pr, a, s);
 }
 
 }  // namespace
@@ -1333,17 +1381,29 @@ cudaError_t launch_prep(const Problem& pr, const QuantLayout& ql, const WorkLayo
     const int sdef = 2 * (pr.d / 6);
     a.rope_default = pr.rope_dim[0] == pr.d - 2 * sdef && pr.rope_dim[1] == sdef && pr.rope_dim[2] == sdef;
   }
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(work + wl.status, 0, 4, stream)) != cudaSuccess) return e;
-  if (!ext && (e = cudaMemsetAsync(work + wl.amax, 0, wl.amax_bytes, stream)) != cudaSuccess) return e;
-  if (a.flags & VC_FLAG_ROPE) {
-    rope_table_kernel<<<(a.rd.entries + 255) / 256, 256, 0, stream>>>(
-        reinterpret_cast<float2*>(work + wl.rope), a.rd, (double)pr.rope_theta);
-    count_launches(1);
+  // the table (one thread per entry), the words that start at zero, supplied statistics
+  SetUp u{};
+  u.status = reinterpret_cast<unsigned int*>(work + wl.status);
+  if (ext) {
+    u.n_ext = pr.BH * pr.d;
+    u.ext_k_mean = (pr.flags & VC_FLAG_K_SMOOTH) ? stats->k_mean : nullptr;
+    u.ext_v_amax = stats->v_amax;
+    u.k_mean = a.k_mean;
+    u.v_scale = a.v_scale;
+  } else {
+    u.zero = reinterpret_cast<unsigned int*>(work + wl.amax);
+    u.n_zero = (int)(wl.amax_bytes / 4);
   }
+  RopeDesc rd = a.rd;
+  if (!(a.flags & VC_FLAG_ROPE)) rd.entries = 0;
+  const int words = (u.n_zero + u.n_ext + 3) / 4, need = rd.entries > words ? rd.entries : words;
+  cudaError_t e = launch_overlapped(rope_table_kernel, dim3((unsigned)(need / 64 + 1)), 64, 0, stream, reinterpret_cast<float2*>(work + wl.rope), rd,
+                                    (double)pr.rope_theta, u);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
   if ((e = launch_perm_check(pr, perm, wl, work, stream)) != cudaSuccess) return e;
-  if (pr.d == 128) return pr.bits == 8 ? run<128, 8>(pr, a, wl, work, stream) : run<128, 4>(pr, a, wl, work, stream);
-  return pr.bits == 8 ? run<64, 8>(pr, a, wl, work, stream) : run<64, 4>(pr, a, wl, work, stream);
+  if (pr.d == 128) return pr.bits == 8 ? run<128, 8>(pr, a, stream) : run<128, 4>(pr, a, stream);
+  return pr.bits == 8 ? run<64, 8>(pr, a, stream) : run<64, 4>(pr, a, stream);
 }
 
 }  // namespace vc
