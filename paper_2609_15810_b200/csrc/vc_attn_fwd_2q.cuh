@@ -125,6 +125,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_allow();                              // (behind the allocation: the next kernel may want tensor memory too)
   const uint32_t tmem = sh->tmem_base;
   const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
 
@@ -433,7 +434,6 @@ template <int D, int PF, bool INT8, bool SMOOTH, bool ONE>
 __global__ void __launch_bounds__(640, 1)
 attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const AttnArgs a) {
-  pdl_allow();
   const TileOf w = tile_of(a.tiles, a.nb);
   if (w.q0 >= a.nb) return;                 // the missing second tile of a head's last pair
   if constexpr (ONE) {
