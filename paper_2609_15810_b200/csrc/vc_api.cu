@@ -280,6 +280,13 @@ vc_status vc_attn_host(const vc_params* p, const void* q_host, const void* k_hos
     for (; middle > 0; middle -= hg) sizes.push_back(middle < hg ? middle : hg);
     sizes.push_back(2 * mult);
     sizes.push_back(last);
+  } else if (pr.BH >= 4 * mult) {
+    // few heads: one group of the smallest size at each end (B1 H12 N32760 d128: 7.34 ms with six
+    // groups of two heads, 6.67 with 1, 2, 2, 2, 2, 2, 1)
+    const int last = mult + pr.BH % mult;
+    sizes.push_back(mult);
+    for (int middle = pr.BH - mult - last; middle > 0; middle -= hg) sizes.push_back(middle < hg ? middle : hg);
+    sizes.push_back(last);
   } else {
     for (int h = 0; h < pr.BH; h += hg) sizes.push_back(pr.BH - h < hg ? pr.BH - h : hg);
   }
