@@ -386,6 +386,10 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
     // ---- last tile's mean term, then the epilogue: O = s_V * A / l
+    // (Without block means nothing above has waited for the product in front of the last one on that
+    // barrier, and a parity wait would take the phase before it for the last.)
+    const int before = TWO ? nb - 2 : nb - 3;
+    if (!SMOOTH && ok && before >= 0) ok = warp_wait2(&sh->o_done[buf(t, before)], par(before), sh, a.wait, 44);
     if (ok && (ok = warp_wait2(&sh->o_done[buf(t, nb - 1)], par(nb - 1), sh, a.wait, 42))) {
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
