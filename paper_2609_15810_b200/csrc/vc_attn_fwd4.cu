@@ -105,7 +105,10 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   constexpr int kTmemCols = 512;
   constexpr int KB = D / 64;                        // K = 64 steps of the score product
   constexpr int kRowB = D / 2;                      // bytes per Q^/K^ row
-  constexpr uint32_t O_COL = 128, O_STRIDE = 144, L_COL = D, S1_COL = O_COL + O_STRIDE;
+  // d = 64 leaves room for a score buffer per query tile.  (B2 H16 N16384: hybrid 1.89 -> 1.88 ms; the
+  // NVFP4 probabilities, which keep a softmax warp busy twice as long, lose by it: 3.44 -> 3.64.)
+  constexpr bool kTwoS = D == 64 && HYB;
+  constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE;
   constexpr uint32_t SF_COL = 416;
   constexpr uint32_t SFQ_COL = SF_COL, SFK_COL = SF_COL + 16, SFP_COL = SF_COL + 24, SFV_COL = SF_COL + 40;
   constexpr int kRegCtl = 48, kRegSoftmax = 160, kRegCorr = 56;
@@ -235,7 +238,9 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
         const uint32_t sf_smem = smem_u32(base + kKBytes + kVBytes + kOnesBytes + kMuPad);
 #pragma unroll
         for (int t = 0; t < (TWO ? 2 : 1); ++t) {
-          if (TWO ? (t == 0 ? j > 0 : true) : j > 1) {
+          if (TWO && kTwoS) {
+            if (j > 0 && !(ok = warp_wait2(&sh->s_free[t], (j - 1) & 1, sh, a.wait, 22))) break;
+          } else if (TWO ? (t == 0 ? j > 0 : true) : j > 1) {
             if (!(ok = warp_wait2(&sh->s_free[TWO ? 1 - t : j & 1], TWO ? (t == 0 ? j - 1 : j) & 1 : par(j) ^ 1, sh, a.wait, 22))) break;
           }
           if (elect_one()) {
@@ -247,7 +252,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
             const uint64_t dq = t == 0 ? dq0 : dq1;
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb)
-              mma_nvfp4_ss(tmem + (TWO ? 0 : (j & 1) * S1_COL), dq + 2 * kb, dk + 2 * kb, idesc_qk, kb > 0, tmem + SFQ_COL + (t * KB + kb) * 4,
+              mma_nvfp4_ss(tmem + (TWO ? (kTwoS ? t * S1_COL : 0) : (j & 1) * S1_COL), dq + 2 * kb, dk + 2 * kb, idesc_qk, kb > 0, tmem + SFQ_COL + (t * KB + kb) * 4,
                            tmem + SFK_COL + kb * 4);
             mma_commit(&sh->s_full[buf(t, j)]);
           }
@@ -339,7 +344,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       if (!warp_wait2(&sh->s_full[buf(t, j)], par(j), sh, a.wait, 30)) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
-      const uint32_t s_col = lane_base + (TWO ? 0 : (j & 1) * S1_COL);
+      const uint32_t s_col = lane_base + (TWO ? (kTwoS ? t * S1_COL : 0) : (j & 1) * S1_COL);
       if (j == nb - 1 && (a.N & 127)) {                   // ragged last tile: padded keys score -inf
 #pragma unroll 1
         for (int c = a.N & 127; c < 128; ++c) tmem_st1(s_col + c, 0xff800000u);

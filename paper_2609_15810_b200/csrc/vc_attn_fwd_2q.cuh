@@ -76,7 +76,10 @@ template <int D, int PF, bool INT8, bool SMOOTH, bool TWO>
 __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                              const AttnArgs& a, const int q0, const int bh) {
   constexpr int kTmemCols = 512;
-  constexpr uint32_t O_COL = 128, O_STRIDE = 144, L_COL = D, S1_COL = O_COL + O_STRIDE;   // A_t at O_COL + t * O_STRIDE; l in its column d
+  // d = 64 leaves room in tensor memory for a score buffer per query tile (B2 H16 N16384 d64: 1.89 -> 1.83 ms,
+  // without smoothing 1.85 -> 1.76); at d = 128 both tiles share one
+  constexpr bool kTwoS = D == 64;
+  constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE;   // A_t at O_COL + t * O_STRIDE; l in its column d
   // Register re-partition (setmaxnreg): the CTA owns 640 x 96 registers; a warpgroup that asks for
   // more than the others released would block forever, so the budget is checked at compile time.
   constexpr int kRegCtl = 48, kRegSoftmax = 160, kRegCorr = 56;
@@ -173,13 +176,15 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
         for (int t = 0; t < (TWO ? 2 : 1); ++t) {
           // S_0(j) waits for the read of S_1(j-1), S_1(j) for the read of S_0(j); with one tile S(j) for
           // the read of S(j-2), the buffer's previous tenant
-          if (TWO ? (t == 0 ? j > 0 : true) : j > 1) {
+          if (TWO && kTwoS) {
+            if (j > 0 && !(ok = warp_wait2(&sh->s_free[t], (j - 1) & 1, sh, a.wait, 22))) break;
+          } else if (TWO ? (t == 0 ? j > 0 : true) : j > 1) {
             if (!(ok = warp_wait2(&sh->s_free[TWO ? 1 - t : j & 1], TWO ? (t == 0 ? j - 1 : j) & 1 : par(j) ^ 1, sh, a.wait, 22))) break;
           }
           if (elect_one()) {
             tc_fence_after();
             const uint64_t dq = t == 0 ? dq0 : dq1;
-            const uint32_t s_col = tmem + (TWO ? 0 : (j & 1) * S1_COL);
+            const uint32_t s_col = tmem + (TWO ? (kTwoS ? t * S1_COL : 0) : (j & 1) * S1_COL);
 #pragma unroll
             for (int k = 0; k < D / 32; ++k) {
               if constexpr (INT8) mma_s8_ss(s_col, dq + 2 * k, dk + 2 * k, idesc_qk, k > 0);
@@ -251,7 +256,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       if (!warp_wait2(&sh->s_full[buf(t, j)], par(j), sh, a.wait, 30)) break;
       tc_fence_after();
       uint32_t s0[32], s1[32], s2[32], s3[32];
-      const uint32_t s_col = lane_base + (TWO ? 0 : (j & 1) * S1_COL);
+      const uint32_t s_col = lane_base + (TWO ? (kTwoS ? t * S1_COL : 0) : (j & 1) * S1_COL);
       if (j == nb - 1 && (a.N & 127)) {                   // ragged last tile: padded keys score -inf
 #pragma unroll 1
         for (int c = a.N & 127; c < 128; ++c) tmem_st1(s_col + c, INT8 ? 0xff800000u - 0x4B400000u : 0xff800000u);
