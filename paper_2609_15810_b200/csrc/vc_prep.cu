@@ -1232,8 +1232,9 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
 // with the per-head finalization in between.
 enum { kPhase1 = 1, kPhase2 = 2, kPhase3 = 3 };
 
-// Time of 128 rows of each pass relative to the Q/K quantizing pass (measured alone at B1 H40 N32760).
-constexpr float kCostRows = 1.0f, kCostAmax = 0.9f, kCostSums = 0.53f, kCostVStats = 0.47f, kCostV8 = 0.7f, kCostV4 = 1.0f;
+// Time of 128 rows of each pass relative to the Q/K quantizing pass, tuned with the passes side by side
+// (B1 H40 N32760 573 -> 569 us, B1 H12 N32760 190 -> 186 against the ratios measured alone).
+constexpr float kCostRows = 1.0f, kCostAmax = 0.9f, kCostSums = 0.6f, kCostVStats = 0.47f, kCostV8 = 0.66f, kCostV4 = 1.0f;
 
 struct Share {
   int n0, n1, n2;            // CTAs of the launch's passes, in order of their CTA numbers
