@@ -267,34 +267,30 @@ template <> struct RopeSplit<128> { static constexpr int p1 = 22, p2 = 43; };   
 template <> struct RopeSplit<64> { static constexpr int p1 = 12, p2 = 22; };    // 24 / 20 / 20
 
 // Reads the thread's row out of the stage, releases the stage, then transforms the row.
-// `red` is [2][4] floats and `kmean_s` [D] floats of compute-warp scratch.
+// `red` is [2][8] floats and `kmean_s` [D] floats of compute-warp scratch.
 // Q and K run through one copy of the row body (TENSOR is a run-time argument): the unrolled body
 // is tens of KB of code, and two copies of it thrash the instruction cache.
 //
-// TPR = threads per row.  With TPR = 1 a thread holds all D channels of its row.  With TPR = 2 the
-// lanes 0..15 of a warp hold channels [0, D/2) of 16 rows and the lanes 16..31 channels [D/2, D)
-// of the same rows: half the registers per thread, so twice the warps per SM; the last Hadamard
-// level crosses the two halves with one shuffle per value.  RoPE pairs and NVFP4 groups stay
-// thread-local either way.
-template <int TPR> __device__ __forceinline__ int qk_row_of(int tid) {
-  return TPR == 1 ? tid : (TPR == 2 ? 16 * (tid >> 5) + (tid & 15) : 8 * (tid >> 5) + (tid & 7));
-}
-template <int TPR> __device__ __forceinline__ int qk_part_of(int tid) {
-  return TPR == 1 ? 0 : (TPR == 2 ? (tid >> 4) & 1 : (tid >> 3) & 3);
-}
+// Two threads per row (kTpr): the lanes 0..15 of a warp hold channels [0, D/2) of 16 rows and the
+// lanes 16..31 channels [D/2, D) of the same rows; the last Hadamard level crosses the two halves with
+// one shuffle per value.  RoPE pairs and NVFP4 groups stay thread-local.  (Measured against it: one
+// thread per row needs twice the registers, so half the warps per SM; four threads per row add a second
+// shuffle level to the shared-memory pipe, B1 H40 N32760 0.70 instead of 0.60 ms.)
+__device__ __forceinline__ int qk_row_of(int tid) { return 16 * (tid >> 5) + (tid & 15); }
+__device__ __forceinline__ int qk_part_of(int tid) { return (tid >> 4) & 1; }
 
 template <int D> __device__ __forceinline__ constexpr int rope_axis_of(int p) {
   return p < RopeSplit<D>::p1 ? 0 : (p < RopeSplit<D>::p2 ? 1 : 2);
 }
 
-template <int D, int STAGE, int TPR>
+template <int D, int STAGE>
 __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR /*0 = Q, 1 = K*/, const unsigned char* stage,
                                             unsigned char* out_tile, float* red, float* kmean_s, const RopeTab& tab, int bh,
                                             int blk, int iter, bool new_head, int src_row) {
-  constexpr int C = D / TPR;                       // channels per thread
-  constexpr int NT = kRowThreads * TPR;
+  constexpr int C = D / kTpr;                      // channels per thread
+  constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row = qk_row_of<TPR>(tid), part = qk_part_of<TPR>(tid);
+  const int row = qk_row_of(tid), part = qk_part_of(tid);
   const bool do_rope = a.flags & VC_FLAG_ROPE;
   const bool do_had = a.flags & VC_FLAG_HADAMARD;
   const bool center = TENSOR == 1 && (a.flags & VC_FLAG_K_SMOOTH);
@@ -342,7 +338,7 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
         for (int a1 = 0; a1 < 3; ++a1) base[a0][a1] = (part ? e[a1] : e[a0]) + p0;
 #pragma unroll
       for (int i = 0; i < C / 2; ++i) {
-        const float2 cs = rope_entry_s(tab.saddr, base[rope_axis_of<D>(i)][rope_axis_of<D>(TPR == 1 ? i : C / 2 + i)] + i);
+        const float2 cs = rope_entry_s(tab.saddr, base[rope_axis_of<D>(i)][rope_axis_of<D>(C / 2 + i)] + i);
         const float x0 = x[2 * i], x1 = x[2 * i + 1];
         x[2 * i] = x0 * cs.x - x1 * cs.y;
         x[2 * i + 1] = x0 * cs.y + x1 * cs.x;
@@ -379,13 +375,11 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
         }
       }
     }
-    if constexpr (TPR == 2) {
-      // the level that pairs channel c with c + D/2: the lower half takes mine + theirs, the upper
-      // half theirs - mine (one fused multiply-add with +-1, exact)
-      const float sgn = part ? -1.0f : 1.0f;
+    // the level that pairs channel c with c + D/2: the lower half takes mine + theirs, the upper
+    // half theirs - mine (one fused multiply-add with +-1, exact)
+    const float sgn = part ? -1.0f : 1.0f;
 #pragma unroll
-      for (int c = 0; c < C; ++c) x[c] = fmaf(x[c], sgn, __shfl_xor_sync(0xffffffffu, x[c], 16));
-    }
+    for (int c = 0; c < C; ++c) x[c] = fmaf(x[c], sgn, __shfl_xor_sync(0xffffffffu, x[c], 16));
   }
   const float rs = do_had ? (D == 128 ? 0.08838834764831845f : 0.125f) : 1.0f;   // 1/sqrt(D)
 
@@ -402,7 +396,7 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
     if (lane == 0) rbuf[warp] = amax;
     __syncthreads();
     amax = fmaxf(fmaxf(rbuf[0], rbuf[1]), fmaxf(rbuf[2], rbuf[3]));
-    if constexpr (TPR == 2) amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
+    amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
     if (tid == 0) atomicMax(&a.qk_amax[TENSOR * a.BH + bh], __float_as_uint(amax));
@@ -499,14 +493,14 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 //  * at 8 bits 1 / sqrt(D) and the quantization scale are one factor.
 // The 4-bit head-maximum and NVFP4 stages run on the same transform.
 // `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed.
-template <int D, int STAGE, int TPR>
+template <int D, int STAGE>
 __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TENSOR, const unsigned char* stage,
                                                  unsigned char* out_tile, float* red, float* kmean_pm, uint32_t tab_saddr,
                                                  int bh, int blk, int iter, bool new_head, int src_row) {
-  constexpr int C = D / TPR, P = C / 2;            // channels and pairs per thread
-  constexpr int NT = kRowThreads * TPR;
+  constexpr int C = D / kTpr, P = C / 2;           // channels and pairs per thread
+  constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row = qk_row_of<TPR>(tid), part = qk_part_of<TPR>(tid);
+  const int row = qk_row_of(tid), part = qk_part_of(tid);
   const bool valid = src_row >= 0;
   const int src = valid ? src_row : 0;
   uint4 raw[C / 8];
@@ -530,10 +524,7 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
   // compile time for either part: one base per combination, selected once per row)
   // (written as a selection per pair; identical selections fold into one value per combination)
   auto base_of = [&](int i) -> uint32_t {          // i is a compile-time constant after unrolling
-    int ee;
-    if constexpr (TPR == 1) ee = e[rope_axis_of<D>(i)];
-    else if constexpr (TPR == 2) ee = part ? e[rope_axis_of<D>(P + i)] : e[rope_axis_of<D>(i)];
-    else ee = part == 0 ? e[rope_axis_of<D>(i)] : (part == 1 ? e[rope_axis_of<D>(P + i)] : (part == 2 ? e[rope_axis_of<D>(2 * P + i)] : e[rope_axis_of<D>(3 * P + i)]));
+    const int ee = part ? e[rope_axis_of<D>(P + i)] : e[rope_axis_of<D>(i)];
     return tab_saddr + 8u * (uint32_t)(ee + p0);
   };
   const float4* km = reinterpret_cast<const float4*>(kmean_pm + part * C);
@@ -572,22 +563,15 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
       }
     }
   }
-  if constexpr (TPR >= 2) {
-    // the levels that pair channels across the threads of a row (distance C, then 2 C with four
-    // threads per row): the lower part takes mine + theirs, the upper part theirs - mine
+  // the level that pairs channel c with c + D/2: the lower half takes mine + theirs, the upper half theirs - mine
+  const float sg = part ? -1.0f : 1.0f;
+  const uint64_t SG = pack_f32x2(sg, sg);
 #pragma unroll
-    for (int lv = 0; lv < (TPR == 2 ? 1 : 2); ++lv) {
-      const int mask = TPR == 2 ? 16 : (lv == 0 ? 8 : 16);
-      const float sg = ((part >> lv) & 1) ? -1.0f : 1.0f;
-      const uint64_t SG = pack_f32x2(sg, sg);
-#pragma unroll
-      for (int i = 0; i < P; ++i) {
-        float lo, hi;
-        unpack2(X[i], lo, hi);
-        const float olo = __shfl_xor_sync(0xffffffffu, lo, mask), ohi = __shfl_xor_sync(0xffffffffu, hi, mask);
-        X[i] = fma2(X[i], SG, pack_f32x2(olo, ohi));
-      }
-    }
+  for (int i = 0; i < P; ++i) {
+    float lo, hi;
+    unpack2(X[i], lo, hi);
+    const float olo = __shfl_xor_sync(0xffffffffu, lo, 16), ohi = __shfl_xor_sync(0xffffffffu, hi, 16);
+    X[i] = fma2(X[i], SG, pack_f32x2(olo, ohi));
   }
   constexpr float rs = D == 128 ? 0.08838834764831845f : 0.125f;   // 1/sqrt(D)
 
@@ -603,15 +587,11 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
       m1 = max3(m1, fabsf(b0), fabsf(b1));
     }
     amax = warp_max(fmaxf(m0, m1) * rs);           // max and the (positive) scale commute exactly
-    float* rbuf = red + 16 * (iter & 1);           // alternate buffers: one barrier per item suffices
+    float* rbuf = red + 8 * (iter & 1);            // alternate buffers: one barrier per item suffices
     if (lane == 0) rbuf[warp] = amax;
     __syncthreads();
     amax = fmaxf(fmaxf(rbuf[0], rbuf[1]), fmaxf(rbuf[2], rbuf[3]));
-    if constexpr (TPR >= 2) amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
-    if constexpr (TPR == 4) {
-      amax = fmaxf(amax, fmaxf(fmaxf(rbuf[8], rbuf[9]), fmaxf(rbuf[10], rbuf[11])));
-      amax = fmaxf(amax, fmaxf(fmaxf(rbuf[12], rbuf[13]), fmaxf(rbuf[14], rbuf[15])));
-    }
+    amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
     if (tid == 0) atomicMax(&a.qk_amax[TENSOR * a.BH + bh], __float_as_uint(amax));
@@ -1128,7 +1108,7 @@ __global__ void prep_finalize_kernel(const PrepArgs a, int which) {
 }
 
 // Q/K pass: STAGE = amax (4-bit head amax of tensor z0), or quantization of Q (z = 0) and K
-// (z = 1).  A warp owns 32 / TPR rows of the block from end to end: it copies them in (consecutive
+// (z = 1).  A warp owns 32 / kTpr rows of the block from end to end: it copies them in (consecutive
 // lanes on consecutive 16-byte chunks, the source rows taken from a small ring of permutation
 // entries in shared memory), its threads read their rows from the padded tile, and the rows'
 // codes leave through the warp's slice of a swizzled tile, again with full-line stores.  So the
@@ -1138,22 +1118,21 @@ __global__ void prep_finalize_kernel(const PrepArgs a, int which) {
 // FAST: the packed row transform (standard configuration), see qk_row_item_fast.
 template <int D, int STAGE, bool FAST>
 __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
-  constexpr int TPR = kTpr;
-  constexpr int NT = kRowThreads * TPR;
+  constexpr int NT = kRowThreads * kTpr;
   constexpr int kRowBytes = STAGE == kStageQuant4 ? D / 2 : D;      // code bytes per row
   constexpr int CPR = kRowBytes / 16;                                // 16-byte chunks per code row
-  constexpr int RW = 32 / TPR;                                       // rows of a warp
+  constexpr int RW = 32 / kTpr;                                      // rows of a warp
   constexpr int LPR = D / 8;                                         // lanes on one input row
   constexpr int RPI = 32 / LPR;                                      // input rows per warp instruction
   unsigned char* out_tile = smem + 2 * Geo<D>::stage_bytes;
   int* src_ring = reinterpret_cast<int*>(out_tile + kBlock * D);     // [3][128]
-  float* red = reinterpret_cast<float*>(src_ring + 3 * kBlock);      // [2][16]
-  float* kmean_s = red + 32;                                         // [D]
+  float* red = reinterpret_cast<float*>(src_ring + 3 * kBlock);      // [2][8]
+  float* kmean_s = red + 16;                                         // [D]
   const int tid = threadIdx.x, lane = tid & 31, row0 = (tid >> 5) * RW;
   if (FAST) {
     for (int c = tid; c < D; c += NT) kmean_s[c] = 0.f;    // (m+, m-) pairs: zeros until a smoothed K head arrives
   }
-  const int my_row = qk_row_of<TPR>(tid);
+  const int my_row = qk_row_of(tid);
   const CursorStep step = cursor_step(sl.stride, a.nb);
   auto fetch = [&](int item, const Cursor& c) -> int {   // input row behind row `row0 + lane` of the item, -1 if none
     if (item >= sl.n_items || lane >= RW) return -1;
@@ -1202,9 +1181,9 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
     const int s0 = src_ring[(i % 3) * kBlock + my_row];
     const int tensor = c0.z + z0, bh = a.bh0 + c0.hh;
     if constexpr (FAST)
-      qk_row_item_fast<D, STAGE, TPR>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
+      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
     else
-      qk_row_item<D, STAGE, TPR>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
+      qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
     if (tensor == 1) last_hh = c0.hh;
     if constexpr (STAGE != kStageAmax) {
       __syncwarp();                           // the warp's rows of the code tile are complete
@@ -1294,12 +1273,10 @@ template <int D, int BITS, bool FAST, int VARIANT>
 cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
   static_assert(kRowThreads * kTpr == kThreads, "the passes of a launch have the same block size");
   const size_t rope_bytes = ((a.flags & VC_FLAG_ROPE) && a.rope_in_smem) ? (size_t)a.rd.entries * 8 : 0;
-  const size_t colsum_smem = 2 * (size_t)kThreads * (D / 16) * 16 + 8 * D * 4 + rope_bytes;
-  const size_t row_smem = 2 * (size_t)Geo<D>::stage_bytes + (size_t)kBlock * D + 3 * kBlock * 4 + 128 + D * 4 + rope_bytes;
+  const size_t row_smem = 2 * (size_t)Geo<D>::stage_bytes + (size_t)kBlock * D + 3 * kBlock * 4 + 64 + D * 4 + rope_bytes;
   const size_t v_smem = 3 * (size_t)kBlock * 2 * D + 16 * D * 4 + 2 * kBlock * 4;
   const size_t smem = row_smem > v_smem ? row_smem : v_smem;
   static_assert(2 * kThreads * (D / 16) * 16 + 8 * D * 4 <= 2 * Geo<D>::stage_bytes + kBlock * D, "the column sums fit the row pass's share");
-  (void)colsum_smem;
   cudaError_t e = cudaSuccess;
   int group = pr.heads_per_pass > 0 ? pr.heads_per_pass : pr.BH;
   if (group > 32768) group = 32768;
