@@ -21,15 +21,24 @@ using namespace attn;
 // feeds 256 query rows.  Two decisions keep the softmax stage - the bottleneck on this GPU -
 // as short as the method allows:
 //   * The probability codes travel through SHARED memory, not through tensor memory, so a
-//     score tile is free as soon as its 128 x 128 values are in registers; one score buffer
-//     serves both query tiles in turn and S_t(j+1) is ready long before it is needed.
+//     score tile is free as soon as its 128 x 128 values are in registers.  At d = 128 one score
+//     buffer serves both query tiles in turn (all that tensor memory has room for); at d = 64 each
+//     tile has its own.
 //   * The row sums of the decoded codes (Eq. 6: r_ij, and the normalizer l) come from the
 //     tensor core: the value operand carries 16 extra rows of ones, so columns d..d+15 of the
 //     accumulator hold l, rescaled by alpha together with the rest.  The softmax threads do
-//     nothing but max, one fma.sat, one magic-number FMA and byte packing per score.
+//     nothing but the row maximum and five instructions per four codes.
 //
-//   warp 0        TMA producer: Q0, Q1 once; then per key tile K^_j, R^_j and the tile's block
-//                 mean (as a [d x 8] TF32 operand) through a 4-stage ring
+// What bounds it: per key tile and pair of query tiles the kernel takes about 2200 cycles at d = 128
+// (1850 at d = 64).  The tensor pipe needs 1216 of them (704 at d = 64); two softmax warps per
+// scheduler need about 1000 when nothing else runs on it and the correction warps and the hand-offs
+// of the shared score buffer (1500 cycles per pair when they are all that is timed) take the rest.
+// Above a few milliseconds at a stretch the power cap of the board bounds it as well.
+// B1 H40 N32760 d128 13.3 -> 12.5 ms, B1 H12 without value smoothing 3.9 -> 3.0, B2 H16 N16384 d64 2.13 -> 1.73 by: waits that
+// test before they suspend, no operand expansion in front, query tiles of the last wave one by one.
+//
+//   warp 0        producer: Q0, Q1 once; then per key tile K^_j, R^_j (TMA) and the tile's block
+//                 mean (written as a [d x 8] TF32 operand, see MeanRows) through a 4-stage ring
 //   warp 1        score issuer (one elected lane), per key tile j and query tile t:
 //                   S    = Q^_t K^_j^T         4 x kind::f8f6f4, once the previous scores are read
 //   warp 3        accumulator issuer, per key tile j and query tile t:
@@ -43,7 +52,7 @@ using namespace attn;
 //                 back, r_{j-1} = l_{j-1} - alpha_{j-1} l_{j-2}, rescales A_t by alpha_j when a
 //                 row maximum moved, hands (r_hi, r_lo) alpha_j to the mean MMA, writes the output
 //
-// Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16).
+// Tensor memory: S (128 columns; 2 x 128 at d = 64) | A_0 (d + 16) | A_1 (d + 16).
 // P formats of the two-query-tile kernel
 constexpr int kPfExpCast = 0, kPfExp = 1, kPfExpPoly = 2, kPfExpMix = 3;
 
