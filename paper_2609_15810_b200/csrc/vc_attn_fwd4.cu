@@ -16,10 +16,10 @@
 // its log2 is folded into the exponent offset, and every element costs one FMA, one ex2 and
 // half a conversion:  code = E2M1(2^(s cs + log2 2688 - m' - log2 f_g)).  (Moving part of the
 // exponentials to a polynomial on the FMA pipe was measured and is slower: the stage is bound by
-// issue slots and hand-off latency before the special-function unit, which runs at 64 %.)
+// issue slots and hand-off latency as much as of the special-function unit, which runs at 69 %.)
 //
 // HYB = true is the hybrid 4-bit arrangement: the score product stays NVFP4, but P is the
-// ExpCast-FP8 code of Eq. 7 (two FMAs per score, as in the 8-bit kernel) and the value product
+// ExpCast-FP8 code of Eq. 7 (five instructions per four scores, as in the 8-bit kernel) and the value product
 // runs as kind::mxf8f6f4: E4M3 P^ times E2M1 R^ under power-of-two factors per 32 tokens.  The
 // value tile arrives through a 4-bit tensor map that spreads it into the 16-byte containers
 // that instruction kind reads; P^ carries the constant factor 1.
@@ -128,7 +128,8 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   unsigned char* sAm = sP + 2 * kPBytes;                       // [2][128 x 8 fp32] row-sum pairs
   unsigned char* sSfq = sAm + 2 * kAmBytes;                    // [2][KB][512] Q^ factors
   unsigned char* sSfp = sSfq + 2 * 1024;                       // [2][2][512]  P^ factors (HYB: one chunk of ones)
-  unsigned char* sSfOnes = sSfp + 2 * kSfpBytes;               // [512] factors of value rows 128..143
+  unsigned char* sSfOnes = sSfp + 2 * kSfpBytes;               // [512] factors of value rows 128..143, then the table of logarithms
+  float* sLg2 = reinterpret_cast<float*>(sSfOnes + 512);       // [128] log2 of the E4M3 values
   unsigned char* sStage = sSfOnes + 1024;                      // [kStages2]{K, V | ones, Mu, factors}
   FaSmem* sh = reinterpret_cast<FaSmem*>(sStage + kStages2 * kStageBytes);
 
@@ -166,6 +167,8 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
     reinterpret_cast<uint4*>(sStage + (i / (kOnesBytes / 16)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 16)] = make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
   for (int i = tid; i < 128; i += 640)
     reinterpret_cast<uint32_t*>(sSfOnes)[i] = ((i & 3) == 0 && i < 64) ? (HYB ? 0x7f7f7f7fu : 0x38383838u) : 0u;
+  if constexpr (!HYB)                                          // (no lane takes code 127, the NaN)
+    for (int i = tid; i < 128; i += 640) sLg2[i] = i ? lg2_approx(decode_ue4m3(i)) : INFINITY;
   if constexpr (HYB)
     for (int i = tid; i < 128; i += 640) reinterpret_cast<uint32_t*>(sSfp)[i] = 0x7f7f7f7fu;
   pdl_wait();
@@ -338,6 +341,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
     const uint32_t p_row = smem_u32(sP + t * kPBytes + row * kVRow) + ((HYB ? row & 7 : (row >> 1) & 3) << 4);
     const uint32_t sfp_row = smem_u32(sSfp + t * kSfpBytes + (row & 31) * 16 + (row >> 5) * 4);
     const float cs = (a.q_g[bh] * a.k_g[bh]) * a.sl;       // code units -> log2 domain
+    const uint32_t lg2_at = smem_u32(sLg2);
     const uint32_t alpha_at = smem_u32(&sh->alpha[0][row]);
     float m_run = -INFINITY;
     for (int j = 0; j < nb; ++j) {
@@ -355,8 +359,9 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       tc_fence_before();
       mbar_arrive(&sh->s_free[buf(t, j)]);                 // the score buffer may be overwritten
       // (never taken: the end of a basic block here keeps the compiler from moving the maxima in front of
-      // the release of the score buffer, which costs 4 to 14 percent of the kernel)
-      if (a.n_pad < 0) break;
+      // the release of the score buffer, which costs 4 to 14 percent of the hybrid kernel; with NVFP4
+      // probabilities the exponentials hide it, and the larger block is 2.4 percent faster)
+      if (HYB && a.n_pad < 0) break;
       float mx[8];                                        // maxima of the eight 16-key groups
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -401,21 +406,25 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       }
       // p = 2^(s cs - m') * 2688: the row maximum maps to 6 * 448, so the largest factor is 448.
       // Per 16-key group: factor = E4M3(max p / 6); element / factor = 2^(s cs + c0 - log2 factor),
-      // a zero factor zeroes the group.  The eight factor chains run before the wait below: they
-      // do not touch the code tile.
+      // a zero factor (log2: +infinity in the table) zeroes the group.  The logarithm comes from a table
+      // of the 128 codes, filled with what the instruction gives: decoding a code and taking its
+      // logarithm eight times per row and key tile cost 14 percent of the kernel (B1 H12 N32760 d128
+      // 5.25 -> 4.50 ms, B2 H16 N16384 d64 3.37 -> 2.83).  What bounds the stage now is the special-function
+      // unit: 137 results per row and tile keep it busy 69 % of the time.
       const float c0 = 11.39231742277876f - m_new;        // log2(2688) - m'
       uint32_t sfw[2] = {0u, 0u};
       float off[8];
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        const float pmax = ex2_approx(fmaf(mx[g], cs, c0));
-        const uint32_t sb = (uint32_t)__nv_cvt_float_to_fp8(pmax * (1.0f / 6.0f), __NV_SATFINITE, __NV_E4M3);
-        sfw[g >> 2] |= sb << (8 * (g & 3));
-        off[g] = sb ? c0 - lg2_approx(decode_ue4m3(sb)) : -INFINITY;
-      }
       // the previous code tile must have been consumed before it is overwritten
       if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
 
+#pragma unroll
+      for (int g = 0; g < 8; g += 2) {
+        const float p0 = ex2_approx(fmaf(mx[g], cs, c0)), p1 = ex2_approx(fmaf(mx[g + 1], cs, c0));
+        const uint32_t sb = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(p0 * (1.0f / 6.0f), p1 * (1.0f / 6.0f)), __NV_SATFINITE, __NV_E4M3);
+        sfw[g >> 2] |= sb << (8 * (g & 2));
+        off[g] = c0 - lds32(lg2_at + 4 * (sb & 0xffu));
+        off[g + 1] = c0 - lds32(lg2_at + 4 * (sb >> 8));
+      }
       const uint64_t cs2 = pack_f32x2(cs, cs);
       auto quant16 = [&](const uint32_t (&sv)[32], int half, int g) -> uint2 {   // keys 16 g .. 16 g + 15
         float v[16];
