@@ -16,7 +16,7 @@
 // its log2 is folded into the exponent offset, and every element costs one FMA, one ex2 and
 // half a conversion:  code = E2M1(2^(s cs + log2 2688 - m' - log2 f_g)).  (Moving part of the
 // exponentials to a polynomial on the FMA pipe was measured and is slower: the stage is bound by
-// issue slots and hand-off latency as much as of the special-function unit, which runs at 69 %.)
+// issue slots and hand-off latency as much as of the special-function unit, which runs at 72 %.)
 //
 // HYB = true is the hybrid 4-bit arrangement: the score product stays NVFP4, but P is the
 // ExpCast-FP8 code of Eq. 7 (five instructions per four scores, as in the 8-bit kernel) and the value product
@@ -111,7 +111,8 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE;
   constexpr uint32_t SF_COL = 416;
   constexpr uint32_t SFQ_COL = SF_COL, SFK_COL = SF_COL + 16, SFP_COL = SF_COL + 24, SFV_COL = SF_COL + 40;
-  constexpr int kRegCtl = 48, kRegSoftmax = 160, kRegCorr = 56;
+  // (the NVFP4 softmax wants the larger share: B1 H12 N32760 d128 4.44 -> 4.39 ms)
+  constexpr int kRegCtl = 48, kRegSoftmax = HYB ? 160 : 168, kRegCorr = HYB ? 56 : 48;
   static_assert(kRegCtl + 2 * kRegSoftmax + 2 * kRegCorr <= 5 * 96, "register budget exceeds the CTA's allocation");
   constexpr int NVC = HYB ? 1 : 2;                  // value factor chunks per key tile
   constexpr uint32_t kVRow = HYB ? 128 : 64;        // bytes of a value row in shared memory
@@ -410,21 +411,28 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       // of the 128 codes, filled with what the instruction gives: decoding a code and taking its
       // logarithm eight times per row and key tile cost 14 percent of the kernel (B1 H12 N32760 d128
       // 5.25 -> 4.50 ms, B2 H16 N16384 d64 3.37 -> 2.83).  What bounds the stage now is the special-function
-      // unit: 137 results per row and tile keep it busy 69 % of the time.
+      // unit: 137 results per row and tile keep it busy 72 % of the time.
       const float c0 = 11.39231742277876f - m_new;        // log2(2688) - m'
       uint32_t sfw[2] = {0u, 0u};
       float off[8];
-      // the previous code tile must have been consumed before it is overwritten
-      if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
-
-#pragma unroll
-      for (int g = 0; g < 8; g += 2) {
+      auto factors = [&](int g) {                         // of groups g and g + 1
         const float p0 = ex2_approx(fmaf(mx[g], cs, c0)), p1 = ex2_approx(fmaf(mx[g + 1], cs, c0));
         const uint32_t sb = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(p0 * (1.0f / 6.0f), p1 * (1.0f / 6.0f)), __NV_SATFINITE, __NV_E4M3);
         sfw[g >> 2] |= sb << (8 * (g & 2));
         off[g] = c0 - lds32(lg2_at + 4 * (sb & 0xffu));
         off[g + 1] = c0 - lds32(lg2_at + 4 * (sb >> 8));
-      }
+      };
+      // Six factors in front of the wait, two behind it, where they overlap the first exponentials (four and
+      // four at d = 64): B1 H12 N32760 d128 4.33 ms with six, 4.39 with four, 4.47 with none;
+      // B2 H16 N16384 d64 2.83 with six, 2.75 with four, 2.79 with none
+      constexpr int kAhead = D == 128 ? 6 : 4;
+#pragma unroll
+      for (int g = 0; g < kAhead; g += 2) factors(g);
+      // the previous code tile must have been consumed before it is overwritten
+      if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
+
+#pragma unroll
+      for (int g = kAhead; g < 8; g += 2) factors(g);
       const uint64_t cs2 = pack_f32x2(cs, cs);
       auto quant16 = [&](const uint32_t (&sv)[32], int half, int g) -> uint2 {   // keys 16 g .. 16 g + 15
         float v[16];
