@@ -397,13 +397,14 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
         l_resc = l_now * alpha;
         if (SMOOTH) put_pair(r_prev * alpha);              // added after the rescale, so referenced to m_j
       }
+      // Without block means a warp may come here without having waited for the product in front of the last one
+      // on the last one's barrier, and the wait below would take that phase for the last.  The wait for
+      // it stands in front of the last arrival: behind it both phases may be over before this warp looks.
+      const int before = j - (TWO ? 1 : 2);
+      if (!SMOOTH && j == nb - 1 && before >= 0 && !(ok = warp_wait2(&sh->o_done[buf(t, before)], par(before), sh, a.wait, 44))) break;
       mbar_arrive(&sh->pc_full[t][j & 1]);
     }
     // ---- last tile's mean term, then the epilogue: O = s_V * A / l
-    // (Without block means nothing above has waited for the product in front of the last one on that
-    // barrier, and a parity wait would take the phase before it for the last.)
-    const int before = TWO ? nb - 2 : nb - 3;
-    if (!SMOOTH && ok && before >= 0) ok = warp_wait2(&sh->o_done[buf(t, before)], par(before), sh, a.wait, 44);
     if (ok && (ok = warp_wait2(&sh->o_done[buf(t, nb - 1)], par(nb - 1), sh, a.wait, 42))) {
       tc_fence_after();
       l_now = __uint_as_float(tmem_ld1(o_base + L_COL));
