@@ -108,9 +108,9 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   // buffer (and barrier) of scores, codes and products of key tile j, and the parity of its phase
   auto buf = [](int t, int j) { return TWO ? t : j & 1; };
   auto par = [](int j) { return TWO ? j & 1 : (j >> 1) & 1; };
-  // alpha hand-off: tile t's two slots alternate; four slots when there is one tile
-  auto a_slot = [](int t, int j) { return TWO ? 2 * t + (j & 1) : j & 3; };
-  auto a_par = [](int j) { return TWO ? (j >> 1) & 1 : (j >> 2) & 1; };
+  // slot of the hand-offs of alpha and of codes and correction (see FaSmem), and the parity of its phase
+  auto slot = [](int t, int j) { return TWO ? 2 * t + (j & 1) : j & 3; };
+  auto slot_par = [](int j) { return TWO ? (j >> 1) & 1 : (j >> 2) & 1; };
 
   const int early = min(kStages2, nb);      // key tiles whose copies are issued before anything else happens
   if (tid == 0) {
@@ -221,7 +221,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
         const uint64_t dm = smem_desc_kmajor(smem_u32(sStage + stp * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
         for (int t = 0; t < (TWO ? 2 : 1); ++t) {
-          if (!(ok = warp_wait2(&sh->pc_full[t][j & 1], (j >> 1) & 1, sh, a.wait, 23))) break;
+          if (!(ok = warp_wait2(&sh->pc_full[slot(t, j)], slot_par(j), sh, a.wait, 23))) break;
           if (elect_one()) {
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
@@ -311,8 +311,8 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       }
       const float mxa = max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
       const float m_new = fmaxf(m_run, mxa * cs);         // m' = max(m, rowmax S_ij)
-      sts32(alpha_at + 512 * a_slot(t, j), ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
-      mbar_arrive(&sh->a_full[a_slot(t, j)]);
+      sts32(alpha_at + 512 * slot(t, j), ex2_approx(m_run - m_new));      // alpha; 0 on the first tile
+      mbar_arrive(&sh->a_full[slot(t, j)]);
       m_run = m_new;
       // the previous code tile must have been consumed before it is overwritten
       if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
@@ -348,7 +348,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
       store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
-      mbar_arrive(&sh->pc_full[t][j & 1]);
+      mbar_arrive(&sh->pc_full[slot(t, j)]);
     }
   } else if (TWO ? warp >= 12 : warp >= 12 && warp < 16) {
     // -------------------------------------------------------------------- correction warpgroups
@@ -369,8 +369,8 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     };
     for (int j = 0; j < nb; ++j) {
-      if (!(ok = warp_wait2(&sh->a_full[a_slot(t, j)], a_par(j), sh, a.wait, 40))) break;
-      const float alpha = lds32(alpha_at + 512 * a_slot(t, j));
+      if (!(ok = warp_wait2(&sh->a_full[slot(t, j)], slot_par(j), sh, a.wait, 40))) break;
+      const float alpha = lds32(alpha_at + 512 * slot(t, j));
       const bool moved = __any_sync(0xffffffffu, alpha != 1.0f);   // a row maximum of the warp moved
       // (without block means nothing needs l tile by tile: a warp whose maxima stand still passes on)
       if (j > 0 && (SMOOTH || moved)) {
@@ -402,7 +402,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       // it stands in front of the last arrival: behind it both phases may be over before this warp looks.
       const int before = j - (TWO ? 1 : 2);
       if (!SMOOTH && j == nb - 1 && before >= 0 && !(ok = warp_wait2(&sh->o_done[buf(t, before)], par(before), sh, a.wait, 44))) break;
-      mbar_arrive(&sh->pc_full[t][j & 1]);
+      mbar_arrive(&sh->pc_full[slot(t, j)]);
     }
     // ---- last tile's mean term, then the epilogue: O = s_V * A / l
     if (ok && (ok = warp_wait2(&sh->o_done[buf(t, nb - 1)], par(nb - 1), sh, a.wait, 42))) {

@@ -60,9 +60,16 @@ inline uint32_t attn_wait_nonblocking() { return wait_limit_override() ? 1u : 0u
 struct FaSmem {
   uint64_t q_full, kv_full[kStages2], kv_empty[kStages2];
   uint64_t s_full[2], s_free[2], o_done[2], fin_full[2], o_final[2];
-  // alpha and codes+correction hand-offs can run ahead of their consumer, so they alternate between
-  // barriers (a parity wait aliases after two phases) and alpha between slots
-  uint64_t a_full[4], pc_full[2][2];
+  // Hand-offs of alpha (a_full, 128 softmax threads) and of codes and correction (pc_full, 128 softmax and 128
+  // correction threads).  Both can run ahead of their consumer and a parity wait aliases after two phases,
+  // so they take slots in turn: two per query tile, four when there is one tile.  Why that is enough:
+  //   pair of tiles   softmax is at key tile j + 2 only when product j is complete, so every arrival for j is in
+  //                   before anyone can make one for j + 2.
+  //   one tile        softmax is at j + 2 when product j - 1 is complete, and without block means a correction
+  //                   warp whose maxima stand still follows it at once, while another still rescales for j.
+  //                   Softmax at j + 4 has seen product j + 1, hence every arrival for j + 1 and for j.
+  // (With block means every correction warp waits for product j - 1 at j, and two slots would do.)
+  uint64_t a_full[4], pc_full[4];
   uint64_t drain[2];      // exit: "every MMA this issuer warp issued has completed"
   float alpha[4][128];
   uint32_t tmem_base;
@@ -76,7 +83,7 @@ __device__ __forceinline__ void init_barriers(FaSmem* sh, bool two) {
   for (int i = 0; i < 2; ++i) {
     mbar_init(&sh->s_full[i], 1); mbar_init(&sh->s_free[i], 128); mbar_init(&sh->o_done[i], 1);
     mbar_init(&sh->fin_full[i], 128); mbar_init(&sh->o_final[i], 1);
-    for (int b = 0; b < 2; ++b) { mbar_init(&sh->a_full[2 * i + b], 128); mbar_init(&sh->pc_full[i][b], 256); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&sh->a_full[2 * i + b], 128); mbar_init(&sh->pc_full[2 * i + b], 256); }
   }
   mbar_init(&sh->drain[0], 1); mbar_init(&sh->drain[1], 1);
   sh->abort = 0;

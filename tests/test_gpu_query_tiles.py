@@ -49,3 +49,39 @@ def test_calls_without_value_smoothing_are_repeatable(N, grid, d, H, fmt):
     first = _attn(q, k, v, grid, fmt, False)
     for _ in range(5):
         assert torch.equal(_attn(q, k, v, grid, fmt, False), first)
+
+
+@pytest.mark.parametrize("moving", [0, 3])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("fmt", list(FORMATS))
+def test_one_warp_rescales_at_every_key_tile_and_the_others_never(fmt, d, moving):
+    """Scores that grow by about a factor of two per key tile for the 32 rows of one warp and fall for the rows of
+    the others: without block means the others hand over at once while that warp still rescales.  One head alone
+    (one query tile per CTA) against 37 copies of it (296 pairs of tiles: whole waves on 148 SMs), bit for bit.
+    (No order of events can be forced here; tests/test_handoff_order.py goes through all of them.)"""
+    nb = 16
+    N, copies = 128 * nb, 37
+    bits, pf, extra = FORMATS[fmt]
+    g = torch.Generator(device="cuda").manual_seed(d + moving)
+    q, k, v = [torch.randn(1, 1, N, d, generator=g, device="cuda") for _ in range(3)]
+    rows = torch.arange(N, device="cuda")
+    sign = torch.where((rows // 32) % 4 == moving, 1.0, -1.0)
+    q, k = 0.05 * q, 0.05 * k
+    q[..., 0] += 4.0 * sign
+    k[..., 0] += (rows // 128 + 1) * (0.6931 * d ** 0.5 / 4.0)       # log2 of exp(q k / sqrt(d)) moves by one per tile
+    q, k, v = [t.bfloat16() for t in (q, k, v)]
+
+    def attn(heads):
+        p = Params.make(1, heads, N, d, (1, 1, N), bits=bits, p_format=pf, flags=extra)
+        quant, work = alloc_buffers(p)
+        o = torch.empty(1, heads, N, d, dtype=torch.bfloat16, device="cuda")
+        vc.vc_attn(p, *[t.expand(1, heads, N, d).contiguous() for t in (q, k, v)], None, o, quant, work)
+        vc.vc_poll_status(work)
+        return o
+
+    pairs = attn(copies)
+    assert torch.equal(pairs, pairs[:, :1].expand_as(pairs))
+    for _ in range(10):
+        assert torch.equal(attn(1), pairs[:, :1])
+    ref = torch.softmax((q.double() @ k.double().transpose(-1, -2)) / d ** 0.5, dim=-1) @ v.double()
+    assert torch.nn.functional.cosine_similarity(pairs[0, 0].double().flatten(), ref.flatten(), dim=0) > (0.999 if bits == 8 else 0.98)
