@@ -101,7 +101,8 @@ struct GroupSmem {
 };
 
 // Bounded wait of a whole warp (see warp_wait2).  When it gives up, the labels of this run are garbage
-// (but in range) and the status word says so: vc_poll_status on the workspace returns VC_ERR_TIMEOUT.
+// (but in range), its chunks count no tokens, positions that come of it are dropped outside [0, N), and the
+// status word says so: vc_poll_status on the workspace returns VC_ERR_TIMEOUT.
 __device__ __forceinline__ bool gwait(uint64_t* bar, uint32_t parity, GroupSmem* sh, const GroupArgs& a) {
   if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
   if (!a.nonblocking) {
@@ -407,7 +408,9 @@ __global__ void __launch_bounds__(kGThreads, 1) group_assign_kernel(const __grid
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh->sum_free[q & 1]);
-            a.counts[at * kGroupK + wtid] = sh->count[q & 3][wtid];
+            // (a run that has given up reports no tokens: the other warpgroup may be anywhere, and what it adds to
+            // this slot from here on would be counted for a later chunk)
+            a.counts[at * kGroupK + wtid] = ok ? sh->count[q & 3][wtid] : 0;
             sh->count[q & 3][wtid] = 0;
           }
         }
@@ -514,7 +517,9 @@ __global__ void __launch_bounds__(32 * kScatterWarps) group_scatter_kernel(const
     if (valid) basepos = next[warp][lab];
     __syncwarp();
     if (valid) {
-      a.perm[(size_t)bh * a.N + basepos + rank] = t_first + 32 * i + lane;
+      // (after a wait that gave up the counts need not add up; they must not become an address for all that)
+      const int at = basepos + rank;
+      if ((unsigned)at < (unsigned)a.N) a.perm[(size_t)bh * a.N + at] = t_first + 32 * i + lane;
       if (rank == __popc(same) - 1) next[warp][lab] = basepos + rank + 1;     // the last of its group moves the cursor
     }
     __syncwarp();

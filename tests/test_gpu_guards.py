@@ -108,3 +108,30 @@ def test_grouping_wait_that_runs_out_is_reported():
     vc.vc_group(p, v, 16, 2, False, cent, out, gwork)
     vc.vc_poll_status(gwork)
     assert torch.equal(out, good)
+
+
+def test_grouping_that_gives_up_writes_nothing_outside_its_permutation():
+    """Runs of nine chunks per CTA, across heads, with waits that run out: the counts of such a run need not add
+    up, but every position stays inside its head's row of `perm` and every entry inside [0, N)."""
+    B, H, N, d, k, guard = 1, 40, 32760, 128, 64, 1 << 16
+    p = Params.make(B, H, N, d, (21, 30, 52))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    v = torch.randn(B, H, N, d, generator=g, device="cuda").bfloat16()
+    work = torch.empty(vc.vc_group_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    cent = torch.zeros(B, H, k, d, dtype=torch.float32, device="cuda")
+    room = torch.full((2 * guard + B * H * N,), -7, dtype=torch.int32, device="cuda")
+    perm = room[guard:guard + B * H * N].view(B, H, N)
+    try:
+        vc.vc_test_set_wait_limit(1)
+        for _ in range(3):
+            vc.vc_group(p, v, k, 2, False, cent, perm, work)
+            with pytest.raises(vc.VcError) as e:
+                vc.vc_poll_status(work)
+            assert e.value.code == vc.VC_ERR_TIMEOUT
+            assert bool((room[:guard] == -7).all()) and bool((room[guard + B * H * N:] == -7).all())
+            assert bool(((perm == -7) | ((perm >= 0) & (perm < N))).all())
+    finally:
+        vc.vc_test_set_wait_limit(0)
+    vc.vc_group(p, v, k, 2, False, cent, perm, work)
+    vc.vc_poll_status(work)
+    assert torch.equal(perm.sort(dim=-1).values, torch.arange(N, device="cuda", dtype=torch.int32).expand(B, H, N))
