@@ -13,6 +13,8 @@
 // can be processed in groups so that the second read of K and V may hit L2.  All passes are
 // persistent kernels that prefetch the next row blocks with cp.async while they transform
 // the current one.
+#include <climits>
+
 #include "vc_launch.h"
 #include "vc_prep_common.cuh"
 
@@ -1205,7 +1207,7 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
 // Launches.  Passes that do not depend on one another share one: the statistics passes wait on their
 // copies, the Q/K row transform on instruction issue and the shared-memory pipe, so CTAs of both kinds
 // on an SM overlap where either kind alone leaves the other resource idle.  Each pass gets a share of
-// the CTAs (2 per SM) in proportion to what it costs alone.
+// the CTAs (2 per SM) in proportion to what it costs alone, or all take every pass in turn (see share_ctas).
 //   8 bits  1: K column sums | V statistics | Q codes      2: K codes | V codes
 //   4 bits  1: K column sums | Q head maximum | V codes    2: K head maximum | Q codes    3: K codes
 // with the per-head finalization in between.
@@ -1215,56 +1217,121 @@ enum { kPhase1 = 1, kPhase2 = 2, kPhase3 = 3 };
 // (B1 H40 N32760 573 -> 569 us, B1 H12 N32760 190 -> 186 against the ratios measured alone).
 constexpr float kCostRows = 1.0f, kCostAmax = 0.9f, kCostSums = 0.6f, kCostVStats = 0.47f, kCostV8 = 0.66f, kCostV4 = 1.0f;
 
+// Which CTAs take the items of which pass.  CTA first[k] + r (modulo the grid) is number r of the ctas[k] that
+// share pass k's items.
 struct Share {
-  int n0, n1, n2;            // CTAs of the launch's passes, in order of their CTA numbers
-  int i0, i1, i2;            // their items
+  int items[3], first[3], ctas[3];
+  int grid;
   int z0;                    // first tensor of the Q/K quantizing pass (0 = Q, 1 = K)
 };
 
 template <int D, int BITS, int PHASE, bool FAST, int VARIANT>   // VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits)
+__device__ __forceinline__ void one_pass(const int k, const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
+  constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
+  if (BITS == 8 && PHASE == kPhase1) {
+    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
+    else if (k == 1) kcolsum_pass<D>(a, smem, sl, nh);
+    else v_pass<D, kVStats>(a, smem, sl, nh);
+  } else if (BITS == 8) {
+    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, z0);
+    else v_pass<D, kVQuant8>(a, smem, sl, nh);
+  } else if (PHASE == kPhase1) {
+    if (k == 0) qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 0);
+    else if (k == 1) kcolsum_pass<D>(a, smem, sl, nh);
+    else v_pass<D, VARIANT ? kVQuant4M : kVQuant4>(a, smem, sl, nh);
+  } else if (PHASE == kPhase2) {
+    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
+    else qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 1);
+  } else {
+    qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 1);
+  }
+}
+
+// TURNS = false: a CTA belongs to one pass.  TURNS = true: every CTA takes its part of every pass, one pass after
+// the other; the second half of the CTAs starts with the second pass, so that kinds still meet on an SM.
+template <int D, int BITS, int PHASE, bool FAST, int VARIANT, bool TURNS>
 __global__ void __launch_bounds__(kThreads, 2) prep_kernel(const PrepArgs a, const Share s, int nh) {
   extern __shared__ __align__(128) unsigned char smem[];
   // (No early pdl_allow: attention CTAs that start one by one as this kernel's leave do not run through a
   // head's key tiles together, and the hybrid attention takes 3.5 percent longer at B1 H40 N32760, 3.6 at
   // B1 H12 N32760.  The next kernel starts when the last CTA has ended.)
-  constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
+  constexpr int kPasses = PHASE == kPhase3 ? 1 : (PHASE == kPhase1 ? 3 : 2);
   const int b = blockIdx.x;
-  if (BITS == 8 && PHASE == kPhase1) {
-    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
-    else if (b < s.n0 + s.n1) kcolsum_pass<D>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
-    else v_pass<D, kVStats>(a, smem, Slot{b - s.n0 - s.n1, s.n2, s.i2}, nh);
-  } else if (BITS == 8) {
-    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, s.z0);
-    else v_pass<D, kVQuant8>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
-  } else if (PHASE == kPhase1) {
-    if (b < s.n0) qk_pass<D, kStageAmax, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
-    else if (b < s.n0 + s.n1) kcolsum_pass<D>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh);
-    else v_pass<D, VARIANT ? kVQuant4M : kVQuant4>(a, smem, Slot{b - s.n0 - s.n1, s.n2, s.i2}, nh);
-  } else if (PHASE == kPhase2) {
-    if (b < s.n0) qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 0);
-    else qk_pass<D, kStageAmax, FAST>(a, smem, Slot{b - s.n0, s.n1, s.i1}, nh, 1);
+  if constexpr (!TURNS) {
+    const int behind0 = b - s.ctas[0], behind1 = behind0 - s.ctas[1];
+    if (kPasses == 1 || behind0 < 0) one_pass<D, BITS, PHASE, FAST, VARIANT>(0, a, smem, Slot{b, s.ctas[0], s.items[0]}, nh, s.z0);
+    else if (kPasses == 2 || behind1 < 0) one_pass<D, BITS, PHASE, FAST, VARIANT>(1, a, smem, Slot{behind0, s.ctas[1], s.items[1]}, nh, s.z0);
+    else one_pass<D, BITS, PHASE, FAST, VARIANT>(2, a, smem, Slot{behind1, s.ctas[2], s.items[2]}, nh, s.z0);
   } else {
-    qk_pass<D, kQuant, FAST>(a, smem, Slot{b, s.n0, s.i0}, nh, 1);
+    int k = 2 * b >= s.grid ? 1 : 0;
+    bool again = false;
+#pragma unroll 1
+    for (int turn = 0; turn < kPasses; ++turn, k = k + 1 < kPasses ? k + 1 : 0) {
+      const int items = k == 0 ? s.items[0] : (k == 1 ? s.items[1] : s.items[2]);
+      const int first = k == 0 ? s.first[0] : (k == 1 ? s.first[1] : s.first[2]);
+      const int ctas = k == 0 ? s.ctas[0] : (k == 1 ? s.ctas[1] : s.ctas[2]);
+      const int rank = b >= first ? b - first : b - first + s.grid;
+      if (rank >= ctas) continue;
+      if (again) { cp_async_wait<0>(); __syncthreads(); }       // the stages are the next pass's
+      again = true;
+      one_pass<D, BITS, PHASE, FAST, VARIANT>(k, a, smem, Slot{rank, ctas, items}, nh, s.z0);
+    }
   }
 }
 
-// CTAs of each pass: all of them while they fit two per SM, else in proportion to items x cost.
-inline Share share_ctas(int i0, float c0, int i1, float c1, int i2, float c2, int z0) {
-  Share s{i0, i1, i2, i0, i1, i2, z0};
-  const int total = 2 * sm_count();
-  if (i0 + i1 + i2 <= total) return s;
-  const float w0 = i0 * c0, w1 = i1 * c1, w2 = i2 * c2, w = w0 + w1 + w2;
-  auto part = [&](float x, int items) { return items == 0 ? 0 : (int)(x / w * total) < 1 ? 1 : (int)(x / w * total) > items ? items : (int)(x / w * total); };
-  s.n1 = part(w1, i1);
-  s.n2 = part(w2, i2);
-  s.n0 = total - s.n1 - s.n2 < i0 ? total - s.n1 - s.n2 : i0;
+// Shared memory that lets two CTAs of a launch stay on an SM.
+constexpr size_t kHalfSm = 113 * 1024;
+
+// Shares of a launch on `per_sm` CTAs per SM.  While they fit, every item has a CTA.  Up to turns_from items per
+// CTA each pass gets CTAs in proportion to items x cost.  Beyond that every CTA takes its part of every pass: the
+// costs hold for one head dimension, one set of passes and one locality of the gather, and a pass whose
+// CTAs have too much keeps the launch waiting.  A CTA pays for it with one more filling of its pipeline
+// per pass, some 3 us.  Measured at 8 bits, d128 (the costs' own case): B1 H24 N32760 in shares 333 us, in
+// turns 339; H32 442 and 436; H40 550 and 540; H24 N118800 1246 and 1159 (a launch per pass: 1206).  Elsewhere
+// turns win from 16 items per CTA on: d64 B1 H8 N32760 80 and 74 us, H12 N327680 1143 and 971 (a
+// launch per pass: 1067); 4 bits d64 H40 N32760 524 and 459 (488); supplied statistics, d128, H24 N118800
+// 1020 and 859 (863); without K smoothing H40 N32760 483 and 452 (474).
+struct Work {
+  int items;
+  float cost;
+};
+inline Share share_ctas(const Work w0, const Work w1, const Work w2, int z0, int per_sm, int turns_from, bool* turns) {
+  const Work w[3] = {w0, w1, w2};
+  const int64_t most = (int64_t)per_sm * sm_count(), items = (int64_t)w0.items + w1.items + w2.items;
+  Share s{};
+  s.z0 = z0;
+  for (int k = 0; k < 3; ++k) s.items[k] = s.ctas[k] = w[k].items;
+  *turns = items > most * (int64_t)turns_from && w0.items != items && w1.items != items && w2.items != items;
+  if (*turns) {
+    int64_t at = 0;
+    for (int k = 0; k < 3; ++k) {
+      s.first[k] = (int)(at % most);          // item i of the launch belongs to CTA i % grid
+      s.ctas[k] = w[k].items < most ? w[k].items : (int)most;
+      at += w[k].items;
+    }
+    s.grid = (int)most;
+    return s;
+  }
+  if (items > most) {
+    const float all = w0.items * w0.cost + w1.items * w1.cost + w2.items * w2.cost;
+    int left = (int)most;
+    for (int k = 2; k >= 0; --k) {
+      if (w[k].items == 0) continue;
+      const int part = k == 0 ? left : (int)(w[k].items * w[k].cost / all * (float)most);
+      s.ctas[k] = part < 1 ? 1 : part < w[k].items ? part : w[k].items;
+      left -= s.ctas[k];
+    }
+  }
+  s.first[1] = s.ctas[0];
+  s.first[2] = s.ctas[0] + s.ctas[1];
+  s.grid = s.first[2] + s.ctas[2];
   return s;
 }
 
 template <auto KERNEL>
 cudaError_t launch_phase(const PrepArgs& a, const Share& sh, int nh, size_t smem, cudaStream_t s) {
   cudaError_t e = allow_smem<KERNEL>();
-  if (e == cudaSuccess) e = launch_overlapped(KERNEL, dim3((unsigned)(sh.n0 + sh.n1 + sh.n2)), kThreads, smem, s, a, sh, nh);
+  if (e == cudaSuccess) e = launch_overlapped(KERNEL, dim3((unsigned)sh.grid), kThreads, smem, s, a, sh, nh);
   count_launches(1);
   return e;
 }
@@ -1277,6 +1344,9 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
   const size_t v_smem = 3 * (size_t)kBlock * 2 * D + 16 * D * 4 + 2 * kBlock * 4;
   const size_t smem = row_smem > v_smem ? row_smem : v_smem;
   static_assert(2 * kThreads * (D / 16) * 16 + 8 * D * 4 <= 2 * Geo<D>::stage_bytes + kBlock * D, "the column sums fit the row pass's share");
+  const bool ext = a.ext_k_mean != nullptr;     // the caller supplied the statistics: no statistics passes
+  const bool tuned = D == 128 && BITS == 8 && !ext && (a.flags & VC_FLAG_K_SMOOTH);
+  const int turns_from = smem > kHalfSm ? INT_MAX : tuned ? 80 : 16;      // (kinds do not meet on an SM that holds one CTA)
   cudaError_t e = cudaSuccess;
   int group = pr.heads_per_pass > 0 ? pr.heads_per_pass : pr.BH;
   if (group > 32768) group = 32768;
@@ -1284,24 +1354,35 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     const int nh = pr.BH - bh0 < group ? pr.BH - bh0 : group;
     const int per = pr.nb * nh;
     a.bh0 = bh0;
-    const bool ext = a.ext_k_mean != nullptr;     // the caller supplied the statistics: no statistics passes
     const int sums = a.flags & VC_FLAG_K_SMOOTH ? per : 0;
     auto finalize = [&](int which, int threads) {
       if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
       count_launches(1);
     };
+    auto phase = [&](auto whole, auto in_turns, Work w0, Work w1, Work w2, int z0) {
+      bool turns;
+      const Share sh = share_ctas(w0, w1, w2, z0, 2, turns_from, &turns);
+      if (e == cudaSuccess) e = turns ? in_turns(a, sh, nh, smem, s) : whole(a, sh, nh, smem, s);
+    };
+    const Work none{0, 0.f};
     if constexpr (BITS == 8) {
-      if (!ext) e = launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT>>(a, share_ctas(per, kCostRows, sums, kCostSums, per, kCostVStats, 0), nh, smem, s);
-      if (!ext) finalize(0, 8 * D);
+      if (!ext) {
+        phase(launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, true>>,
+              Work{per, kCostRows}, Work{sums, kCostSums}, Work{per, kCostVStats}, 0);
+        finalize(0, 8 * D);
+      }
       // (with supplied statistics Q has no launch of its own to share)
-      const Share sh = ext ? share_ctas(2 * per, kCostRows, per, kCostV8, 0, 0.f, 0) : share_ctas(per, kCostRows, per, kCostV8, 0, 0.f, 1);
-      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT>>(a, sh, nh, smem, s);
+      phase(launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>,
+            Work{ext ? 2 * per : per, kCostRows}, Work{per, kCostV8}, none, ext ? 0 : 1);
     } else {
-      e = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT>>(a, share_ctas(per, kCostAmax, sums, kCostSums, per, kCostV4, 0), nh, smem, s);
+      phase(launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, true>>,
+            Work{per, kCostAmax}, Work{sums, kCostSums}, Work{per, kCostV4}, 0);
       finalize(0, 8 * D);
-      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0>>(a, share_ctas(per, kCostRows, per, kCostAmax, 0, 0.f, 0), nh, smem, s);
+      phase(launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, false>>, launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, true>>,
+            Work{per, kCostRows}, Work{per, kCostAmax}, none, 0);
       finalize(1, 32);
-      if (e == cudaSuccess) e = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0>>(a, share_ctas(per, kCostRows, 0, 0.f, 0, 0.f, 1), nh, smem, s);
+      phase(launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>, launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>,
+            Work{per, kCostRows}, none, none, 1);
     }
   }
   return e != cudaSuccess ? e : cudaGetLastError();
