@@ -1210,6 +1210,7 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
 // the CTAs (2 per SM) in proportion to what it costs alone, or all take every pass in turn (see share_ctas).
 //   8 bits  1: K column sums | V statistics | Q codes      2: K codes | V codes
 //   4 bits  1: K column sums | Q head maximum | V codes    2: K head maximum | Q codes    3: K codes
+// (On a wide grid the passes over rows leave the launches they share with the others, see run_phases.)
 // with the per-head finalization in between.
 enum { kPhase1 = 1, kPhase2 = 2, kPhase3 = 3 };
 
@@ -1217,34 +1218,26 @@ enum { kPhase1 = 1, kPhase2 = 2, kPhase3 = 3 };
 // (B1 H40 N32760 573 -> 569 us, B1 H12 N32760 190 -> 186 against the ratios measured alone).
 constexpr float kCostRows = 1.0f, kCostAmax = 0.9f, kCostSums = 0.6f, kCostVStats = 0.47f, kCostV8 = 0.66f, kCostV4 = 1.0f;
 
-// Which CTAs take the items of which pass.  CTA first[k] + r (modulo the grid) is number r of the ctas[k] that
-// share pass k's items.
+// Which CTAs take the items of which pass: ctas[k] CTAs share pass k's items, in shares one pass's CTAs behind
+// the other's, in turns from CTA first[k] on (modulo the grid).
 struct Share {
   int items[3], first[3], ctas[3];
   int grid;
   int z0;                    // first tensor of the Q/K quantizing pass (0 = Q, 1 = K)
 };
 
-template <int D, int BITS, int PHASE, bool FAST, int VARIANT>   // VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits)
-__device__ __forceinline__ void one_pass(const int k, const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
+// Pass PASS of a launch.  VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits).
+template <int D, int BITS, int PHASE, bool FAST, int VARIANT, int PASS>
+__device__ __forceinline__ void one_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
   constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
-  if (BITS == 8 && PHASE == kPhase1) {
-    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
-    else if (k == 1) kcolsum_pass<D>(a, smem, sl, nh);
-    else v_pass<D, kVStats>(a, smem, sl, nh);
-  } else if (BITS == 8) {
-    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, z0);
-    else v_pass<D, kVQuant8>(a, smem, sl, nh);
-  } else if (PHASE == kPhase1) {
-    if (k == 0) qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 0);
-    else if (k == 1) kcolsum_pass<D>(a, smem, sl, nh);
-    else v_pass<D, VARIANT ? kVQuant4M : kVQuant4>(a, smem, sl, nh);
-  } else if (PHASE == kPhase2) {
-    if (k == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
-    else qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 1);
-  } else {
-    qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 1);
-  }
+  if constexpr (PHASE == kPhase1 && PASS == 0) qk_pass<D, BITS == 8 ? kQuant : kStageAmax, FAST>(a, smem, sl, nh, 0);
+  else if constexpr (PHASE == kPhase1 && PASS == 1) kcolsum_pass<D>(a, smem, sl, nh);
+  else if constexpr (PHASE == kPhase1) v_pass<D, BITS == 8 ? kVStats : (VARIANT ? kVQuant4M : kVQuant4)>(a, smem, sl, nh);
+  else if constexpr (BITS == 8 && PASS == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, z0);
+  else if constexpr (BITS == 8) v_pass<D, kVQuant8>(a, smem, sl, nh);
+  else if constexpr (PHASE == kPhase2 && PASS == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
+  else if constexpr (PHASE == kPhase2) qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 1);
+  else qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 1);
 }
 
 // TURNS = false: a CTA belongs to one pass.  TURNS = true: every CTA takes its part of every pass, one pass after
@@ -1258,10 +1251,10 @@ __global__ void __launch_bounds__(kThreads, 2) prep_kernel(const PrepArgs a, con
   constexpr int kPasses = PHASE == kPhase3 ? 1 : (PHASE == kPhase1 ? 3 : 2);
   const int b = blockIdx.x;
   if constexpr (!TURNS) {
-    const int behind0 = b - s.ctas[0], behind1 = behind0 - s.ctas[1];
-    if (kPasses == 1 || behind0 < 0) one_pass<D, BITS, PHASE, FAST, VARIANT>(0, a, smem, Slot{b, s.ctas[0], s.items[0]}, nh, s.z0);
-    else if (kPasses == 2 || behind1 < 0) one_pass<D, BITS, PHASE, FAST, VARIANT>(1, a, smem, Slot{behind0, s.ctas[1], s.items[1]}, nh, s.z0);
-    else one_pass<D, BITS, PHASE, FAST, VARIANT>(2, a, smem, Slot{behind1, s.ctas[2], s.items[2]}, nh, s.z0);
+    const int n0 = s.ctas[0], n1 = s.ctas[1];
+    if (kPasses == 1 || b < n0) one_pass<D, BITS, PHASE, FAST, VARIANT, 0>(a, smem, Slot{b, n0, s.items[0]}, nh, s.z0);
+    else if (kPasses == 2 || b < n0 + n1) one_pass<D, BITS, PHASE, FAST, VARIANT, 1>(a, smem, Slot{b - n0, n1, s.items[1]}, nh, s.z0);
+    else one_pass<D, BITS, PHASE, FAST, VARIANT, 2>(a, smem, Slot{b - n0 - n1, s.ctas[2], s.items[2]}, nh, s.z0);
   } else {
     int k = 2 * b >= s.grid ? 1 : 0;
     bool again = false;
@@ -1274,7 +1267,10 @@ __global__ void __launch_bounds__(kThreads, 2) prep_kernel(const PrepArgs a, con
       if (rank >= ctas) continue;
       if (again) { cp_async_wait<0>(); __syncthreads(); }       // the stages are the next pass's
       again = true;
-      one_pass<D, BITS, PHASE, FAST, VARIANT>(k, a, smem, Slot{rank, ctas, items}, nh, s.z0);
+      const Slot sl{rank, ctas, items};
+      if (k == 0) one_pass<D, BITS, PHASE, FAST, VARIANT, 0>(a, smem, sl, nh, s.z0);
+      else if (kPasses == 2 || k == 1) one_pass<D, BITS, PHASE, FAST, VARIANT, 1>(a, smem, sl, nh, s.z0);
+      else one_pass<D, BITS, PHASE, FAST, VARIANT, 2>(a, smem, sl, nh, s.z0);
     }
   }
 }
@@ -1322,9 +1318,7 @@ inline Share share_ctas(const Work w0, const Work w1, const Work w2, int z0, int
       left -= s.ctas[k];
     }
   }
-  s.first[1] = s.ctas[0];
-  s.first[2] = s.ctas[0] + s.ctas[1];
-  s.grid = s.first[2] + s.ctas[2];
+  s.grid = s.ctas[0] + s.ctas[1] + s.ctas[2];
   return s;
 }
 
@@ -1342,11 +1336,17 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
   const size_t rope_bytes = ((a.flags & VC_FLAG_ROPE) && a.rope_in_smem) ? (size_t)a.rd.entries * 8 : 0;
   const size_t row_smem = 2 * (size_t)Geo<D>::stage_bytes + (size_t)kBlock * D + 3 * kBlock * 4 + 64 + D * 4 + rope_bytes;
   const size_t v_smem = 3 * (size_t)kBlock * 2 * D + 16 * D * 4 + 2 * kBlock * 4;
-  const size_t smem = row_smem > v_smem ? row_smem : v_smem;
+  const size_t sum_smem = 2 * (size_t)kThreads * (D / 16) * 16 + 8 * D * 4 + rope_bytes;
+  const size_t smem = row_smem > v_smem ? row_smem : v_smem, rest_smem = sum_smem > v_smem ? sum_smem : v_smem;
   static_assert(2 * kThreads * (D / 16) * 16 + 8 * D * 4 <= 2 * Geo<D>::stage_bytes + kBlock * D, "the column sums fit the row pass's share");
   const bool ext = a.ext_k_mean != nullptr;     // the caller supplied the statistics: no statistics passes
   const bool tuned = D == 128 && BITS == 8 && !ext && (a.flags & VC_FLAG_K_SMOOTH);
-  const int turns_from = smem > kHalfSm ? INT_MAX : tuned ? 80 : 16;      // (kinds do not meet on an SM that holds one CTA)
+  const int turns_from = tuned ? 80 : 16;
+  // A grid with long axes has a table that leaves an SM room for one CTA of the row pass (at d128 from 27.6 KB on,
+  // 3448 entries).  The rows then get launches of their own, so that the passes that need less do not come
+  // down to one CTA per SM too.  8 bits, d128: 21 x 68 x 120 H3 332 -> 283 us, 1 x 128 x 128 H39 394 -> 337,
+  // 33 x 90 x 160 H1 335 -> 318 (all passes in launches of their own: 321, 363, 347).
+  const bool wide = smem > kHalfSm;
   cudaError_t e = cudaSuccess;
   int group = pr.heads_per_pass > 0 ? pr.heads_per_pass : pr.BH;
   if (group > 32768) group = 32768;
@@ -1359,30 +1359,34 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
       if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
       count_launches(1);
     };
-    auto phase = [&](auto whole, auto in_turns, Work w0, Work w1, Work w2, int z0) {
-      bool turns;
-      const Share sh = share_ctas(w0, w1, w2, z0, 2, turns_from, &turns);
-      if (e == cudaSuccess) e = turns ? in_turns(a, sh, nh, smem, s) : whole(a, sh, nh, smem, s);
+    auto launch = [&](auto whole, auto in_turns, size_t bytes, Work w0, Work w1, Work w2, int z0) {
+      bool turns;                                // (kinds do not meet on an SM that holds one CTA: no turns)
+      const Share sh = bytes > kHalfSm ? share_ctas(w0, w1, w2, z0, 1, INT_MAX, &turns) : share_ctas(w0, w1, w2, z0, 2, turns_from, &turns);
+      if (e == cudaSuccess) e = turns ? in_turns(a, sh, nh, bytes, s) : whole(a, sh, nh, bytes, s);
     };
-    const Work none{0, 0.f};
+    const Work none{0, 0.f}, rows{per, kCostRows}, amax{per, kCostAmax}, k_sums{sums, kCostSums}, v_stats{per, kCostVStats}, v_codes{per, kCostV8},
+        v_codes4{per, kCostV4};
     if constexpr (BITS == 8) {
+      const auto first = launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, false>>, first_turns = launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, true>>,
+                 second = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, second_turns = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>;
       if (!ext) {
-        phase(launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 8, kPhase1, FAST, VARIANT, true>>,
-              Work{per, kCostRows}, Work{sums, kCostSums}, Work{per, kCostVStats}, 0);
+        launch(first, first_turns, wide ? rest_smem : smem, wide ? none : rows, k_sums, v_stats, 0);
         finalize(0, 8 * D);
       }
-      // (with supplied statistics Q has no launch of its own to share)
-      phase(launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>,
-            Work{ext ? 2 * per : per, kCostRows}, Work{per, kCostV8}, none, ext ? 0 : 1);
+      // (with supplied statistics there is no first launch for Q to share; on a wide grid it does not share one)
+      const bool q_too = ext || wide;
+      launch(second, second_turns, wide ? row_smem : smem, Work{q_too ? 2 * per : per, kCostRows}, wide ? none : v_codes, none, q_too ? 0 : 1);
+      if (wide) launch(second, second_turns, v_smem, none, v_codes, none, 0);
     } else {
-      phase(launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, false>>, launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, true>>,
-            Work{per, kCostAmax}, Work{sums, kCostSums}, Work{per, kCostV4}, 0);
+      const auto first = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, false>>, first_turns = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, true>>,
+                 second = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, false>>, second_turns = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, true>>,
+                 third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>;
+      launch(first, first_turns, wide ? rest_smem : smem, wide ? none : amax, k_sums, v_codes4, 0);
+      if (wide) launch(first, first_turns, row_smem, amax, none, none, 0);
       finalize(0, 8 * D);
-      phase(launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, false>>, launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, true>>,
-            Work{per, kCostRows}, Work{per, kCostAmax}, none, 0);
+      launch(second, second_turns, smem, rows, amax, none, 0);
       finalize(1, 32);
-      phase(launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>, launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>,
-            Work{per, kCostRows}, none, none, 1);
+      launch(third, third, smem, rows, none, none, 1);
     }
   }
   return e != cudaSuccess ? e : cudaGetLastError();
