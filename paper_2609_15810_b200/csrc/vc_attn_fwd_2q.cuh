@@ -108,9 +108,12 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   // buffer (and barrier) of scores, codes and products of key tile j, and the parity of its phase
   auto buf = [](int t, int j) { return TWO ? t : j & 1; };
   auto par = [](int j) { return TWO ? j & 1 : (j >> 1) & 1; };
-  // slot of the hand-offs of alpha and of codes and correction (see FaSmem), and the parity of its phase
+  // slot of the hand-off of alpha (see FaSmem) and the parity of its phase, and the same for codes and correction
+  // (with block means two slots do there: B1 H8 N2048 d128, INT8 scores, 40.2 us instead of 40.6 with four)
   auto slot = [](int t, int j) { return TWO ? 2 * t + (j & 1) : j & 3; };
   auto slot_par = [](int j) { return TWO ? (j >> 1) & 1 : (j >> 2) & 1; };
+  auto pc_slot = [](int t, int j) { return TWO || SMOOTH ? 2 * t + (j & 1) : j & 3; };
+  auto pc_par = [](int j) { return TWO || SMOOTH ? (j >> 1) & 1 : (j >> 2) & 1; };
 
   const int early = min(kStages2, nb);      // key tiles whose copies are issued before anything else happens
   if (tid == 0) {
@@ -221,7 +224,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
         const uint64_t dm = smem_desc_kmajor(smem_u32(sStage + stp * kStageBytes + kKBytes + kVBytes + kOnesBytes), 32);
 #pragma unroll
         for (int t = 0; t < (TWO ? 2 : 1); ++t) {
-          if (!(ok = warp_wait2(&sh->pc_full[slot(t, j)], slot_par(j), sh, a.wait, 23))) break;
+          if (!(ok = warp_wait2(&sh->pc_full[pc_slot(t, j)], pc_par(j), sh, a.wait, 23))) break;
           if (elect_one()) {
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
@@ -348,7 +351,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
       store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
-      mbar_arrive(&sh->pc_full[slot(t, j)]);
+      mbar_arrive(&sh->pc_full[pc_slot(t, j)]);
     }
   } else if (TWO ? warp >= 12 : warp >= 12 && warp < 16) {
     // -------------------------------------------------------------------- correction warpgroups
@@ -402,7 +405,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       // it stands in front of the last arrival: behind it both phases may be over before this warp looks.
       const int before = j - (TWO ? 1 : 2);
       if (!SMOOTH && j == nb - 1 && before >= 0 && !(ok = warp_wait2(&sh->o_done[buf(t, before)], par(before), sh, a.wait, 44))) break;
-      mbar_arrive(&sh->pc_full[slot(t, j)]);
+      mbar_arrive(&sh->pc_full[pc_slot(t, j)]);
     }
     // ---- last tile's mean term, then the epilogue: O = s_V * A / l
     if (ok && (ok = warp_wait2(&sh->o_done[buf(t, nb - 1)], par(nb - 1), sh, a.wait, 42))) {
