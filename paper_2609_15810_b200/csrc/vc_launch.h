@@ -1,5 +1,5 @@
 // Kernel launches that may overlap the end of the kernel in front of them (programmatic dependent
-// launch), and shared-memory limits raised once per kernel and device.
+// launch), and shared-memory limits raised once per kernel and context.
 //
 // Every kernel launched this way calls pdl_wait() before it touches anything an earlier kernel on
 // the stream wrote or still reads: the call returns when the kernel in front has completed and its writes
@@ -8,6 +8,7 @@
 // are simply waited for.  What is gained is the gap between two kernels (about 1.5 us) and the
 // successor's prologue.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -30,18 +31,30 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int thread
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-// Lets KERNEL use up to the whole SM's shared memory.  One driver call per kernel and device for the
-// life of the process (it used to be one per kernel and call).
+// A number for the current context that no other context of the process gets, 0 if there is none yet.
+inline uint64_t context_number() {
+  typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+  static const GetId get = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<GetId>(p) : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get && get(nullptr, &id) == CUDA_SUCCESS ? id + 1 : 0;
+}
+
+// Lets KERNEL use up to the whole SM's shared memory.  The limit belongs to the context (a second context of
+// the device, or the one behind cudaDeviceReset, starts without it): one driver call per kernel and context,
+// and one more whenever more than 64 contexts share a slot.
 template <auto KERNEL>
 inline cudaError_t allow_smem() {
-  static std::atomic<uint64_t> done{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
-  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  static std::atomic<uint64_t> done[64];
+  const uint64_t ctx = context_number();
+  std::atomic<uint64_t>& slot = done[ctx % 64];
+  if (ctx && slot.load(std::memory_order_acquire) == ctx) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e == cudaSuccess) slot.store(ctx, std::memory_order_release);
   return e;
 }
 
