@@ -1,12 +1,18 @@
 // Kernel launches that may overlap the end of the kernel in front of them (programmatic dependent
 // launch), and shared-memory limits raised once per kernel and context.
 //
-// Every kernel launched this way calls pdl_wait() before it touches anything an earlier kernel on
-// the stream wrote or still reads: the call returns when the kernel in front has completed and its writes
-// are visible.  Because each of them waits, and allows its successor only behind its own wait, whatever
-// happened before the kernel in front is complete as well; a caller's own kernels, which allow nothing,
-// are simply waited for.  What is gained is the gap between two kernels (about 1.5 us) and the
-// successor's prologue.
+// What makes it sound:
+//   - Every kernel launched this way calls pdl_wait() in front of whatever the kernel before it on the stream may
+//     write or still read: the call returns when that kernel has completed and its writes are visible.
+//   - A kernel allows its successor (pdl_allow) only behind its own wait.  So when a kernel starts, everything
+//     in front of the kernel before it is complete, and a caller's own kernels, which allow nothing, are
+//     simply waited for.  (One exception: the assignment of vc_group allows early.  Its successor, the update,
+//     waits before it does anything.)
+//   - Therefore a kernel may read, in front of its wait, what the kernel before it neither writes nor makes
+//     late: the preprocessing passes read Q, K, V and the permutation, the assignment of vc_group reads V.  The
+//     kernels before them (table, permutation check, passes, finalize; init, update) write none of these.  Another
+//     kernel put in between has to keep to that, and has to wait before it allows.
+// What is gained is the gap between two kernels (about 1.5 us) and the successor's prologue.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
