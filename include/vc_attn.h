@@ -185,7 +185,8 @@ vc_status vc_prep_stats_view(const vc_params *p, const void *quant, const void *
 /* Quantized attention forward (Eq. 1, Eq. 6, Eq. 7) from a bundle in vc_prep's layout.
  * o: [B][H][N][d] bf16.  workspace as above.  `p` must describe the bundle: the same shape,
  * bits, p_format (it selects the value format at 4 bits) and flags as the vc_prep call that
- * wrote it, and `quant` must hold vc_quant_bytes(p) bytes; a mismatch is not detected. */
+ * wrote it, and `quant` must hold vc_quant_bytes(p) bytes; a mismatch is not detected.  (Without
+ * VC_FLAG_V_SMOOTH every block mean is zero by that rule, and the bundle's means need not be read.) */
 vc_status vc_attn_fwd(const vc_params *p, const void *quant, void *o, void *workspace,
                       void *stream);
 
@@ -265,7 +266,10 @@ int32_t vc_group_schedule(int32_t step, int32_t n_steps, int32_t reuse);
  *     without ordering between their streams) race on the array: serialize them.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current; make that first call outside any
- *     stream capture.  Later calls only launch kernels on `stream`.
+ *     stream capture.  Later calls launch kernels on `stream`; a configuration (d, bits, format,
+ *     stages) that is used for the first time in a context also raises its kernels' shared-memory
+ *     limit (a host-side call that allocates nothing), and a call with VC_FLAG_CHECK_PERM and a
+ *     permutation issues one memset on `stream`.
  * It calls no cudaMalloc / cudaFree and no allocating library routine.  The output is
  * the same bundle vc_prep writes. */
 #define VC_NOALLOC_SCRATCH_BYTES (4u << 20)

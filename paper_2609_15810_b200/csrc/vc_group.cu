@@ -82,10 +82,10 @@ __global__ void group_init_kernel(const GroupArgs a, int warm) {
 //               memory, argmin, label, one-hot entry; the warpgroup that had a chunk's last tile
 //               writes the chunk's sums and counts out
 // Tensor memory: two score buffers of 64 columns | two cluster-sum buffers (d columns, rows = clusters).
-// What bounds it: the tensor pipe, 2200 cycles per tile (24 score products, each as long as its A operand takes to
-// read however few the centroids, and 8 sum products), then the values
-// read once.  At B1 H40 N32760 d128: 190 us with a CTA per chunk, one label warpgroup and serial minima,
-// 125 us now (the products alone: 24 x 64 + 8 x 80 cycles per tile = 77 us; the values at the copy rate: 51 us).
+// What bounds it: at B1 H40 N32760 d128 it takes 125 us, about 3550 cycles per tile (190 us with a CTA per chunk, one
+// label warpgroup and serial minima).  2176 of them are the products: 24 for the scores, 64 cycles each, as long as
+// the A operand takes to read however few the centroids, and 8 of 80 for the sums; alone they would take 77 us.  Where
+// the rest goes (hand-offs, chunk ends, a head's set-up) has not been measured.  The values at the copy rate: 51 us.
 constexpr int kGStages = 4;
 constexpr int kGThreads = 320;
 constexpr uint32_t kGroupWaitLimit = 1u << 22;   // default number of polls of a wait
