@@ -16,7 +16,7 @@
 // its log2 is folded into the exponent offset, and every element costs one FMA, one ex2 and
 // half a conversion:  code = E2M1(2^(s cs + log2 2688 - m' - log2 f_g)).  (Moving part of the
 // exponentials to a polynomial on the FMA pipe was measured and is slower: the stage is bound by
-// issue slots and hand-off latency as much as of the special-function unit, which runs at 72 %.)
+// issue slots and hand-off latency as much as of the special-function unit, which runs at 75 %.)
 //
 // HYB = true is the hybrid 4-bit arrangement: the score product stays NVFP4, but P is the
 // ExpCast-FP8 code of Eq. 7 (five instructions per four scores, as in the 8-bit kernel) and the value product
@@ -411,7 +411,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
       // of the 128 codes, filled with what the instruction gives: decoding a code and taking its
       // logarithm eight times per row and key tile cost 14 percent of the kernel (B1 H12 N32760 d128
       // 5.25 -> 4.50 ms, B2 H16 N16384 d64 3.37 -> 2.83).  What bounds the stage now is the special-function
-      // unit: 137 results per row and tile keep it busy 72 % of the time.
+      // unit: 137 results per row and tile keep it busy 75 % of the time.
       const float c0 = 11.39231742277876f - m_new;        // log2(2688) - m'
       uint32_t sfw[2] = {0u, 0u};
       float off[8];

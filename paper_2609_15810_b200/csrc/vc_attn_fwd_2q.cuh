@@ -29,12 +29,12 @@ using namespace attn;
 //     accumulator hold l, rescaled by alpha together with the rest.  The softmax threads do
 //     nothing but the row maximum and five instructions per four codes.
 //
-// What bounds it: per key tile and pair of query tiles the kernel takes about 2200 cycles at d = 128
+// What bounds it: per key tile and pair of query tiles the kernel takes about 2070 cycles at d = 128
 // (1850 at d = 64).  The tensor pipe needs 1216 of them (704 at d = 64); two softmax warps per
 // scheduler need about 1000 when nothing else runs on it and the correction warps and the hand-offs
 // of the shared score buffer (1500 cycles per pair when they are all that is timed) take the rest.
 // Above a few milliseconds at a stretch the power cap of the board bounds it as well.
-// B1 H40 N32760 d128 13.3 -> 12.5 ms, B1 H12 without value smoothing 3.9 -> 3.0, B2 H16 N16384 d64 2.13 -> 1.73 by: waits that
+// B1 H40 N32760 d128 13.3 -> 12.5 ms, B1 H12 without value smoothing 3.9 -> 3.1 (3.5 under the power cap), B2 H16 N16384 d64 2.13 -> 1.73 by: waits that
 // test before they suspend, no operand expansion in front, query tiles of the last wave one by one.
 //
 //   warp 0        producer: Q0, Q1 once; then per key tile K^_j, R^_j (TMA) and the tile's block

@@ -43,7 +43,8 @@ def test_output_does_not_depend_on_the_split(N, grid, d, H, fmt, smooth):
 @pytest.mark.parametrize("fmt", list(FORMATS))
 @pytest.mark.parametrize("N,grid,d,H", [(4096, (4, 32, 32), 64, 32), (4096, (4, 32, 32), 128, 32), (2048, (2, 32, 32), 64, 8)])
 def test_calls_without_value_smoothing_are_repeatable(N, grid, d, H, fmt):
-    """Without block means the correction warps skip their waits for products; the output must still wait for the last."""
+    """Without block means the correction warps skip their waits for products; the output must still wait for the last.
+    (A repeated call cannot show an order that is only likely: tests/test_handoff_order.py goes through all of them.)"""
     g = torch.Generator(device="cuda").manual_seed(N + d)
     q, k, v = [torch.randn(1, H, N, d, generator=g, device="cuda").bfloat16() for _ in range(3)]
     first = _attn(q, k, v, grid, fmt, False)
