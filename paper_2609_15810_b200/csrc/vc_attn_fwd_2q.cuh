@@ -20,10 +20,14 @@ using namespace attn;
 // and streams each K^_j / R^_j tile through both, so every key/value byte fetched from L2
 // feeds 256 query rows.  Two decisions keep the softmax stage - the bottleneck on this GPU -
 // as short as the method allows:
-//   * The probability codes travel through SHARED memory, not through tensor memory, so a
-//     score tile is free as soon as its 128 x 128 values are in registers.  At d = 128 one score
-//     buffer serves both query tiles in turn (all that tensor memory has room for); at d = 64 each
-//     tile has its own.
+//   * The probability codes have tensor-memory columns of their own (32 per tile) and are the A operand
+//     of the value product there, so a score tile is free as soon as its 128 x 128 values are in
+//     registers.  At d = 128 one score buffer serves both query tiles in turn (all that tensor memory
+//     has room for); at d = 64 each tile has its own.  (An MMA with both operands in shared memory reads
+//     128 bytes a clock, all a shared-memory port gives.  With the codes there as well, 32 KB written and
+//     32 KB read per pair of tiles, every copy and store slowed the products down: B2 H16 N16384 d64
+//     1956 -> 1870 us, B1 H12 N32760 d128 without value smoothing 3677 -> 3604, B1 H40 12.49 -> 12.33 ms
+//     under the power cap, B1 H6 N1955 d64 29.8 -> 28.9 us.)
 //   * The row sums of the decoded codes (Eq. 6: r_ij, and the normalizer l) come from the
 //     tensor core: the value operand carries 16 extra rows of ones, so columns d..d+15 of the
 //     accumulator hold l, rescaled by alpha together with the rest.  The softmax threads do
@@ -42,17 +46,17 @@ using namespace attn;
 //   warp 1        score issuer (one elected lane), per key tile j and query tile t:
 //                   S    = Q^_t K^_j^T         4 x kind::f8f6f4, once the previous scores are read
 //   warp 3        accumulator issuer, per key tile j and query tile t:
-//                   A_t += P^_t(j) [R^_j | 1]  4 x kind::f8f6f4, N = d + 16, codes from shared memory
+//                   A_t += P^_t(j) [R^_j | 1]  4 x kind::f8f6f4, N = d + 16, codes from tensor memory
 //                   A_t += rho_{j-1} mu~_{j-1} 1 x kind::tf32: the rank-one mean term of Eq. 6, one
 //                                              tile late, because r_{j-1} is read back from A_t first
 //   warps 4-7     softmax warpgroup of tile 0, one thread per query row (128 scores in
 //   warps 8-11    registers); likewise tile 1: running max, alpha, ExpCast-FP8 codes (Eq. 7: no
-//                 exponential, no conversion), code tile in the swizzled K-major layout
+//                 exponential, no conversion), code tile to tensor memory (4 keys a column)
 //   warps 12-15   correction warpgroup of tile 0 (16-19: tile 1), one thread per row: reads l
 //                 back, r_{j-1} = l_{j-1} - alpha_{j-1} l_{j-2}, rescales A_t by alpha_j when a
 //                 row maximum moved, hands (r_hi, r_lo) alpha_j to the mean MMA, writes the output
 //
-// Tensor memory: S (128 columns; 2 x 128 at d = 64) | A_0 (d + 16) | A_1 (d + 16).
+// Tensor memory: S (128 columns; 2 x 128 at d = 64) | A_0 (d + 16) | A_1 (d + 16) | P_0 (32) | P_1 (32) at column 416.
 // P formats of the two-query-tile kernel
 constexpr int kPfExpCast = 0, kPfExp = 1, kPfExpPoly = 2, kPfExpMix = 3;
 
@@ -88,18 +92,17 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
   // d = 64 leaves room in tensor memory for a score buffer per query tile (B2 H16 N16384 d64: 1.89 -> 1.83 ms,
   // without smoothing 1.85 -> 1.76); at d = 128 both tiles share one
   constexpr bool kTwoS = D == 64;
-  constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE;   // A_t at O_COL + t * O_STRIDE; l in its column d
+  constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE, P_COL = 416;   // A_t at O_COL + t * O_STRIDE; l in its column d
   // Register re-partition (setmaxnreg): the CTA owns 640 x 96 registers; a warpgroup that asks for
   // more than the others released would block forever, so the budget is checked at compile time.
   constexpr int kRegCtl = 48, kRegSoftmax = 160, kRegCorr = 56;
   static_assert(kRegCtl + 2 * kRegSoftmax + 2 * kRegCorr <= 5 * 96, "register budget exceeds the CTA's allocation");
   constexpr uint32_t kQBytes = 128 * D, kKBytes = 128 * D, kVBytes = D * 128, kOnesBytes = 16 * 128, kMuBytes = D * 32;
   constexpr uint32_t kStageBytes = kKBytes + kVBytes + kOnesBytes + ((kMuBytes + 1023) / 1024) * 1024;
-  constexpr uint32_t kPBytes = 128 * 128, kAmBytes = 128 * 32;
+  constexpr uint32_t kAmBytes = 128 * 32;
   extern __shared__ __align__(1024) unsigned char smem[];     // (the swizzled tiles want 1024-byte alignment)
   unsigned char* sQ = smem;                                    // [2][128 x D]
-  unsigned char* sP = smem + 2 * kQBytes;                      // [2][128 x 128] probability codes
-  unsigned char* sAm = sP + 2 * kPBytes;                       // [2][128 x 8 fp32] row-sum pairs
+  unsigned char* sAm = smem + 2 * kQBytes;                       // [2][128 x 8 fp32] row-sum pairs
   unsigned char* sStage = sAm + 2 * kAmBytes;                  // [kStages2]{K, V | ones, Mu}
   FaSmem* sh = reinterpret_cast<FaSmem*>(sStage + kStages2 * kStageBytes);
 
@@ -213,7 +216,6 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       // A_t += P^_t(j) [R^_j | 1] once the codes are written, A_t is rescaled by alpha_j and the
       // row-sum pair of tile j-1 is in place; then the mean term of tile j-1.
       const uint32_t idesc_pv = idesc_e4m3(128, D + 16), idesc_mu = idesc_tf32(128, D);
-      const uint64_t dp[2] = {smem_desc_kmajor(smem_u32(sP), 128), smem_desc_kmajor(smem_u32(sP + kPBytes), 128)};
       const uint64_t dam[2] = {smem_desc_kmajor(smem_u32(sAm), 32), smem_desc_kmajor(smem_u32(sAm + kAmBytes), 32)};
       bool ok = true;
       for (int j = 0; ok && j < nb; ++j) {
@@ -229,7 +231,7 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) mma_f8_ss(o_col, (buf(t, j) ? dp[1] : dp[0]) + 2 * k, dv + 2 * k, idesc_pv, (j > 0) | (k > 0));
+            for (int k = 0; k < 4; ++k) mma_f8_ts(o_col, tmem + P_COL + 32 * buf(t, j) + 8 * k, dv + 2 * k, idesc_pv, (j > 0) | (k > 0));
             if (j > 0 && SMOOTH) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
             mma_commit(&sh->o_done[buf(t, j)]);
             if (j > 0) mma_commit(&sh->kv_empty[stp]);    // this tile is done with stage j-1
@@ -256,8 +258,6 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
     const int t = TWO ? (warp - 4) >> 2 : 0;               // query tile of this warpgroup
     const int row = (warp & 3) * 32 + lane;
     const int qblk = q0 + t;
-    // my row of the swizzled code tile: 16-byte chunk c sits at chunk position c ^ (row % 8)
-    const uint32_t p_row = smem_u32(sP + t * kPBytes + row * 128) + ((row & 7) << 4);
     const float sq = qblk < nb ? a.q_scale[(size_t)bh * nb + qblk] : 1.0f;
     const uint32_t alpha_at = smem_u32(&sh->alpha[0][row]);
     float m_run = -INFINITY;
@@ -345,12 +345,17 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
           return lo | (hi << 16);
         }
       };
-      auto store16 = [&](const uint32_t (&sv)[32], int half, int chunk) {   // keys 16*chunk .. +15
-        sts128((p_row + (TWO ? 0 : (j & 1) * kPBytes)) ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
+      const uint32_t p_col = lane_base + P_COL + 32 * buf(t, j);
+      auto store32 = [&](const uint32_t (&sv)[32], int q) {                 // keys 32 q .. + 31
+        uint32_t c[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) c[w] = code4(sv, w);
+        tmem_st8(p_col + 8 * q, c);
       };
-      store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
-      store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
+      tc_fence_after();
+      store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
+      tmem_wait_st();
+      tc_fence_before();
       mbar_arrive(&sh->pc_full[pc_slot(t, j)]);
     }
   } else if (TWO ? warp >= 12 : warp >= 12 && warp < 16) {
@@ -474,7 +479,7 @@ cudaError_t run_2q(const Problem& pr, const QuantLayout& ql, const WorkLayout& w
   AttnArgs a{};
   if (!fill_args8<D>(pr, ql, wl, quant, o, work, &a, &tq, &tk, &tv)) return cudaErrorUnknown;
   constexpr size_t stage = 2 * 128 * D + 2048 + ((D * 32 + 1023) / 1024) * 1024;
-  constexpr size_t smem = 2 * 128 * D + 2 * 128 * 128 + 2 * 128 * 32 + kStages2 * stage + sizeof(FaSmem);
+  constexpr size_t smem = 2 * 128 * D + 2 * 128 * 32 + kStages2 * stage + sizeof(FaSmem);
   static_assert(smem <= 227 * 1024, "shared memory of the kernel exceeds the SM");
   const bool int8 = pr.flags & VC_FLAG_INT8_QK, smooth = pr.flags & VC_FLAG_V_SMOOTH;
   const int pf = pr.p_format == VC_P_EXPCAST_E4M3 ? kPfExpCast
