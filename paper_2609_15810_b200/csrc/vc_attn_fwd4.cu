@@ -9,7 +9,7 @@
 // reads a tile's factors from the bundle's row-major arrays and writes them in chunk order.
 //
 // The pipeline is the one of the 8-bit kernel (two query tiles per CTA, one shared score
-// buffer, probability codes through shared memory, the row sums l from 16 rows of ones behind
+// buffer, probability codes through tensor memory, the row sums l from 16 rows of ones behind
 // the value tile, the block-mean term as a TF32 MMA one tile late).  What differs is the
 // softmax stage: P is quantized to NVFP4 per row and 16 keys.  The group maxima are a
 // by-product of the running-max pass; per group the E4M3 factor of max p / 6 is formed once,
@@ -91,6 +91,9 @@ __device__ __forceinline__ float decode_ue4m3(uint32_t code) {
   return code >= 8u ? __uint_as_float((code + 960u) << 20) : (float)code * 0.001953125f;
 }
 
+// The codes are the A operand of the value product in tensor memory; through shared memory, where the copies and both
+// operands of the score product meet, B1 H40 N32760 d128 took 11.69 ms instead of 11.20 (hybrid), B1 H24 N118800
+// 83.3 instead of 80.1, and B1 H12 N32760 4.49 instead of 4.45 (NVFP4).
 //   warp 0        TMA producer: Q^ tiles and their factors once; per key tile K^_j, R^_j, the
 //                 tile's factor chunks and block mean through a 4-stage ring
 //   warp 1        score issuer:        S = Q^_t K^_j^T            D/64 x kind::mxf4nvf4
@@ -98,7 +101,7 @@ __device__ __forceinline__ float decode_ue4m3(uint32_t code) {
 //                                      A_t += rho_{j-1} mu_{j-1}  1 x kind::tf32
 //   warps 4-11    softmax warpgroups (tile 0, tile 1), one thread per query row
 //   warps 12-19   correction warpgroups, one thread per query row
-// Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16) | scale factors (56 columns).
+// Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16) | scale factors (56 columns; HYB 32) | P_0 | P_1 (16 each; HYB 32).
 template <int D, bool HYB, bool SMOOTH, bool TWO>
 __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                               const Attn4Args& a, const int q0, const int bh) {
@@ -110,7 +113,10 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   constexpr bool kTwoS = D == 64 && HYB;
   constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE;
   constexpr uint32_t SF_COL = 416;
-  constexpr uint32_t SFQ_COL = SF_COL, SFK_COL = SF_COL + 16, SFP_COL = SF_COL + 24, SFV_COL = SF_COL + 40;
+  // (HYB: P^ takes the factor 1 for every row, and so do the rows of ones, value rows 128..143: one chunk serves both)
+  constexpr uint32_t SFQ_COL = SF_COL, SFK_COL = SF_COL + 16, SFV_COL = SF_COL + (HYB ? 24 : 40), SFP_COL = SF_COL + (HYB ? 28 : 24);
+  constexpr uint32_t P_COL = SF_COL + (HYB ? 32 : 56), kPCols = HYB ? 32 : 16;
+  static_assert(P_COL + 2 * kPCols <= kTmemCols, "tensor memory of the 4-bit kernel");
   // (the NVFP4 softmax wants the larger share: B1 H12 N32760 d128 4.44 -> 4.39 ms)
   constexpr int kRegCtl = 48, kRegSoftmax = HYB ? 160 : 168, kRegCorr = HYB ? 56 : 48;
   static_assert(kRegCtl + 2 * kRegSoftmax + 2 * kRegCorr <= 5 * 96, "register budget exceeds the CTA's allocation");
@@ -121,14 +127,13 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   constexpr uint32_t kMuBytes = D * 32, kMuPad = ((kMuBytes + 1023) / 1024) * 1024;
   constexpr uint32_t kSfBytes = (KB + NVC) * 512, kSfPad = ((kSfBytes + 1023) / 1024) * 1024;
   constexpr uint32_t kStageBytes = kKBytes + kVBytes + kOnesBytes + kMuPad + kSfPad;
-  constexpr uint32_t kPBytes = 128 * kVRow, kSfpBytes = 1024, kAmBytes = 128 * 32;
+  constexpr uint32_t kSfpBytes = 1024, kAmBytes = 128 * 32;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* sQ = smem;                                    // [2][128 x D/2]
-  unsigned char* sP = sQ + 2 * kQBytes;                        // [2][128 x 64] probability codes (HYB: 128 x 128)
-  unsigned char* sAm = sP + 2 * kPBytes;                       // [2][128 x 8 fp32] row-sum pairs
+  unsigned char* sAm = sQ + 2 * kQBytes;                       // [2][128 x 8 fp32] row-sum pairs
   unsigned char* sSfq = sAm + 2 * kAmBytes;                    // [2][KB][512] Q^ factors
-  unsigned char* sSfp = sSfq + 2 * 1024;                       // [2][2][512]  P^ factors (HYB: one chunk of ones)
+  unsigned char* sSfp = sSfq + 2 * 1024;                       // [2][2][512]  P^ factors (HYB: unused)
   unsigned char* sSfOnes = sSfp + 2 * kSfpBytes;               // [512] factors of value rows 128..143, then the table of logarithms
   float* sLg2 = reinterpret_cast<float*>(sSfOnes + 512);       // [128] log2 of the E4M3 values
   unsigned char* sStage = sSfOnes + 1024;                      // [kStages2]{K, V | ones, Mu, factors}
@@ -167,11 +172,9 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   for (int i = tid; i < kStages2 * (int)kOnesBytes / 16; i += 640)
     reinterpret_cast<uint4*>(sStage + (i / (kOnesBytes / 16)) * kStageBytes + kKBytes + kVBytes)[i % (kOnesBytes / 16)] = make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
   for (int i = tid; i < 128; i += 640)
-    reinterpret_cast<uint32_t*>(sSfOnes)[i] = ((i & 3) == 0 && i < 64) ? (HYB ? 0x7f7f7f7fu : 0x38383838u) : 0u;
+    reinterpret_cast<uint32_t*>(sSfOnes)[i] = HYB ? 0x7f7f7f7fu : ((i & 3) == 0 && i < 64) ? 0x38383838u : 0u;
   if constexpr (!HYB)                                          // (no lane takes code 127, the NaN)
     for (int i = tid; i < 128; i += 640) sLg2[i] = i ? lg2_approx(decode_ue4m3(i)) : INFINITY;
-  if constexpr (HYB)
-    for (int i = tid; i < 128; i += 640) reinterpret_cast<uint32_t*>(sSfp)[i] = 0x7f7f7f7fu;
   pdl_wait();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor-core reads
   if (warp == 2) { tmem_alloc<kTmemCols>(&sh->tmem_base); tmem_relinquish(); }
@@ -267,14 +270,14 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
     } else if (warp == 3) {
       // ------------------------------------------------------------------ accumulator issuer
       const uint32_t idesc_pv = idesc_nvfp4(128, D + 16), idesc_mu = idesc_tf32(128, D);
-      const uint64_t dp[2] = {smem_desc_kmajor(smem_u32(sP), kVRow), smem_desc_kmajor(smem_u32(sP + kPBytes), kVRow)};
       const uint64_t dam[2] = {smem_desc_kmajor(smem_u32(sAm), 32), smem_desc_kmajor(smem_u32(sAm + kAmBytes), 32)};
       if (elect_one()) {
-        if (D == 128) {                                    // factors of the rows of ones (value rows 128..143)
+        if (HYB) {                                         // P^, and at d = 128 the rows of ones
+          tmem_cp_sf(tmem + SFP_COL, smem_desc_sf_chunk(smem_u32(sSfOnes)));
+        } else if (D == 128) {                             // factors of the rows of ones (value rows 128..143)
           tmem_cp_sf(tmem + SFV_COL + 4, smem_desc_sf_chunk(smem_u32(sSfOnes)));
-          if (!HYB) tmem_cp_sf(tmem + SFV_COL + 12, smem_desc_sf_chunk(smem_u32(sSfOnes)));
+          tmem_cp_sf(tmem + SFV_COL + 12, smem_desc_sf_chunk(smem_u32(sSfOnes)));
         }
-        if (HYB) tmem_cp_sf(tmem + SFP_COL, smem_desc_sf_chunk(smem_u32(sSfp)));   // P^: factor 1 everywhere
       }
       __syncwarp();
       bool ok = true;
@@ -293,12 +296,12 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
             tc_fence_after();
             const uint32_t o_col = tmem + O_COL + O_STRIDE * t;
             const int b = buf(t, j);
-            const uint64_t dpt = b ? dp[1] : dp[0];
+            const uint32_t p_at = tmem + P_COL + kPCols * b;
             if constexpr (HYB) {
               if (t == 0) tmem_cp_sf(tmem + SFV_COL, smem_desc_sf_chunk(sfv_smem));
 #pragma unroll
               for (int k = 0; k < 4; ++k)                  // 32 keys each; factor byte k of the value rows
-                mma_mxf8_ss(o_col, dpt + 2 * k, dv + 2 * k, idesc_mxf8_e4m3_e2m1(128, D + 16, k), (j > 0) | (k > 0),
+                mma_mxf8_ts(o_col, p_at + 8 * k, dv + 2 * k, idesc_mxf8_e4m3_e2m1(128, D + 16, k), (j > 0) | (k > 0),
                             tmem + SFP_COL, tmem + SFV_COL);
             } else {
               if (t == 0) {
@@ -309,7 +312,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
               tmem_cp_sf(tmem + SFP_COL + b * 8 + 4, smem_desc_sf_chunk(smem_u32(sSfp + b * kSfpBytes + 512)));
 #pragma unroll
               for (int kb = 0; kb < 2; ++kb)
-                mma_nvfp4_ss(o_col, dpt + 2 * kb, dv + 2 * kb, idesc_pv, (j > 0) | (kb > 0), tmem + SFP_COL + b * 8 + kb * 4,
+                mma_nvfp4_ts(o_col, p_at + 8 * kb, dv + 2 * kb, idesc_pv, (j > 0) | (kb > 0), tmem + SFP_COL + b * 8 + kb * 4,
                              tmem + SFV_COL + kb * 8);
             }
             if (j > 0 && SMOOTH) mma_tf32_ss(o_col, dam[t], dm, idesc_mu, 1);
@@ -337,9 +340,6 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
     reg_inc<kRegSoftmax>();
     const int t = TWO ? (warp - 4) >> 2 : 0;               // query tile of this warpgroup
     const int row = (warp & 3) * 32 + lane;
-    // my row of the swizzled code tile: 64-byte rows, chunk c sits at chunk position c ^ ((row / 2) % 4)
-    // (HYB: 128-byte rows, chunk c at position c ^ (row % 8))
-    const uint32_t p_row = smem_u32(sP + t * kPBytes + row * kVRow) + ((HYB ? row & 7 : (row >> 1) & 3) << 4);
     const uint32_t sfp_row = smem_u32(sSfp + t * kSfpBytes + (row & 31) * 16 + (row >> 5) * 4);
     const float cs = (a.q_g[bh] * a.k_g[bh]) * a.sl;       // code units -> log2 domain
     const uint32_t lg2_at = smem_u32(sLg2);
@@ -396,12 +396,17 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
         auto code4 = [&](const uint32_t (&sv)[32], int w) -> uint32_t {
           return expcast_codes4(sv[4 * w], sv[4 * w + 1], sv[4 * w + 2], sv[4 * w + 3], fa2, fb2);
         };
-        auto store16 = [&](const uint32_t (&sv)[32], int half, int chunk) {   // keys 16 chunk .. +15
-          sts128((p_row + (TWO ? 0 : (j & 1) * kPBytes)) ^ (chunk << 4), code4(sv, 4 * half), code4(sv, 4 * half + 1), code4(sv, 4 * half + 2), code4(sv, 4 * half + 3));
+        const uint32_t p_col = lane_base + P_COL + kPCols * buf(t, j);
+        auto store32 = [&](const uint32_t (&sv)[32], int q) {               // keys 32 q .. + 31, four a column
+          uint32_t c[8];
+#pragma unroll
+          for (int w = 0; w < 8; ++w) c[w] = code4(sv, w);
+          tmem_st8(p_col + 8 * q, c);
         };
-        store16(s0, 0, 0); store16(s0, 1, 1); store16(s1, 0, 2); store16(s1, 1, 3);
-        store16(s2, 0, 4); store16(s2, 1, 5); store16(s3, 0, 6); store16(s3, 1, 7);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
+        tc_fence_after();
+        store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
+        tmem_wait_st();
+        tc_fence_before();
         mbar_arrive(&sh->pc_full[slot(t, j)]);
         continue;
       }
@@ -447,14 +452,18 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
         return make_uint2(cvt_e2m1x8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]),
                           cvt_e2m1x8(v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]));
       };
-      auto store32 = [&](const uint32_t (&sv)[32], int chunk) {   // keys 32 chunk .. +31 -> 16 bytes
-        const uint2 lo = quant16(sv, 0, 2 * chunk), hi = quant16(sv, 1, 2 * chunk + 1);
-        sts128((p_row + (TWO ? 0 : (j & 1) * kPBytes)) ^ (chunk << 4), lo.x, lo.y, hi.x, hi.y);
+      const uint32_t p_col = lane_base + P_COL + kPCols * buf(t, j);
+      auto store32 = [&](const uint32_t (&sv)[32], int q) {       // keys 32 q .. + 31, eight a column
+        const uint2 lo = quant16(sv, 0, 2 * q), hi = quant16(sv, 1, 2 * q + 1);
+        tmem_st4(p_col + 4 * q, lo.x, lo.y, hi.x, hi.y);
       };
+      tc_fence_after();
       store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
       sts32(sfp_row + (TWO ? 0 : (j & 1) * kSfpBytes), __uint_as_float(sfw[0]));
       sts32(sfp_row + (TWO ? 0 : (j & 1) * kSfpBytes) + 512, __uint_as_float(sfw[1]));                               // the chunk of keys 64..127
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // my stores -> tensor-core reads
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");          // the factors -> tensor-core reads
+      tmem_wait_st();
+      tc_fence_before();
       mbar_arrive(&sh->pc_full[slot(t, j)]);
     }
   } else if (TWO ? warp >= 12 : warp >= 12 && warp < 16) {
@@ -582,7 +591,7 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   a.code_off = 120.0f + pr.beta;
   a.wait = {a.status, attn_wait_limit(), attn_wait_nonblocking()};
   constexpr size_t stage = 128 * (D / 2) + (D + 16) * kVRow + ((D * 32 + 1023) / 1024) * 1024 + (((KB + NVC) * 512 + 1023) / 1024) * 1024;
-  constexpr size_t smem = 1024 + 2 * 128 * (D / 2) + 2 * 128 * kVRow + 2 * 128 * 32 + 2 * 1024 + 2 * 1024 + 1024 + kStages2 * stage + sizeof(FaSmem);
+  constexpr size_t smem = 1024 + 2 * 128 * (D / 2) + 2 * 128 * 32 + 2 * 1024 + 2 * 1024 + 1024 + kStages2 * stage + sizeof(FaSmem);
   static_assert(smem <= 227 * 1024, "shared memory of the 4-bit kernel exceeds the SM");
   unsigned grid;
   a.tiles = split_tiles(pr, true, &grid);
