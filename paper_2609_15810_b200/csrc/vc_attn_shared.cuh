@@ -72,6 +72,7 @@ struct FaSmem {
   uint64_t a_full[4], pc_full[4];
   uint64_t drain[2];      // exit: "every MMA this issuer warp issued has completed"
   float alpha[4][128];
+  alignas(16) float v_scale[2][128];  // s_V, one copy per correction warpgroup
   uint32_t tmem_base;
   volatile int abort;
 };
