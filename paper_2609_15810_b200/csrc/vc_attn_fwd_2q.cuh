@@ -430,28 +430,28 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
     }
     if (ok && (!SMOOTH || warp_wait2(&sh->o_final[t], 0, sh, a.wait, 43))) {
       tc_fence_after();
-      const int grow = qblk * 128 + row;
+      static_assert(kStageBytes >= 128 * 2 * D, "a query tile's output fits a stage");
+      using Out = OutTile<D>;
+      const int row0 = qblk * 128 + (warp & 3) * 32;       // the warp's first row
+      const uint32_t tile = smem_u32(sStage + ((nb + t) % kStages2) * kStageBytes) + (warp & 3) * 32 * Out::ROW;
       const float inv_l = 1.0f / l_now;
 #pragma unroll 1
       for (int c = 0; c < D / 16; ++c) {
-        uint32_t r[16];
+        uint32_t r[16], out[8];
         tmem_ld16(o_base + 16 * c, r);
         tmem_wait_ld();
-        if (grow < a.N) {
-          uint32_t out[8];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 s4 = lds128(vs_at + 64 * c + 16 * i);
-            const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(r[4 * i]) * inv_l * s4.x, __uint_as_float(r[4 * i + 1]) * inv_l * s4.y);
-            const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(r[4 * i + 2]) * inv_l * s4.z, __uint_as_float(r[4 * i + 3]) * inv_l * s4.w);
-            out[2 * i] = *reinterpret_cast<const uint32_t*>(&h0);
-            out[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&h1);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(a.o + ((size_t)bh * a.N + grow) * D + 16 * c);
-          dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-          dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+        for (int i = 0; i < 4; ++i) {
+          const float4 s4 = lds128(vs_at + 64 * c + 16 * i);
+          const __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(r[4 * i]) * inv_l * s4.x, __uint_as_float(r[4 * i + 1]) * inv_l * s4.y);
+          const __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(r[4 * i + 2]) * inv_l * s4.z, __uint_as_float(r[4 * i + 3]) * inv_l * s4.w);
+          out[2 * i] = *reinterpret_cast<const uint32_t*>(&h0);
+          out[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&h1);
         }
+        sts128(Out::chunk(tile, lane, 2 * c), out[0], out[1], out[2], out[3]);
+        sts128(Out::chunk(tile, lane, 2 * c + 1), out[4], out[5], out[6], out[7]);
       }
+      Out::store(tile, reinterpret_cast<unsigned char*>(a.o + ((size_t)bh * a.N + row0) * D), 2 * D, a.N - row0, lane);
     }
   }
   tc_fence_before();
