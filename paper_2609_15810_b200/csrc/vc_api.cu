@@ -171,7 +171,7 @@ size_t vc_workspace_bytes(const vc_params* p) {
 }
 
 static vc_status prep_impl(const vc_params* p, const void* q, const void* k, const void* v, const int32_t* perm,
-                           const vc_prep_stats* stats, void* quant, void* workspace, void* stream) {
+                           const vc_prep_stats* stats, void* quant, void* workspace, void* stream, bool then_attention = false) {
   Problem pr;
   vc_status st = resolve(p, &pr);
   if (st != VC_OK) return st;
@@ -187,7 +187,7 @@ static vc_status prep_impl(const vc_params* p, const void* q, const void* k, con
     if (misaligned(stats->k_mean) || misaligned(stats->v_block_mean) || misaligned(stats->v_amax)) return VC_ERR_INVALID_ARG;
   }
   cudaError_t e = launch_prep(pr, ql, wl, q, k, v, perm, (uint8_t*)quant, (uint8_t*)workspace,
-                              (cudaStream_t)stream, stats);
+                              (cudaStream_t)stream, stats, then_attention);
   return e == cudaSuccess ? VC_OK : VC_ERR_CUDA;
 }
 
@@ -238,7 +238,7 @@ vc_status vc_attn_fwd(const vc_params* p, const void* quant, void* o, void* work
 
 vc_status vc_attn(const vc_params* p, const void* q, const void* k, const void* v,
                   const int32_t* perm, void* o, void* quant, void* workspace, void* stream) {
-  vc_status st = vc_prep(p, q, k, v, perm, quant, workspace, stream);
+  vc_status st = prep_impl(p, q, k, v, perm, nullptr, quant, workspace, stream, true);
   if (st != VC_OK) return st;
   return attn_fwd_impl(p, quant, o, workspace, stream, false);   // keeps what the pass recorded in the status word
 }

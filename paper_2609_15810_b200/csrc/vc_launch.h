@@ -10,7 +10,8 @@
 //     waits before it does anything.)
 //   - Therefore a kernel may read, in front of its wait, what the kernel before it neither writes nor makes
 //     late: the preprocessing passes read Q, K, V and the permutation, the assignment of vc_group reads V.  The
-//     kernels before them (table, permutation check, passes, finalize; init, update) write none of these.  Another
+//     kernels before them (table, permutation check, passes, finalize; init, update) write none of these.  (The one launch
+//     of short heads stands behind a caller's kernels and reads nothing in front of its wait.)  Another
 //     kernel put in between has to keep to that, and has to wait before it allows.
 // What is gained is the gap between two kernels (about 1.5 us) and the successor's prologue.
 #pragma once
@@ -23,18 +24,25 @@
 namespace vc {
 
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+inline cudaError_t launch_clusters(void (*kernel)(P...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_clusters(kernel, grid, 1, threads, smem, s, args...);
 }
 
 // A number for the current context that no other context of the process gets, 0 if there is none yet.

@@ -13,6 +13,7 @@
 // can be processed in groups so that the second read of K and V may hit L2.  All passes are
 // persistent kernels that prefetch the next row blocks with cp.async while they transform
 // the current one.
+#include <algorithm>
 #include <climits>
 
 #include "vc_launch.h"
@@ -34,8 +35,22 @@ struct SetUp {
   float *k_mean, *v_scale;
 };
 __device__ __forceinline__ float value_scale(float amax) { return amax > 0.f ? amax / 448.0f : 1.0f; }
+__device__ __forceinline__ float outer_scale(float amax) { return amax > 0.f ? amax / 2688.0f : 1.0f; }     // NVFP4, per head
+
+// Frequency of pair i of an axis with `pairs` channel pairs, and the entry of a position: (cos, sin) and, in `folded`, the
+// rotation folded into the first Hadamard level, u = x0 (c + s) + x1 (c - s), v = x0 (c - s) - x1 (c + s), each
+// coefficient rounded once.
+__device__ __forceinline__ double rope_freq(double theta, int i, int pairs) { return pow(theta, -2.0 * (double)i / (double)(2 * pairs)); }
+__device__ __forceinline__ void rope_entry_of(int pos, double freq, float2* plain, float2* folded) {
+  double c, sn;
+  sincos((double)pos * freq, &sn, &c);
+  *plain = make_float2((float)c, (float)sn);
+  *folded = make_float2((float)(c + sn), (float)(c - sn));
+}
 
 __global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta, const SetUp u) {
+  // (The wait stands in front of the arithmetic: entries computed beside the end of the attention before them make calls
+  // of 2000 to 4000 tokens 1 to 3 percent slower.)
   pdl_wait();
   pdl_allow();
   const int e = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
@@ -46,18 +61,11 @@ __global__ void rope_table_kernel(float2* tab, RopeDesc rd, double theta, const 
     u.v_scale[i] = value_scale(u.ext_v_amax[i]);
   }
   if (e >= rd.entries) return;
-  int a = e >= rd.off[2] ? 2 : (e >= rd.off[1] ? 1 : 0);
-  int r = e - rd.off[a];
-  int pos = r / rd.pairs[a];
-  int i = r - pos * rd.pairs[a];
-  double freq = pow(theta, -2.0 * (double)i / (double)(2 * rd.pairs[a]));
-  double phi = (double)pos * freq;
-  double c, sn;
-  sincos(phi, &sn, &c);
-  tab[e] = make_float2((float)c, (float)sn);
-  // second table: the rotation folded into the first Hadamard level, u = x0 (c + s) + x1 (c - s),
-  // v = x0 (c - s) - x1 (c + s), each coefficient rounded once
-  tab[rd.entries + e] = make_float2((float)(c + sn), (float)(c - sn));
+  const int a = e >= rd.off[2] ? 2 : (e >= rd.off[1] ? 1 : 0), r = e - rd.off[a], pos = r / rd.pairs[a], i = r - pos * rd.pairs[a];
+  float2 plain, folded;
+  rope_entry_of(pos, rope_freq(theta, i, rd.pairs[a]), &plain, &folded);
+  tab[e] = plain;
+  tab[rd.entries + e] = folded;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -150,8 +158,9 @@ __device__ __forceinline__ PairSlots pair_slots(const RopeDesc& rd, int first_pa
 }
 
 template <int D>
-__device__ __forceinline__ void k_colsum_item(const PrepArgs& a, const unsigned char* stage, float* red, const RopeTab& tab,
-                                              const PairSlots& ps, int bh, int blk) {
+__device__ __forceinline__ void k_colsum_item(const PrepArgs& a, const unsigned char* mine /*this thread's chunk of its first row*/,
+                                              int step /*bytes to its next row's*/, float* red, const RopeTab& tab, const PairSlots& ps,
+                                              float* out /*[D]*/, int blk) {
   constexpr int LPR = D / 8;         // lanes per row
   constexpr int RPL = LPR / 2;       // rows per lane (a warp covers 16 rows)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -188,7 +197,7 @@ __device__ __forceinline__ void k_colsum_item(const PrepArgs& a, const unsigned 
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
       if (i >= n_rows) break;
-      const uint4 raw = *reinterpret_cast<const uint4*>(stage + (i * kThreads + tid) * 16);   // the chunk this thread fetched
+      const uint4 raw = *reinterpret_cast<const uint4*>(mine + i * step);
       const unsigned int w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -216,7 +225,7 @@ __device__ __forceinline__ void k_colsum_item(const PrepArgs& a, const unsigned 
 #pragma unroll
     for (int i = 0; i < RPL; ++i) {
       if (i >= n_rows) break;
-      const uint4 raw = *reinterpret_cast<const uint4*>(stage + (i * kThreads + tid) * 16);   // the chunk this thread fetched
+      const uint4 raw = *reinterpret_cast<const uint4*>(mine + i * step);
       const unsigned int w[4] = {raw.x, raw.y, raw.z, raw.w};
       float x[8];
 #pragma unroll
@@ -254,7 +263,7 @@ __device__ __forceinline__ void k_colsum_item(const PrepArgs& a, const unsigned 
     float t = 0.f;
 #pragma unroll
     for (int w8 = 0; w8 < 8; ++w8) t += red[w8 * D + tid];
-    a.k_part[((size_t)bh * a.nb + blk) * D + tid] = t;
+    out[tid] = t;
   }
 }
 
@@ -288,7 +297,7 @@ template <int D> __device__ __forceinline__ constexpr int rope_axis_of(int p) {
 template <int D, int STAGE>
 __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR /*0 = Q, 1 = K*/, const unsigned char* stage,
                                             unsigned char* out_tile, float* red, float* kmean_s, const RopeTab& tab, int bh,
-                                            int blk, int iter, bool new_head, int src_row) {
+                                            int blk, int iter, bool new_head, int src_row, unsigned int* amax_at) {
   constexpr int C = D / kTpr;                      // channels per thread
   constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -401,7 +410,7 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
     amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
-    if (tid == 0) atomicMax(&a.qk_amax[TENSOR * a.BH + bh], __float_as_uint(amax));
+    if (tid == 0) atomicMax(amax_at, __float_as_uint(amax));
     return;
   }
   const size_t row_g = (size_t)bh * a.n_pad + (size_t)blk * kBlock + row;
@@ -494,11 +503,12 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 //    operation per lane, one instruction issued for two);
 //  * at 8 bits 1 / sqrt(D) and the quantization scale are one factor.
 // The 4-bit head-maximum and NVFP4 stages run on the same transform.
-// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed.
+// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed; `outer` is the head's NVFP4
+// scale, `amax_at` where the head maximum is collected.
 template <int D, int STAGE>
 __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TENSOR, const unsigned char* stage,
                                                  unsigned char* out_tile, float* red, float* kmean_pm, uint32_t tab_saddr,
-                                                 int bh, int blk, int iter, bool new_head, int src_row) {
+                                                 int bh, int blk, int iter, bool new_head, int src_row, unsigned int* amax_at, float outer) {
   constexpr int C = D / kTpr, P = C / 2;           // channels and pairs per thread
   constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -596,13 +606,13 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
     amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
-    if (tid == 0) atomicMax(&a.qk_amax[TENSOR * a.BH + bh], __float_as_uint(amax));
+    if (tid == 0) atomicMax(amax_at, __float_as_uint(amax));
     return;
   }
   if constexpr (STAGE == kStageQuant4) {
     // NVFP4: outer scale g per (b, h), microscale per token per 16 channels (the arithmetic of the
     // general row body: y = x / sqrt(D), then y / (g * microscale), each rounded once)
-    const float g = (TENSOR == 0 ? a.q_scale : a.k_scale)[bh];
+    const float g = outer;
     const float inv6 = 1.0f / (6.0f * g);
     const uint64_t RS = pack_f32x2(rs, rs);
     constexpr int MB = C / 16;                     // microscale bytes of this thread
@@ -702,7 +712,7 @@ enum { kVStats = 0, kVQuant8 = 1, kVQuant4 = 2, kVQuant4M = 3 };   // 4M: E2M1 u
 //     max_i |v_i - mu| = max(max_i v_i - mu, mu - min_i v_i)
 // bit for bit, because the FP32 subtraction is monotonic.
 template <int D, bool FULL>
-__device__ __forceinline__ void v_stats_item(const PrepArgs& a, const unsigned char* stage, float* red, int bh, int blk) {
+__device__ __forceinline__ void v_stats_item(const PrepArgs& a, const unsigned char* stage, float* red, int bh, int blk, unsigned int* amax_at /*[D]*/) {
   constexpr int CP = D / 2, TG = kThreads / CP, TPG = kBlock / TG;
   const int tid = threadIdx.x;
   const int cp = tid % CP, tg = tid / CP;
@@ -746,8 +756,8 @@ __device__ __forceinline__ void v_stats_item(const PrepArgs& a, const unsigned c
     *reinterpret_cast<float2*>(a.v_mu + mu_at) = make_float2(mu0, mu1);
     const float2 hi = __bfloat1622float2(mx), lo = __bfloat1622float2(mn);
     const float m0 = fmaxf(hi.x - mu0, mu0 - lo.x), m1 = fmaxf(hi.y - mu1, mu1 - lo.y);
-    atomicMax(&a.v_amax[(size_t)bh * D + 2 * cp], __float_as_uint(m0));
-    atomicMax(&a.v_amax[(size_t)bh * D + 2 * cp + 1], __float_as_uint(m1));
+    atomicMax(&amax_at[2 * cp], __float_as_uint(m0));
+    atomicMax(&amax_at[2 * cp + 1], __float_as_uint(m1));
   }
 }
 
@@ -985,7 +995,7 @@ __device__ __forceinline__ void kcolsum_pass(const PrepArgs& a, unsigned char* s
   for (int item = sl.rank; item < sl.n_items; item += sl.stride, ++i) {
     issue(item + sl.stride, nxt, (i + 1) & 1);
     cp_async_wait<1>();                       // this thread's chunks of item i have landed
-    k_colsum_item<D>(a, smem + (i & 1) * kStage, red, tab, ps, a.bh0 + cur.hh, cur.blk);
+    k_colsum_item<D>(a, smem + (i & 1) * kStage + tid * 16, kThreads * 16, red, tab, ps, a.k_part + ((size_t)(a.bh0 + cur.hh) * a.nb + cur.blk) * D, cur.blk);
     cur = nxt;
     advance(nxt, step, a.nb, nh);
   }
@@ -1062,8 +1072,9 @@ __device__ __forceinline__ void v_pass(const PrepArgs& a, unsigned char* smem, c
     const unsigned char* stage = smem + (i % 3) * kStage;
     const bool full = a.N - c0.blk * kBlock >= kBlock;
     if constexpr (STAGE == kVStats) {
-      if (full) v_stats_item<D, true>(a, stage, red, a.bh0 + c0.hh, c0.blk);
-      else v_stats_item<D, false>(a, stage, red, a.bh0 + c0.hh, c0.blk);
+      unsigned int* amax_at = a.v_amax + (size_t)(a.bh0 + c0.hh) * D;
+      if (full) v_stats_item<D, true>(a, stage, red, a.bh0 + c0.hh, c0.blk, amax_at);
+      else v_stats_item<D, false>(a, stage, red, a.bh0 + c0.hh, c0.blk, amax_at);
     } else {
       if (full) v_item<D, STAGE, true>(a, stage, red, a.bh0 + c0.hh, c0.blk, mu, am);
       else v_item<D, STAGE, false>(a, stage, red, a.bh0 + c0.hh, c0.blk, mu, am);
@@ -1099,13 +1110,22 @@ __global__ void prep_finalize_kernel(const PrepArgs a, int which) {
       a.k_mean[(size_t)bh * D + c] = (float)(s / (double)a.N);
       a.v_scale[(size_t)bh * D + c] = BITS == 8 ? value_scale(__uint_as_float(a.v_amax[(size_t)bh * D + c])) : 1.0f;
     }
-    if (BITS == 4 && threadIdx.x == 0) {
-      const float am = __uint_as_float(a.qk_amax[bh]);
-      a.q_scale[bh] = am > 0.f ? am / 2688.0f : 1.0f;
-    }
+    if (BITS == 4 && threadIdx.x == 0) a.q_scale[bh] = outer_scale(__uint_as_float(a.qk_amax[bh]));
   } else if (BITS == 4 && threadIdx.x == 0) {
-    const float am = __uint_as_float(a.qk_amax[a.BH + bh]);
-    a.k_scale[bh] = am > 0.f ? am / 2688.0f : 1.0f;
+    a.k_scale[bh] = outer_scale(__uint_as_float(a.qk_amax[a.BH + bh]));
+  }
+}
+
+// A warp's rows of the swizzled code tile, from row0 on -> the block's code rows: full-line stores.
+template <int ROW_BYTES>
+__device__ __forceinline__ void store_warp_rows(uint8_t* block, const unsigned char* out_tile, int row0, int lane) {
+  constexpr int CPR = ROW_BYTES / 16, RW = 32 / kTpr;                // 16-byte chunks per code row, rows of a warp
+  uint4* gdst = reinterpret_cast<uint4*>(block + (size_t)row0 * ROW_BYTES) + lane;
+#pragma unroll
+  for (int k = 0; k < CPR * RW / 32; ++k) {
+    const int idx = k * 32 + lane, row = row0 + idx / CPR, chunk = idx % CPR;
+    const int sw = (row / (8 / CPR)) & (CPR - 1);
+    gdst[k * 32] = *reinterpret_cast<const uint4*>(out_tile + row * ROW_BYTES + ((chunk ^ sw) << 4));
   }
 }
 
@@ -1122,7 +1142,6 @@ template <int D, int STAGE, bool FAST>
 __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
   constexpr int NT = kRowThreads * kTpr;
   constexpr int kRowBytes = STAGE == kStageQuant4 ? D / 2 : D;      // code bytes per row
-  constexpr int CPR = kRowBytes / 16;                                // 16-byte chunks per code row
   constexpr int RW = 32 / kTpr;                                      // rows of a warp
   constexpr int LPR = D / 8;                                         // lanes on one input row
   constexpr int RPI = 32 / LPR;                                      // input rows per warp instruction
@@ -1182,20 +1201,16 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
     const unsigned char* stage = smem + (i & 1) * Geo<D>::stage_bytes;
     const int s0 = src_ring[(i % 3) * kBlock + my_row];
     const int tensor = c0.z + z0, bh = a.bh0 + c0.hh;
+    unsigned int* amax_at = a.qk_amax + tensor * a.BH + bh;
     if constexpr (FAST)
-      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
+      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at,
+                                 STAGE == kStageQuant4 ? (tensor == 0 ? a.q_scale : a.k_scale)[bh] : 0.f);
     else
-      qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0);
+      qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at);
     if (tensor == 1) last_hh = c0.hh;
     if constexpr (STAGE != kStageAmax) {
       __syncwarp();                           // the warp's rows of the code tile are complete
-      uint4* gdst = reinterpret_cast<uint4*>((tensor == 0 ? a.q_codes : a.k_codes) + ((size_t)bh * a.n_pad + (size_t)c0.blk * kBlock + row0) * kRowBytes) + lane;
-#pragma unroll
-      for (int k = 0; k < CPR * RW / 32; ++k) {
-        const int idx = k * 32 + lane, row = row0 + idx / CPR, chunk = idx % CPR;
-        const int sw = (row / (8 / CPR)) & (CPR - 1);
-        gdst[k * 32] = *reinterpret_cast<const uint4*>(out_tile + row * kRowBytes + ((chunk ^ sw) << 4));
-      }
+      store_warp_rows<kRowBytes>((tensor == 0 ? a.q_codes : a.k_codes) + ((size_t)bh * a.n_pad + (size_t)c0.blk * kBlock) * kRowBytes, out_tile, row0, lane);
     }
     c0 = c1;
     advance(c1, step, a.nb, nh);
@@ -1247,7 +1262,8 @@ __global__ void __launch_bounds__(kThreads, 2) prep_kernel(const PrepArgs a, con
   extern __shared__ __align__(128) unsigned char smem[];
   // (No early pdl_allow: attention CTAs that start one by one as this kernel's leave do not run through a
   // head's key tiles together, and the hybrid attention takes 3.5 percent longer at B1 H40 N32760, 3.6 at
-  // B1 H12 N32760.  The next kernel starts when the last CTA has ended.)
+  // B1 H12 N32760.  Nor where the attention is one wave: 1 to 2 percent at 2000 to 4000 tokens.  The next kernel
+  // starts when the last CTA has ended.)
   constexpr int kPasses = PHASE == kPhase3 ? 1 : (PHASE == kPhase1 ? 3 : 2);
   const int b = blockIdx.x;
   if constexpr (!TURNS) {
@@ -1392,12 +1408,250 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------------------
+// Short heads in front of an attention launch: the whole pass in one launch, a cluster of CTAs per head and tensor, a CTA
+// per block.  Few blocks keep the GPU busy for a few microseconds, and what the pass then costs is its chain of
+// launches: table, statistics, finalization, codes, at 4 bits two more, 0.8 to 1.5 us from the end of each to the start of
+// the next beside its own filling of a pipeline (13.2 us from the table's start to the attention's at B1 H2 N1024 d128).  Here
+//   - every CTA computes the RoPE tables it needs itself, in front of the wait for the kernel before it;
+//   - a CTA keeps its block in shared memory, so K and V are read once and the statistics of a head meet in distributed
+//     shared memory, behind one cluster barrier each;
+//   - K is staged twice when a permutation gathers it: in sequence order for the column sums (and the head maximum),
+//     gathered for the codes.  The sums run over the same blocks, in the same order, as in the launches above.
+// The row and value transforms are the ones of the other launches, and the bundle is the same, byte for byte.
+// Whole calls (d128; four launches before): FP8 B1 H2 N1024 24.0 -> 19.5 us, H12 28.8 -> 25.9, N576 H12 25.6 -> 19.6, N200 H12
+// 21.7 -> 14.8; NVFP4 (six launches) N1024 H12 37.3 -> 30.7, N200 H12 27.9 -> 18.3.  What bounds it: latency. Tables 1.5 to
+// 2.5 us (hidden when calls follow one another), rows 1.5, column sums 2, barrier 0.8, fold 1, codes 2.
+struct Short {
+  double theta, n;           // n: tokens
+  unsigned int* status;
+};
+enum { kShortK = 0, kShortV = 1, kShortQ = 2 };
+// Blocks of a head at most: the CTAs of a portable cluster.  (Clusters of 16 find room on few GPCs at a time: B1 H6 N1955
+// d64 35.1 us instead of 27.7 when calls follow one another.  Two blocks a CTA in clusters of 8: 27.7, no gain.)
+constexpr int kShortCluster = 8;
+constexpr int kShortEntries = 1408;    // RoPE table entries at most: at d128 two CTAs stay on an SM
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// The word at `p` of this CTA's shared memory, in the CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_word(const void* p, int rank) {
+  uint32_t at, v;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+// x / n, correctly rounded, with inv = 1 / n already at hand: a quotient within an ulp and one correction by its exact
+// remainder (Markstein's theorem), three operations in place of a division behind the sums.
+__device__ __forceinline__ double divided(double x, double n, double inv) {
+  const double q = x * inv;
+  return isfinite(q) ? fma(fma(-q, n, x), inv, q) : q;
+}
+
+template <int D> struct ShortSmem {
+  static constexpr int tile = 2 * Geo<D>::stage_bytes;     // behind the rows, in place and gathered: codes [128 x D]
+  static constexpr int red = tile + kBlock * D;            // 8 D floats
+  static constexpr int part = red + 8 * D * 4;             // column sums or value maxima [D]
+  static constexpr int pm = part + D * 4;                  // (m+, m-) pairs [D]
+  static constexpr int qred = pm + D * 4;                  // [2][8] floats, the head maximum
+  static constexpr int src = qred + 80;                    // source rows [128]
+  static constexpr int freq = src + kBlock * 4;            // [D / 2] doubles
+  static constexpr int plain = freq + D / 2 * 8;           // the tables
+  static constexpr size_t bytes(int entries) { return (size_t)plain + 16 * (size_t)entries; }
+};
+
+// Source of row t of a block: the gather by `perm` (clamped: never a bad address), -1 behind the last token.
+__device__ __forceinline__ int source_row(const PrepArgs& a, const int32_t* perm, int blk, int t) {
+  const int pos = blk * kBlock + t;
+  return pos >= a.N ? -1 : (perm ? min(max(__ldg(perm + pos), 0), a.N - 1) : pos);
+}
+// 128 threads (t) copy the rows of a block; `mine` is the source of row t.  The lanes of a warp fetch its 32 rows 16 bytes at a time.
+template <int D>
+__device__ __forceinline__ void fetch_block(const PrepArgs& a, const char* head, int mine, int pitch, unsigned char* dst, int t) {
+  constexpr int LPR = D / 8, RPI = 32 / LPR;
+  const int lane = t & 31;
+  dst += (t & ~31) * pitch + (lane / LPR) * pitch + 16 * (lane % LPR);
+  head += 16 * (lane % LPR);
+#pragma unroll
+  for (int k = 0; k < 32 / RPI; ++k) {
+    const int sr = __shfl_sync(0xffffffffu, mine, k * RPI + lane / LPR);
+    if (sr >= 0) cp_async16(dst + k * RPI * pitch, head + (int64_t)sr * a.stride_n_bytes);
+  }
+}
+
+template <int D, int BITS, int VARIANT>
+__global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs a, const Short s) {
+  using L = ShortSmem<D>;
+  constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
+  constexpr int kRowBytes = BITS == 4 ? D / 2 : D;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int group = blockIdx.x / a.nb, blk = blockIdx.x - group * a.nb;  // (a cluster is a group: blk is the rank in it)
+  const int kind = group / a.BH, bh = group - kind * a.BH;
+  const bool full = a.N - blk * kBlock >= kBlock;
+  float* part = reinterpret_cast<float*>(smem + L::part);
+  const int64_t head = head_offset_bytes(a, bh);
+  const int32_t* perm = a.perm ? a.perm + (size_t)bh * a.N : nullptr;
+
+  if (kind == kShortV) {
+    unsigned int* amax = reinterpret_cast<unsigned int*>(part);
+    float* red = reinterpret_cast<float*>(smem + kBlock * 2 * D);          // 16 D floats, behind the value tile
+    if (tid < D) amax[tid] = 0u;
+    pdl_wait();
+    if (warp >= 4) {
+      fetch_block<D>(a, reinterpret_cast<const char*>(a.v) + head, source_row(a, perm, blk, tid - 128), 2 * D, smem, tid - 128);
+      cp_async_commit();
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    pdl_allow();
+    const int cp = tid % (D / 2);
+    float2 am = make_float2(0.f, 0.f), mu = am;
+    if constexpr (BITS == 8) {
+      if (full) v_stats_item<D, true>(a, smem, red, bh, blk, amax);
+      else v_stats_item<D, false>(a, smem, red, bh, blk, amax);
+      cluster_arrive();
+      cluster_wait();
+      mu = *reinterpret_cast<const float2*>(a.v_mu + ((size_t)bh * a.nb + blk) * D + 2 * cp);
+      unsigned int m0 = 0u, m1 = 0u;
+#pragma unroll
+      for (int r = 0; r < kShortCluster; ++r) {
+        if (r >= a.nb) break;
+        m0 = max(m0, peer_word(amax + 2 * cp, r));
+        m1 = max(m1, peer_word(amax + 2 * cp + 1, r));
+      }
+      cluster_arrive();                       // (this CTA has read its peers)
+      am = make_float2(__uint_as_float(m0), __uint_as_float(m1));
+      if (blk == 0 && tid < D / 2) *reinterpret_cast<uint2*>(a.v_amax + (size_t)bh * D + 2 * cp) = make_uint2(m0, m1);
+    }
+    if (blk == 0 && tid < D / 2)
+      *reinterpret_cast<float2*>(a.v_scale + (size_t)bh * D + 2 * cp) = BITS == 8 ? make_float2(value_scale(am.x), value_scale(am.y)) : make_float2(1.0f, 1.0f);
+    constexpr int kV = BITS == 8 ? kVQuant8 : (VARIANT ? kVQuant4M : kVQuant4);
+    if (full) v_item<D, kV, true>(a, smem, red, bh, blk, mu, am);
+    else v_item<D, kV, false>(a, smem, red, bh, blk, mu, am);
+    if constexpr (BITS == 8) cluster_wait();  // a CTA stays until its peers have read it
+    return;
+  }
+
+  // ---- Q and K: the tables (warps 0 to 3) while the rows are on their way (warps 4 to 7)
+  const int tensor = kind == kShortK ? 1 : 0;
+  const bool smooth = tensor == 1 && (a.flags & VC_FLAG_K_SMOOTH), gather = tensor == 1 && perm;
+  unsigned char *in_place = smem, *gathered = gather ? smem + Geo<D>::stage_bytes : smem, *out_tile = smem + L::tile;
+  float *red = reinterpret_cast<float*>(smem + L::red), *pm = reinterpret_cast<float*>(smem + L::pm), *qred = reinterpret_cast<float*>(smem + L::qred);
+  unsigned int* amax = reinterpret_cast<unsigned int*>(qred + 16);
+  int* src = reinterpret_cast<int*>(smem + L::src);
+  float2 *plain = reinterpret_cast<float2*>(smem + L::plain), *folded = plain + a.rd.entries;
+  double inv_n = 0.0;
+  if (warp < 4) {
+    double* freq = reinterpret_cast<double*>(smem + L::freq);
+    if (tid < D / 2) {
+      const int ax = tid >= a.rd.pair_start[2] ? 2 : (tid >= a.rd.pair_start[1] ? 1 : 0);
+      freq[tid] = rope_freq(s.theta, tid - a.rd.pair_start[ax], a.rd.pairs[ax]);
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll 1
+    for (int e = tid; e < a.rd.entries; e += 128) {
+      const int ax = e >= a.rd.off[2] ? 2 : (e >= a.rd.off[1] ? 1 : 0);
+      const int pos = (e - a.rd.off[ax]) / a.rd.pairs[ax], i = e - a.rd.off[ax] - pos * a.rd.pairs[ax];
+      rope_entry_of(pos, freq[a.rd.pair_start[ax] + i], plain + e, folded + e);
+    }
+    if (tid < D) pm[tid] = 0.f;
+    if (tid == 0) *amax = 0u;
+    inv_n = 1.0 / s.n;
+    pdl_wait();
+  } else {
+    pdl_wait();
+    const char* x = reinterpret_cast<const char*>(tensor ? a.k : a.q) + head;
+    const int t = tid - 128, from = source_row(a, tensor ? perm : nullptr, blk, t);      // (asked for first: the copies in place cover the round trip)
+    if (!gather || smooth || BITS == 4) fetch_block<D>(a, x, source_row(a, nullptr, blk, t), Geo<D>::pitch, in_place, t);
+    cp_async_commit();
+    src[t] = from;
+    if (gather) fetch_block<D>(a, x, from, Geo<D>::pitch, gathered, t);
+    cp_async_commit();
+    cp_async_wait<1>();
+  }
+  constexpr int LPR = D / 8, RPL = LPR / 2;   // (a lane's place in the column sums)
+  const int lr = lane % LPR, hb = lane / LPR;
+  const PairSlots ps = pair_slots(a.rd, 4 * lr);
+  __syncthreads();
+  pdl_allow();
+  if (blockIdx.x == 0 && tid == 0) *s.status = 0u;
+
+  const int my_row = qk_row_of(tid), row0 = warp * (32 / kTpr);
+  if (tensor == 1) {
+    if (smooth) {
+      const RopeTab tab{smem_u32(plain), nullptr};
+      k_colsum_item<D>(a, in_place + (16 * warp + RPL * hb) * Geo<D>::pitch + 16 * lr, Geo<D>::pitch, red, tab, ps, part, blk);
+    }
+    cp_async_wait<0>();
+    cluster_arrive();
+    cluster_wait();
+    if (tid < D) {                            // the sums of the head's blocks, as the finalization launch adds them
+      double sum = 0.0;
+      if (smooth) {
+        float p[kShortCluster];               // (all asked for, then added)
+#pragma unroll
+        for (int j = 0; j < kShortCluster; ++j) p[j] = j < a.nb ? __uint_as_float(peer_word(part + tid, j)) : 0.f;
+#pragma unroll
+        for (int j = 0; j < kShortCluster; ++j) sum += (double)p[j];
+      }
+      red[tid] = (float)divided(sum, s.n, inv_n);
+      if (blk == 0) a.k_mean[(size_t)bh * D + tid] = red[tid];
+    }
+    cluster_arrive();
+    __syncthreads();
+    if (smooth && tid < D / 2) *reinterpret_cast<float2*>(pm + 2 * tid) = make_float2(red[2 * tid] + red[2 * tid + 1], red[2 * tid] - red[2 * tid + 1]);
+    __syncthreads();
+    if constexpr (BITS == 4) cluster_wait();
+  }
+  float outer = 0.f;
+  if constexpr (BITS == 4) {                  // the head maximum, over the rows in place
+    const int pos = blk * kBlock + my_row;
+    qk_row_item_fast<D, kStageAmax>(a, tensor, in_place, out_tile, qred, pm, smem_u32(folded), bh, blk, 0, false, pos < a.N ? pos : -1, amax, 0.f);
+    cluster_arrive();
+    cluster_wait();
+    outer = outer_scale(__uint_as_float(__reduce_max_sync(0xffffffffu, lane < a.nb ? peer_word(amax, lane) : 0u)));
+    cluster_arrive();
+    if (blk == 0 && tid == 0) (tensor ? a.k_scale : a.q_scale)[bh] = outer;
+  }
+  qk_row_item_fast<D, kQuant>(a, tensor, gathered, out_tile, qred, pm, smem_u32(folded), bh, blk, 1, false, src[my_row], nullptr, outer);
+  __syncwarp();                               // the warp's rows of the code tile are complete
+  store_warp_rows<kRowBytes>((tensor ? a.k_codes : a.q_codes) + ((size_t)bh * a.n_pad + (size_t)blk * kBlock) * kRowBytes, out_tile, row0, lane);
+  if (BITS == 4 || tensor == 1) cluster_wait();       // a CTA stays until its peers have read it
+}
+
+// Which calls take it: heads of at most eight blocks whose CTAs are resident at once at 8 bits (two per SM), or in two
+// waves at 4 bits, where two more launches fall away.  Beyond, a launch per phase whose CTAs prefetch their next blocks
+// is faster: FP8 d128 N576 H24 (432 CTAs in clusters of 8) 31.9 us against 27.0, NVFP4 H40 55.9 against 50.1; N1024 NVFP4 H24
+// (576 CTAs) 43.3 against 48.8, FP8 H18 (432) 30.0 against 30.0.
+inline bool short_heads(const Problem& pr, const PrepArgs& a) {
+  return pr.nb <= kShortCluster && a.rd.entries <= kShortEntries && !(pr.flags & VC_FLAG_CHECK_PERM) && 3 * pr.BH * pr.nb <= (pr.bits == 8 ? 2 : 4) * sm_count();
+}
+template <int D, int BITS, int VARIANT>
+cudaError_t run_short(const PrepArgs& a, const Short& s, cudaStream_t stream) {
+  constexpr auto kernel = prep_short_kernel<D, BITS, VARIANT>;
+  cudaError_t e = allow_smem<kernel>();
+  if (e == cudaSuccess)
+    e = launch_clusters(kernel, dim3((unsigned)(3 * a.BH * a.nb)), a.nb, kThreads, ShortSmem<D>::bytes(a.rd.entries), stream, a, s);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
+  return cudaGetLastError();
+}
+template <int D, int BITS>
+cudaError_t run_short(const Problem& pr, const PrepArgs& a, const Short& s, cudaStream_t stream) {
+  const bool variant = BITS == 8 ? (a.flags & VC_FLAG_INT8_QK) != 0 : hybrid4(pr);
+  return variant ? run_short<D, BITS, 1>(a, s, stream) : run_short<D, BITS, 0>(a, s, stream);
+}
+
+// The packed row transform serves the standard configuration.
+inline bool fast_rows(const PrepArgs& a) {
+  return (a.flags & VC_FLAG_ROPE) && (a.flags & VC_FLAG_HADAMARD) && a.rope_default && a.rope_in_smem;
+}
+
 template <int D, int BITS>
 cudaError_t run(const Problem& pr, const PrepArgs& a, cudaStream_t s) {
-  // the packed row transform serves the standard configuration
-  const bool fast = (a.flags & VC_FLAG_ROPE) && (a.flags & VC_FLAG_HADAMARD) && a.rope_default && a.rope_in_smem;
   const bool variant = BITS == 8 ? (a.flags & VC_FLAG_INT8_QK) != 0 : hybrid4(pr);
-  if (fast) return variant ? run_phases<D, BITS, true, 1>(pr, a, s) : run_phases<D, BITS, true, 0>(pr, a, s);
+  if (fast_rows(a)) return variant ? run_phases<D, BITS, true, 1>(pr, a, s) : run_phases<D, BITS, true, 0>(pr, a, s);
   return variant ? run_phases<D, BITS, false, 1>(pr, a, s) : run_phases<D, BITS, false, 0>(pr, a, s);
 }
 
@@ -1405,7 +1659,7 @@ cudaError_t run(const Problem& pr, const PrepArgs& a, cudaStream_t s) {
 
 cudaError_t launch_prep(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
                         const void* q, const void* k, const void* v, const int32_t* perm,
-                        uint8_t* quant, uint8_t* work, cudaStream_t stream, const vc_prep_stats* stats) {
+                        uint8_t* quant, uint8_t* work, cudaStream_t stream, const vc_prep_stats* stats, bool then_attention) {
   PrepArgs a{};
   a.q = (const __nv_bfloat16*)q; a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
   a.perm = perm;
@@ -1445,6 +1699,11 @@ cudaError_t launch_prep(const Problem& pr, const QuantLayout& ql, const WorkLayo
   {
     const int sdef = 2 * (pr.d / 6);
     a.rope_default = pr.rope_dim[0] == pr.d - 2 * sdef && pr.rope_dim[1] == sdef && pr.rope_dim[2] == sdef;
+  }
+  if (then_attention && !ext && fast_rows(a) && short_heads(pr, a)) {
+    const Short s{(double)pr.rope_theta, (double)pr.N, reinterpret_cast<unsigned int*>(work + wl.status)};
+    if (pr.d == 128) return pr.bits == 8 ? run_short<128, 8>(pr, a, s, stream) : run_short<128, 4>(pr, a, s, stream);
+    return pr.bits == 8 ? run_short<64, 8>(pr, a, s, stream) : run_short<64, 4>(pr, a, s, stream);
   }
   // the table (one thread per entry), the words that start at zero, supplied statistics
   SetUp u{};
@@ -1519,6 +1778,6 @@ extern "C" vc_status vc_prep_noalloc(const vc_params* p, const void* q, const vo
   unsigned char* scratch = nullptr;
   if (scratch_address(&scratch) != cudaSuccess) return VC_ERR_CUDA;
   // launch_prep clears the words that must start at zero (status, amax) on the stream itself
-  cudaError_t e = vc::launch_prep(pr, ql, wl, q, k, v, perm, (uint8_t*)quant, scratch, (cudaStream_t)stream, nullptr);
+  cudaError_t e = vc::launch_prep(pr, ql, wl, q, k, v, perm, (uint8_t*)quant, scratch, (cudaStream_t)stream, nullptr, false);
   return e == cudaSuccess ? VC_OK : VC_ERR_CUDA;
 }
