@@ -449,7 +449,8 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 
   if constexpr (STAGE == kStageQuant4) {
     // NVFP4: outer scale g per (b, h), microscale per token per 16 channels
-    const float g = (TENSOR == 0 ? a.q_scale : a.k_scale)[bh];
+    const float g = outer_scale(__uint_as_float(*amax_at));
+    if (tid == 0 && blk == 0) (TENSOR == 0 ? a.q_scale : a.k_scale)[bh] = g;
     const float inv6 = 1.0f / (6.0f * g);
     constexpr int MB = C / 16;                   // microscale bytes of this thread
     unsigned int codes[C / 8], micro[(MB + 3) / 4];
@@ -503,12 +504,12 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 //    operation per lane, one instruction issued for two);
 //  * at 8 bits 1 / sqrt(D) and the quantization scale are one factor.
 // The 4-bit head-maximum and NVFP4 stages run on the same transform.
-// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed; `outer` is the head's NVFP4
-// scale, `amax_at` where the head maximum is collected.
+// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed; `amax_at`: where the head maximum
+// is collected, and at 4 bits taken from (the outer scale follows from it, one of the head's blocks stores it).
 template <int D, int STAGE>
 __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TENSOR, const unsigned char* stage,
                                                  unsigned char* out_tile, float* red, float* kmean_pm, uint32_t tab_saddr,
-                                                 int bh, int blk, int iter, bool new_head, int src_row, unsigned int* amax_at, float outer) {
+                                                 int bh, int blk, int iter, bool new_head, int src_row, unsigned int* amax_at) {
   constexpr int C = D / kTpr, P = C / 2;           // channels and pairs per thread
   constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -612,7 +613,8 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
   if constexpr (STAGE == kStageQuant4) {
     // NVFP4: outer scale g per (b, h), microscale per token per 16 channels (the arithmetic of the
     // general row body: y = x / sqrt(D), then y / (g * microscale), each rounded once)
-    const float g = outer;
+    const float g = outer_scale(__uint_as_float(*amax_at));
+    if (tid == 0 && blk == 0) (TENSOR == 0 ? a.q_scale : a.k_scale)[bh] = g;
     const float inv6 = 1.0f / (6.0f * g);
     const uint64_t RS = pack_f32x2(rs, rs);
     constexpr int MB = C / 16;                     // microscale bytes of this thread
@@ -1086,33 +1088,27 @@ __device__ __forceinline__ void v_pass(const PrepArgs& a, unsigned char* smem, c
   }
 }
 
-// Per-head finalization: K channel mean, V scale, g_Q.
+// Per-head finalization: K channel mean, V scale.  A block of 8 D threads per head; the block partial sums are added in
+// double, in eight interleaved slices that are then added in a fixed order.
 template <int D, int BITS>
-__global__ void prep_finalize_kernel(const PrepArgs a, int which) {
-  // which 0: a block of 8 D threads per head; the block partial sums are added in double, in eight
-  // interleaved slices that are then added in a fixed order.  which 1 (4 bits): the outer scale of K.
+__global__ void prep_finalize_kernel(const PrepArgs a) {
   __shared__ double part[8][D];
   const int bh = a.bh0 + blockIdx.x, c = threadIdx.x % D, slice = threadIdx.x / D;
   pdl_wait();
   pdl_allow();
-  if (which == 0) {
-    if (a.flags & VC_FLAG_K_SMOOTH) {
-      double s = 0.0;
+  if (a.flags & VC_FLAG_K_SMOOTH) {
+    double s = 0.0;
 #pragma unroll 8
-      for (int j = slice; j < a.nb; j += 8) s += (double)a.k_part[((size_t)bh * a.nb + j) * D + c];
-      part[slice][c] = s;
-      __syncthreads();
-    }
-    if (slice == 0) {
-      double s = 0.0;
-      if (a.flags & VC_FLAG_K_SMOOTH)
-        for (int k = 0; k < 8; ++k) s += part[k][c];
-      a.k_mean[(size_t)bh * D + c] = (float)(s / (double)a.N);
-      a.v_scale[(size_t)bh * D + c] = BITS == 8 ? value_scale(__uint_as_float(a.v_amax[(size_t)bh * D + c])) : 1.0f;
-    }
-    if (BITS == 4 && threadIdx.x == 0) a.q_scale[bh] = outer_scale(__uint_as_float(a.qk_amax[bh]));
-  } else if (BITS == 4 && threadIdx.x == 0) {
-    a.k_scale[bh] = outer_scale(__uint_as_float(a.qk_amax[a.BH + bh]));
+    for (int j = slice; j < a.nb; j += 8) s += (double)a.k_part[((size_t)bh * a.nb + j) * D + c];
+    part[slice][c] = s;
+    __syncthreads();
+  }
+  if (slice == 0) {
+    double s = 0.0;
+    if (a.flags & VC_FLAG_K_SMOOTH)
+      for (int k = 0; k < 8; ++k) s += part[k][c];
+    a.k_mean[(size_t)bh * D + c] = (float)(s / (double)a.N);
+    a.v_scale[(size_t)bh * D + c] = BITS == 8 ? value_scale(__uint_as_float(a.v_amax[(size_t)bh * D + c])) : 1.0f;
   }
 }
 
@@ -1203,8 +1199,7 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
     const int tensor = c0.z + z0, bh = a.bh0 + c0.hh;
     unsigned int* amax_at = a.qk_amax + tensor * a.BH + bh;
     if constexpr (FAST)
-      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at,
-                                 STAGE == kStageQuant4 ? (tensor == 0 ? a.q_scale : a.k_scale)[bh] : 0.f);
+      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at);
     else
       qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at);
     if (tensor == 1) last_hh = c0.hh;
@@ -1371,8 +1366,8 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     const int per = pr.nb * nh;
     a.bh0 = bh0;
     const int sums = a.flags & VC_FLAG_K_SMOOTH ? per : 0;
-    auto finalize = [&](int which, int threads) {
-      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
+    auto finalize = [&]() {
+      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), 8 * D, 0, s, a);
       count_launches(1);
     };
     auto launch = [&](auto whole, auto in_turns, size_t bytes, Work w0, Work w1, Work w2, int z0) {
@@ -1387,7 +1382,7 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
                  second = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, second_turns = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>;
       if (!ext) {
         launch(first, first_turns, wide ? rest_smem : smem, wide ? none : rows, k_sums, v_stats, 0);
-        finalize(0, 8 * D);
+        finalize();
       }
       // (with supplied statistics there is no first launch for Q to share; on a wide grid it does not share one)
       const bool q_too = ext || wide;
@@ -1399,9 +1394,9 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
                  third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>;
       launch(first, first_turns, wide ? rest_smem : smem, wide ? none : amax, k_sums, v_codes4, 0);
       if (wide) launch(first, first_turns, row_smem, amax, none, none, 0);
-      finalize(0, 8 * D);
+      finalize();
       launch(second, second_turns, smem, rows, amax, none, 0);
-      finalize(1, 32);
+      // (the outer scale of K follows from its head maximum where the codes are made: a launch of its own was 2 us)
       launch(third, third, smem, rows, none, none, 1);
     }
   }
@@ -1411,7 +1406,7 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
 // ---------------------------------------------------------------------------------------
 // Short heads in front of an attention launch: the whole pass in one launch, a cluster of CTAs per head and tensor, a CTA
 // per block.  Few blocks keep the GPU busy for a few microseconds, and what the pass then costs is its chain of
-// launches: table, statistics, finalization, codes, at 4 bits two more, 0.8 to 1.5 us from the end of each to the start of
+// launches: table, statistics, finalization, codes, at 4 bits one more, 0.8 to 1.5 us from the end of each to the start of
 // the next beside its own filling of a pipeline (13.2 us from the table's start to the attention's at B1 H2 N1024 d128).  Here
 //   - every CTA computes the RoPE tables it needs itself, in front of the wait for the kernel before it;
 //   - a CTA keeps its block in shared memory, so K and V are read once and the statistics of a head meet in distributed
@@ -1453,7 +1448,7 @@ template <int D> struct ShortSmem {
   static constexpr int red = tile + kBlock * D;            // 8 D floats
   static constexpr int part = red + 8 * D * 4;             // column sums or value maxima [D]
   static constexpr int pm = part + D * 4;                  // (m+, m-) pairs [D]
-  static constexpr int qred = pm + D * 4;                  // [2][8] floats, the head maximum
+  static constexpr int qred = pm + D * 4;                  // [2][8] floats, the block's and the head's maximum
   static constexpr int src = qred + 80;                    // source rows [128]
   static constexpr int freq = src + kBlock * 4;            // [D / 2] doubles
   static constexpr int plain = freq + D / 2 * 8;           // the tables
@@ -1604,24 +1599,24 @@ __global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs 
     __syncthreads();
     if constexpr (BITS == 4) cluster_wait();
   }
-  float outer = 0.f;
   if constexpr (BITS == 4) {                  // the head maximum, over the rows in place
     const int pos = blk * kBlock + my_row;
-    qk_row_item_fast<D, kStageAmax>(a, tensor, in_place, out_tile, qred, pm, smem_u32(folded), bh, blk, 0, false, pos < a.N ? pos : -1, amax, 0.f);
+    qk_row_item_fast<D, kStageAmax>(a, tensor, in_place, out_tile, qred, pm, smem_u32(folded), bh, blk, 0, false, pos < a.N ? pos : -1, amax);
     cluster_arrive();
     cluster_wait();
-    outer = outer_scale(__uint_as_float(__reduce_max_sync(0xffffffffu, lane < a.nb ? peer_word(amax, lane) : 0u)));
+    const unsigned int most = __reduce_max_sync(0xffffffffu, lane < a.nb ? peer_word(amax, lane) : 0u);
     cluster_arrive();
-    if (blk == 0 && tid == 0) (tensor ? a.k_scale : a.q_scale)[bh] = outer;
+    if (tid == 0) amax[1] = most;
+    __syncthreads();
   }
-  qk_row_item_fast<D, kQuant>(a, tensor, gathered, out_tile, qred, pm, smem_u32(folded), bh, blk, 1, false, src[my_row], nullptr, outer);
+  qk_row_item_fast<D, kQuant>(a, tensor, gathered, out_tile, qred, pm, smem_u32(folded), bh, blk, 1, false, src[my_row], amax + 1);
   __syncwarp();                               // the warp's rows of the code tile are complete
   store_warp_rows<kRowBytes>((tensor ? a.k_codes : a.q_codes) + ((size_t)bh * a.n_pad + (size_t)blk * kBlock) * kRowBytes, out_tile, row0, lane);
   if (BITS == 4 || tensor == 1) cluster_wait();       // a CTA stays until its peers have read it
 }
 
 // Which calls take it: heads of at most eight blocks whose CTAs are resident at once at 8 bits (two per SM), or in two
-// waves at 4 bits, where two more launches fall away.  Beyond, a launch per phase whose CTAs prefetch their next blocks
+// waves at 4 bits, where one more launch falls away.  Beyond, a launch per phase whose CTAs prefetch their next blocks
 // is faster: FP8 d128 N576 H24 (432 CTAs in clusters of 8) 31.9 us against 27.0, NVFP4 H40 55.9 against 50.1; N1024 NVFP4 H24
 // (576 CTAs) 43.3 against 48.8, FP8 H18 (432) 30.0 against 30.0.
 inline bool short_heads(const Problem& pr, const PrepArgs& a) {
