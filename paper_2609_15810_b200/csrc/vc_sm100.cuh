@@ -393,6 +393,19 @@ __device__ __forceinline__ uint32_t cvt_e2m1x8(float v0, float v1, float v2, flo
       : "f"(v0), "f"(v1), "f"(v2), "f"(v3), "f"(v4), "f"(v5), "f"(v6), "f"(v7));
   return out;
 }
+// The same with negative values taken as zero.
+__device__ __forceinline__ uint32_t cvt_relu_e2m1x8(float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7) {
+  uint32_t out;
+  asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b0, %2, %1;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b1, %4, %3;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b2, %6, %5;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b3, %8, %7;\n\t"
+      "mov.b32 %0, {b0, b1, b2, b3};\n\t}"
+      : "=r"(out)
+      : "f"(v0), "f"(v1), "f"(v2), "f"(v3), "f"(v4), "f"(v5), "f"(v6), "f"(v7));
+  return out;
+}
 __device__ __forceinline__ float lg2_approx(float x) {
   float d;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(x));
