@@ -107,7 +107,9 @@ typedef struct {
   float rope_theta;                 /* 0 => 10000                                       */
   int64_t stride_b, stride_h, stride_n;       /* of Q, K and V, in elements; 0 => packed; stride_n < 2^30 */
   int32_t heads_per_pass;           /* heads preprocessed per launch group (L2 reuse of
-                                       the second read of K and V); 0 => library default */
+                                       the second read of K and V); 0 => library default.
+                                       vc_attn may prepare heads of up to 1024 tokens in
+                                       one launch, whatever it says                     */
   int32_t kernel_variant;           /* attention kernel: 0 = pipelined, two query tiles per
                                        CTA (default); 1 = simple serial kernel, kept for
                                        A/B measurement and cross-checks                  */
