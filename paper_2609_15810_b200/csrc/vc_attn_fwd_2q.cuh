@@ -23,7 +23,7 @@ using namespace attn;
 //   * The probability codes have tensor-memory columns of their own (32 per tile) and are the A operand
 //     of the value product there, so a score tile is free as soon as its 128 x 128 values are in
 //     registers.  At d = 128 one score buffer serves both query tiles in turn (all that tensor memory
-//     has room for); at d = 64 each tile has its own.  (An MMA with both operands in shared memory reads
+//     has room for); at d = 64 each tile has its own, but for kSfu.  (An MMA with both operands in shared memory reads
 //     128 bytes a clock, all a shared-memory port gives.  With the codes there as well, 32 KB written and
 //     32 KB read per pair of tiles, every copy and store slowed the products down: B2 H16 N16384 d64
 //     1956 -> 1870 us, B1 H12 N32760 d128 without value smoothing 3677 -> 3604, B1 H40 12.49 -> 12.33 ms
@@ -89,9 +89,14 @@ template <int D, int PF, bool INT8, bool SMOOTH, bool TWO>
 __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                              const AttnArgs& a, const int q0, const int bh) {
   constexpr int kTmemCols = 512;
+  // exponentials of the special-function unit: a softmax warp then waits for that unit, which the warp of the other
+  // query tile wants too, and the two run better out of step and with results that leave a few at a time
+  constexpr bool kSfu = PF == kPfExp || PF == kPfExpMix;
   // d = 64 leaves room in tensor memory for a score buffer per query tile (B2 H16 N16384 d64: 1.89 -> 1.83 ms,
-  // without smoothing 1.85 -> 1.76); at d = 128 both tiles share one
-  constexpr bool kTwoS = D == 64;
+  // without smoothing 1.85 -> 1.76); at d = 128 both tiles share one, and with kSfu as well, because the shared
+  // buffer is what keeps the two tiles out of step (B1 H16 N16384 d64, exponentials of E4M3 scores 1593 -> 1461 us, of
+  // INT8 scores 1793 -> 1611, three of four by the unit 1523 -> 1494; all by polynomial 3004 -> 3033, so that one keeps two)
+  constexpr bool kTwoS = D == 64 && !kSfu;
   constexpr uint32_t O_COL = kTwoS ? 256 : 128, O_STRIDE = D + 16, L_COL = D, S1_COL = kTwoS ? 128 : O_COL + O_STRIDE, P_COL = 416;   // A_t at O_COL + t * O_STRIDE; l in its column d
   // Register re-partition (setmaxnreg): the CTA owns 640 x 96 registers; a warpgroup that asks for
   // more than the others released would block forever, so the budget is checked at compile time.
@@ -347,10 +352,18 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
       };
       const uint32_t p_col = lane_base + P_COL + 32 * buf(t, j);
       auto store32 = [&](const uint32_t (&sv)[32], int q) {                 // keys 32 q .. + 31
-        uint32_t c[8];
+        if constexpr (kSfu) {
+          // Four columns a store: with eight, 32 exponentials have to be done before any code leaves (B1 H16 N16384
+          // d128, E4M3 / INT8 scores 1639 / 1801 us with eight, 1489 / 1683 with four, 1526 / 1718 with two; codes through
+          // shared memory 1582 / 1773).  Without the unit eight are as good or better.
 #pragma unroll
-        for (int w = 0; w < 8; ++w) c[w] = code4(sv, w);
-        tmem_st8(p_col + 8 * q, c);
+          for (int w = 0; w < 8; w += 4) tmem_st4(p_col + 8 * q + w, code4(sv, w), code4(sv, w + 1), code4(sv, w + 2), code4(sv, w + 3));
+        } else {
+          uint32_t c[8];
+#pragma unroll
+          for (int w = 0; w < 8; ++w) c[w] = code4(sv, w);
+          tmem_st8(p_col + 8 * q, c);
+        }
       };
       tc_fence_after();
       store32(s0, 0); store32(s1, 1); store32(s2, 2); store32(s3, 3);
