@@ -294,10 +294,10 @@ template <int D> __device__ __forceinline__ constexpr int rope_axis_of(int p) {
   return p < RopeSplit<D>::p1 ? 0 : (p < RopeSplit<D>::p2 ? 1 : 2);
 }
 
-template <int D, int STAGE>
+template <int D, int STAGE, typename AmaxAt, typename Outer>
 __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR /*0 = Q, 1 = K*/, const unsigned char* stage,
                                             unsigned char* out_tile, float* red, float* kmean_s, const RopeTab& tab, int bh,
-                                            int blk, int iter, bool new_head, int src_row, unsigned int* amax_at) {
+                                            int blk, int iter, bool new_head, int src_row, AmaxAt amax_at, Outer outer) {
   constexpr int C = D / kTpr;                      // channels per thread
   constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -410,7 +410,7 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
     amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
-    if (tid == 0) atomicMax(amax_at, __float_as_uint(amax));
+    if (tid == 0) atomicMax(amax_at(), __float_as_uint(amax));
     return;
   }
   const size_t row_g = (size_t)bh * a.n_pad + (size_t)blk * kBlock + row;
@@ -449,8 +449,7 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 
   if constexpr (STAGE == kStageQuant4) {
     // NVFP4: outer scale g per (b, h), microscale per token per 16 channels
-    const float g = outer_scale(__uint_as_float(*amax_at));
-    if (tid == 0 && blk == 0) (TENSOR == 0 ? a.q_scale : a.k_scale)[bh] = g;
+    const float g = outer();
     const float inv6 = 1.0f / (6.0f * g);
     constexpr int MB = C / 16;                   // microscale bytes of this thread
     unsigned int codes[C / 8], micro[(MB + 3) / 4];
@@ -504,12 +503,13 @@ __device__ __forceinline__ void qk_row_item(const PrepArgs& a, const int TENSOR 
 //    operation per lane, one instruction issued for two);
 //  * at 8 bits 1 / sqrt(D) and the quantization scale are one factor.
 // The 4-bit head-maximum and NVFP4 stages run on the same transform.
-// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed; `amax_at`: where the head maximum
-// is collected, and at 4 bits taken from (the outer scale follows from it, one of the head's blocks stores it).
-template <int D, int STAGE>
+// `kmean_pm` holds (m+, m-) per pair, zeros while Q rows or unsmoothed K rows are processed.  `amax_at()`: where the head
+// maximum is collected; `outer()`: the head's NVFP4 outer scale.  (Functions, and not values: a pointer that lives through the item
+// costs the general row body spills, B1 H24 N118800 d128 without RoPE 1429 -> 1500 us.)
+template <int D, int STAGE, typename AmaxAt, typename Outer>
 __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TENSOR, const unsigned char* stage,
                                                  unsigned char* out_tile, float* red, float* kmean_pm, uint32_t tab_saddr,
-                                                 int bh, int blk, int iter, bool new_head, int src_row, unsigned int* amax_at) {
+                                                 int bh, int blk, int iter, bool new_head, int src_row, AmaxAt amax_at, Outer outer) {
   constexpr int C = D / kTpr, P = C / 2;           // channels and pairs per thread
   constexpr int NT = kRowThreads * kTpr;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -607,14 +607,13 @@ __device__ __forceinline__ void qk_row_item_fast(const PrepArgs& a, const int TE
     amax = fmaxf(amax, fmaxf(fmaxf(rbuf[4], rbuf[5]), fmaxf(rbuf[6], rbuf[7])));
   }
   if constexpr (STAGE == kStageAmax) {
-    if (tid == 0) atomicMax(amax_at, __float_as_uint(amax));
+    if (tid == 0) atomicMax(amax_at(), __float_as_uint(amax));
     return;
   }
   if constexpr (STAGE == kStageQuant4) {
     // NVFP4: outer scale g per (b, h), microscale per token per 16 channels (the arithmetic of the
     // general row body: y = x / sqrt(D), then y / (g * microscale), each rounded once)
-    const float g = outer_scale(__uint_as_float(*amax_at));
-    if (tid == 0 && blk == 0) (TENSOR == 0 ? a.q_scale : a.k_scale)[bh] = g;
+    const float g = outer();
     const float inv6 = 1.0f / (6.0f * g);
     const uint64_t RS = pack_f32x2(rs, rs);
     constexpr int MB = C / 16;                     // microscale bytes of this thread
@@ -1088,14 +1087,17 @@ __device__ __forceinline__ void v_pass(const PrepArgs& a, unsigned char* smem, c
   }
 }
 
-// Per-head finalization: K channel mean, V scale.  A block of 8 D threads per head; the block partial sums are added in
-// double, in eight interleaved slices that are then added in a fixed order.
+// Per-head finalization.  which 0: K channel mean, V scale, at 4 bits the outer scale of Q; a block of 8 D threads per head, the
+// block partial sums are added in double, in eight interleaved slices that are then added in a fixed order.
+// which 1 (4 bits): the outer scale of K.
 template <int D, int BITS>
-__global__ void prep_finalize_kernel(const PrepArgs a) {
+__global__ void prep_finalize_kernel(const PrepArgs a, int which) {
   __shared__ double part[8][D];
   const int bh = a.bh0 + blockIdx.x, c = threadIdx.x % D, slice = threadIdx.x / D;
   pdl_wait();
   pdl_allow();
+  if (BITS == 4 && threadIdx.x == 0) (which == 0 ? a.q_scale : a.k_scale)[bh] = outer_scale(__uint_as_float(a.qk_amax[which * a.BH + bh]));
+  if (which) return;
   if (a.flags & VC_FLAG_K_SMOOTH) {
     double s = 0.0;
 #pragma unroll 8
@@ -1112,11 +1114,11 @@ __global__ void prep_finalize_kernel(const PrepArgs a) {
   }
 }
 
-// A warp's rows of the swizzled code tile, from row0 on -> the block's code rows: full-line stores.
+// A warp's rows of the swizzled code tile, from row0 on -> rows `first` + row0 and on of `codes`: full-line stores.
 template <int ROW_BYTES>
-__device__ __forceinline__ void store_warp_rows(uint8_t* block, const unsigned char* out_tile, int row0, int lane) {
+__device__ __forceinline__ void store_warp_rows(uint8_t* codes, size_t first, const unsigned char* out_tile, int row0, int lane) {
   constexpr int CPR = ROW_BYTES / 16, RW = 32 / kTpr;                // 16-byte chunks per code row, rows of a warp
-  uint4* gdst = reinterpret_cast<uint4*>(block + (size_t)row0 * ROW_BYTES) + lane;
+  uint4* gdst = reinterpret_cast<uint4*>(codes + (first + row0) * ROW_BYTES) + lane;
 #pragma unroll
   for (int k = 0; k < CPR * RW / 32; ++k) {
     const int idx = k * 32 + lane, row = row0 + idx / CPR, chunk = idx % CPR;
@@ -1133,8 +1135,9 @@ __device__ __forceinline__ void store_warp_rows(uint8_t* block, const unsigned c
 // data needs warp-level synchronization only; the one CTA-wide barrier per item is the exchange
 // of the block maximum.
 // Shared memory: [2 stages x 128 x pitch][out tile 128 x D][src ring 3 x 128][scratch][RoPE table].
-// FAST: the packed row transform (standard configuration), see qk_row_item_fast.
-template <int D, int STAGE, bool FAST>
+// FAST: the packed row transform (standard configuration), see qk_row_item_fast.  OUTER: the items form the NVFP4 outer scale
+// from the head maximum themselves, one of a head's blocks stores it (else it is read).
+template <int D, int STAGE, bool FAST, bool OUTER = false>
 __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
   constexpr int NT = kRowThreads * kTpr;
   constexpr int kRowBytes = STAGE == kStageQuant4 ? D / 2 : D;      // code bytes per row
@@ -1197,15 +1200,21 @@ __device__ __forceinline__ void qk_pass(const PrepArgs& a, unsigned char* smem, 
     const unsigned char* stage = smem + (i & 1) * Geo<D>::stage_bytes;
     const int s0 = src_ring[(i % 3) * kBlock + my_row];
     const int tensor = c0.z + z0, bh = a.bh0 + c0.hh;
-    unsigned int* amax_at = a.qk_amax + tensor * a.BH + bh;
+    auto amax_at = [&] { return a.qk_amax + tensor * a.BH + bh; };
+    auto outer = [&] {
+      if constexpr (!OUTER) return (tensor == 0 ? a.q_scale : a.k_scale)[bh];
+      const float s = outer_scale(__uint_as_float(*amax_at()));
+      if (tid == 0 && c0.blk == 0) (tensor == 0 ? a.q_scale : a.k_scale)[bh] = s;
+      return s;
+    };
     if constexpr (FAST)
-      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at);
+      qk_row_item_fast<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab.saddr, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at, outer);
     else
-      qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at);
+      qk_row_item<D, STAGE>(a, tensor, stage, out_tile, red, kmean_s, tab, bh, c0.blk, i, tensor == 1 && c0.hh != last_hh, s0, amax_at, outer);
     if (tensor == 1) last_hh = c0.hh;
     if constexpr (STAGE != kStageAmax) {
       __syncwarp();                           // the warp's rows of the code tile are complete
-      store_warp_rows<kRowBytes>((tensor == 0 ? a.q_codes : a.k_codes) + ((size_t)bh * a.n_pad + (size_t)c0.blk * kBlock) * kRowBytes, out_tile, row0, lane);
+      store_warp_rows<kRowBytes>(tensor == 0 ? a.q_codes : a.k_codes, (size_t)bh * a.n_pad + (size_t)c0.blk * kBlock, out_tile, row0, lane);
     }
     c0 = c1;
     advance(c1, step, a.nb, nh);
@@ -1236,7 +1245,8 @@ struct Share {
   int z0;                    // first tensor of the Q/K quantizing pass (0 = Q, 1 = K)
 };
 
-// Pass PASS of a launch.  VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits).
+// Pass PASS of a launch.  VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits, launch 1), outer scale formed from the
+// head maximum by every item (4 bits, launch 3).
 template <int D, int BITS, int PHASE, bool FAST, int VARIANT, int PASS>
 __device__ __forceinline__ void one_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
   constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
@@ -1247,7 +1257,7 @@ __device__ __forceinline__ void one_pass(const PrepArgs& a, unsigned char* smem,
   else if constexpr (BITS == 8) v_pass<D, kVQuant8>(a, smem, sl, nh);
   else if constexpr (PHASE == kPhase2 && PASS == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
   else if constexpr (PHASE == kPhase2) qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 1);
-  else qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 1);
+  else qk_pass<D, kQuant, FAST, VARIANT != 0>(a, smem, sl, nh, 1);
 }
 
 // TURNS = false: a CTA belongs to one pass.  TURNS = true: every CTA takes its part of every pass, one pass after
@@ -1366,8 +1376,8 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     const int per = pr.nb * nh;
     a.bh0 = bh0;
     const int sums = a.flags & VC_FLAG_K_SMOOTH ? per : 0;
-    auto finalize = [&]() {
-      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), 8 * D, 0, s, a);
+    auto finalize = [&](int which, int threads) {
+      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
       count_launches(1);
     };
     auto launch = [&](auto whole, auto in_turns, size_t bytes, Work w0, Work w1, Work w2, int z0) {
@@ -1382,7 +1392,7 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
                  second = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, second_turns = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>;
       if (!ext) {
         launch(first, first_turns, wide ? rest_smem : smem, wide ? none : rows, k_sums, v_stats, 0);
-        finalize();
+        finalize(0, 8 * D);
       }
       // (with supplied statistics there is no first launch for Q to share; on a wide grid it does not share one)
       const bool q_too = ext || wide;
@@ -1391,13 +1401,21 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     } else {
       const auto first = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, false>>, first_turns = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, true>>,
                  second = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, false>>, second_turns = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, true>>,
-                 third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>;
+                 third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>, third_outer = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 1, false>>;
       launch(first, first_turns, wide ? rest_smem : smem, wide ? none : amax, k_sums, v_codes4, 0);
       if (wide) launch(first, first_turns, row_smem, amax, none, none, 0);
-      finalize();
+      finalize(0, 8 * D);
       launch(second, second_turns, smem, rows, amax, none, 0);
-      // (the outer scale of K follows from its head maximum where the codes are made: a launch of its own was 2 us)
-      launch(third, third, smem, rows, none, none, 1);
+      // The outer scale of K: a launch of its own is some 0.6 us of the chain, forming it in every item 1 percent of the K codes'
+      // pass, so the items form it while a CTA has few.  By items / by a launch, NVFP4: B1 H12 N4096 d64 29.0 / 29.5 us, d128
+      // 41.6 / 42.2; H12 N16384 d64 81.0 / 81.6; H12 N32760 (10 items per CTA) d64 146.5 / 146.4; H40 (35) d64 436.8 / 435.2;
+      // H24 N118800 (75) d64 904 / 899, d128 1468 / 1463.
+      if (per <= 16 * 2 * sm_count()) {
+        launch(third_outer, third_outer, smem, rows, none, none, 1);
+      } else {
+        finalize(1, 32);
+        launch(third, third, smem, rows, none, none, 1);
+      }
     }
   }
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -1573,6 +1591,7 @@ __global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs 
   if (blockIdx.x == 0 && tid == 0) *s.status = 0u;
 
   const int my_row = qk_row_of(tid), row0 = warp * (32 / kTpr);
+  auto none = [] { return (unsigned int*)nullptr; };   // (what a stage does not ask for)
   if (tensor == 1) {
     if (smooth) {
       const RopeTab tab{smem_u32(plain), nullptr};
@@ -1601,7 +1620,7 @@ __global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs 
   }
   if constexpr (BITS == 4) {                  // the head maximum, over the rows in place
     const int pos = blk * kBlock + my_row;
-    qk_row_item_fast<D, kStageAmax>(a, tensor, in_place, out_tile, qred, pm, smem_u32(folded), bh, blk, 0, false, pos < a.N ? pos : -1, amax);
+    qk_row_item_fast<D, kStageAmax>(a, tensor, in_place, out_tile, qred, pm, smem_u32(folded), bh, blk, 0, false, pos < a.N ? pos : -1, [&] { return amax; }, none);
     cluster_arrive();
     cluster_wait();
     const unsigned int most = __reduce_max_sync(0xffffffffu, lane < a.nb ? peer_word(amax, lane) : 0u);
@@ -1609,9 +1628,14 @@ __global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs 
     if (tid == 0) amax[1] = most;
     __syncthreads();
   }
-  qk_row_item_fast<D, kQuant>(a, tensor, gathered, out_tile, qred, pm, smem_u32(folded), bh, blk, 1, false, src[my_row], amax + 1);
+  auto outer = [&] {
+    const float g = outer_scale(__uint_as_float(amax[1]));
+    if (tid == 0 && blk == 0) (tensor ? a.k_scale : a.q_scale)[bh] = g;
+    return g;
+  };
+  qk_row_item_fast<D, kQuant>(a, tensor, gathered, out_tile, qred, pm, smem_u32(folded), bh, blk, 1, false, src[my_row], none, outer);
   __syncwarp();                               // the warp's rows of the code tile are complete
-  store_warp_rows<kRowBytes>((tensor ? a.k_codes : a.q_codes) + ((size_t)bh * a.n_pad + (size_t)blk * kBlock) * kRowBytes, out_tile, row0, lane);
+  store_warp_rows<kRowBytes>(tensor ? a.k_codes : a.q_codes, (size_t)bh * a.n_pad + (size_t)blk * kBlock, out_tile, row0, lane);
   if (BITS == 4 || tensor == 1) cluster_wait();       // a CTA stays until its peers have read it
 }
 
