@@ -15,8 +15,8 @@
 // by-product of the running-max pass; per group the E4M3 factor of max p / 6 is formed once,
 // its log2 is folded into the exponent offset, and an element costs one FMA, one ex2 and half a conversion:
 // code = E2M1(2^(s cs + log2 2688 - m' - log2 f_g)).  Some of the groups take a polynomial in place of the ex2 (see
-// e2m1_poly2), because the special-function unit is what the stage waits for.  (A polynomial that is an exponential,
-// with its range reduction, was slower: ten instructions an element instead of three and a half.)
+// vc_nvfp4_codes.cuh), because the special-function unit is what the stage waits for.  (A polynomial that is an
+// exponential, with its range reduction, was slower: ten instructions an element instead of three and a half.)
 //
 // HYB = true is the hybrid 4-bit arrangement: the score product stays NVFP4, but P is the
 // ExpCast-FP8 code of Eq. 7 (five instructions per four scores, as in the 8-bit kernel) and the value product
@@ -29,6 +29,7 @@
 #include "vc_attn_shared.cuh"
 #include "vc_internal.h"
 #include "vc_launch.h"
+#include "vc_nvfp4_codes.cuh"
 #include "vc_sm100.cuh"
 
 namespace vc {
@@ -86,28 +87,7 @@ struct Attn4Args {
   WaitArgs wait;
 };
 
-// Value of a non-negative E4M3 byte.
-__device__ __forceinline__ float decode_ue4m3(uint32_t code) {
-  return code >= 8u ? __uint_as_float((code + 960u) << 20) : (float)code * 0.001953125f;
-}
-
-// The codes are the A operand of the value product in tensor memory; through shared memory, where the copies and both
-// operands of the score product meet, B1 H40 N32760 d128 took 11.69 ms instead of 11.20 (hybrid), B1 H24 N118800
-// 83.3 instead of 80.1, and B1 H12 N32760 4.49 instead of 4.45 (NVFP4).
-// E2M1 codes need no exponential, only something that lies on the right side of the format's seven rounding thresholds
-// 0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.  This polynomial in x = log2(value) + 2 goes through all seven (x = 0 at the first),
-// grows all the way to the top of the range and falls to minus infinity below zero, where the conversion clamps:
-// degree 6 through the points plus 1.2e-4 times the product of their distances, in seven packed FMAs per two elements.
-// Evaluated in FP32 its thresholds are within 2.4e-7 in the log2 domain (ex2.approx: 2^-22 of the value, 3.4e-7).
-__device__ __forceinline__ uint64_t e2m1_poly2(uint64_t x) {
-  constexpr float c[8] = {0.25f, 0.23001262545585632f, -0.06627432256937027f, 0.12829358875751495f,
-                          -0.0517636276781559f, 0.014539925381541252f, -0.0019345706095919013f, 0.00011999999696854502f};
-  uint64_t r = pack_f32x2(c[7], c[7]);
-#pragma unroll
-  for (int k = 6; k >= 0; --k) r = fma2(r, x, pack_f32x2(c[k], c[k]));
-  return r;
-}
-
+// One query tile or pair of tiles (TWO) of head bh, first tile q0.
 //   warp 0        TMA producer: Q^ tiles and their factors once; per key tile K^_j, R^_j, the
 //                 tile's factor chunks and block mean through a 4-stage ring
 //   warp 1        score issuer:        S = Q^_t K^_j^T            D/64 x kind::mxf4nvf4
@@ -116,6 +96,9 @@ __device__ __forceinline__ uint64_t e2m1_poly2(uint64_t x) {
 //   warps 4-11    softmax warpgroups (tile 0, tile 1), one thread per query row
 //   warps 12-19   correction warpgroups, one thread per query row
 // Tensor memory: S (128 columns) | A_0 (d + 16) | A_1 (d + 16) | scale factors (56 columns; HYB 32) | P_0 | P_1 (16 each; HYB 32).
+// The codes are the A operand of the value product there.  Through shared memory, where the copies and both operands
+// of the score product meet, B1 H40 N32760 d128 took 11.69 ms instead of 11.20 (hybrid), B1 H24 N118800 83.3
+// instead of 80.1, and B1 H12 N32760 4.49 instead of 4.45 (NVFP4).
 template <int D, bool HYB, bool SMOOTH, bool TWO>
 __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                               const Attn4Args& a, const int q0, const int bh) {
@@ -188,7 +171,7 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
   for (int i = tid; i < 128; i += 640)
     reinterpret_cast<uint32_t*>(sSfOnes)[i] = HYB ? 0x7f7f7f7fu : ((i & 3) == 0 && i < 64) ? 0x38383838u : 0u;
   if constexpr (!HYB)                                          // (no lane takes code 127, the NaN)
-    for (int i = tid; i < 128; i += 640) sLg2[i] = i ? lg2_approx(decode_ue4m3(i)) : INFINITY;
+    for (int i = tid; i < 128; i += 640) sLg2[i] = nvfp4::log2_entry(i);
   pdl_wait();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor-core reads
   if (warp == 2) { tmem_alloc<kTmemCols>(&sh->tmem_base); tmem_relinquish(); }
@@ -424,62 +407,23 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
         mbar_arrive(&sh->pc_full[slot(t, j)]);
         continue;
       }
-      // p = 2^(s cs - m') * 2688: the row maximum maps to 6 * 448, so the largest factor is 448.
-      // Per 16-key group: factor = E4M3(max p / 6); element / factor = 2^(s cs + c0 - log2 factor),
-      // a zero factor (log2: +infinity in the table) zeroes the group.  The logarithm comes from a table
-      // of the 128 codes, filled with what the instruction gives: decoding a code and taking its
-      // logarithm eight times per row and key tile cost 14 percent of the kernel (B1 H12 N32760 d128
-      // 5.25 -> 4.50 ms, B2 H16 N16384 d64 3.37 -> 2.83).
-      // Groups whose codes come from the polynomial: two of the eight at d = 128, three at d = 64 (the
-      // special-function unit is the longer queue there).  None 4.44 / 4.35 ms (B1 H12 N32760 d128 with / without value
-      // smoothing) and 2.89 (B2 H16 N16384 d64); groups 2 and 4 4.29 / 4.09 and 2.79; 1, 4 and 7 4.47 / 4.33 and 2.74;
-      // other pairs and threes lie between, four groups 4.43 / 4.37 and 2.89.
-      auto by_poly = [](int g) { return ((D == 128 ? 0x14 : 0x92) >> g) & 1; };
-      const float c0 = 11.39231742277876f - m_new;        // log2(2688) - m'
-      const float c0p = 13.39231742277876f - m_new;       // ... + 2, where the polynomial's argument starts
+      // NVFP4 (see nvfp4::Row)
+      const nvfp4::Row<D> nv(cs, m_new, lg2_at);
       uint32_t sfw[2] = {0u, 0u};
       float off[8];
-      auto factors = [&](int g) {                         // of groups g and g + 1
-        const float p0 = ex2_approx(fmaf(mx[g], cs, c0)), p1 = ex2_approx(fmaf(mx[g + 1], cs, c0));
-        const uint32_t sb = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(p0 * (1.0f / 6.0f), p1 * (1.0f / 6.0f)), __NV_SATFINITE, __NV_E4M3);
-        sfw[g >> 2] |= sb << (8 * (g & 2));
-        off[g] = (by_poly(g) ? c0p : c0) - lds32(lg2_at + 4 * (sb & 0xffu));
-        off[g + 1] = (by_poly(g + 1) ? c0p : c0) - lds32(lg2_at + 4 * (sb >> 8));
-      };
       // Six factors in front of the wait, two behind it, where they overlap the first exponentials (four and
       // four at d = 64): B1 H12 N32760 d128 4.33 ms with six, 4.39 with four, 4.47 with none;
       // B2 H16 N16384 d64 2.83 with six, 2.75 with four, 2.79 with none
       constexpr int kAhead = D == 128 ? 6 : 4;
 #pragma unroll
-      for (int g = 0; g < kAhead; g += 2) factors(g);
+      for (int g = 0; g < kAhead; g += 2) nv.factors(g, mx, sfw, off);
       // the previous code tile must have been consumed before it is overwritten
       if (TWO ? j > 0 && !warp_wait2(&sh->o_done[t], (j - 1) & 1, sh, a.wait, 31) : j > 1 && !warp_wait2(&sh->o_done[j & 1], par(j) ^ 1, sh, a.wait, 31)) break;
-
 #pragma unroll
-      for (int g = kAhead; g < 8; g += 2) factors(g);
-      const uint64_t cs2 = pack_f32x2(cs, cs);
-      auto quant16 = [&](const uint32_t (&sv)[32], int half, int g) -> uint2 {   // keys 16 g .. 16 g + 15
-        float v[16];
-        const uint64_t off2 = pack_f32x2(off[g], off[g]);
-        if (by_poly(g)) {
-#pragma unroll
-          for (int i = 0; i < 16; i += 2) unpack2(e2m1_poly2(fma2(pack_b32x2(sv[16 * half + i], sv[16 * half + i + 1]), cs2, off2)), v[i], v[i + 1]);
-          return make_uint2(cvt_relu_e2m1x8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]),
-                            cvt_relu_e2m1x8(v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]));
-        }
-#pragma unroll
-        for (int i = 0; i < 16; i += 2) {                 // the exponent's FMA on two scores per instruction
-          float x0, x1;
-          unpack2(fma2(pack_b32x2(sv[16 * half + i], sv[16 * half + i + 1]), cs2, off2), x0, x1);
-          v[i] = ex2_approx(x0);
-          v[i + 1] = ex2_approx(x1);
-        }
-        return make_uint2(cvt_e2m1x8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]),
-                          cvt_e2m1x8(v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]));
-      };
+      for (int g = kAhead; g < 8; g += 2) nv.factors(g, mx, sfw, off);
       const uint32_t p_col = lane_base + P_COL + kPCols * buf(t, j);
       auto store32 = [&](const uint32_t (&sv)[32], int q) {       // keys 32 q .. + 31, eight a column
-        const uint2 lo = quant16(sv, 0, 2 * q), hi = quant16(sv, 1, 2 * q + 1);
+        const uint2 lo = nv.codes16(sv, 0, 2 * q, off), hi = nv.codes16(sv, 1, 2 * q + 1, off);
         tmem_st4(p_col + 4 * q, lo.x, lo.y, hi.x, hi.y);
       };
       tc_fence_after();

@@ -1,4 +1,4 @@
-"""The polynomial that stands in for the exponential in front of an E2M1 conversion (vc_attn_fwd4.cu): evaluated in FP32
+"""The polynomial that stands in for the exponential in front of an E2M1 conversion (vc_nvfp4_codes.cuh): evaluated in FP32
 as the kernel does, it gives the code of 2^(x - 2) everywhere but within a rounding error of a threshold."""
 import os
 import re
@@ -6,7 +6,7 @@ import re
 import numpy as np
 import pytest
 
-SOURCE = os.path.join(os.path.dirname(__file__), "..", "paper_2609_15810_b200", "csrc", "vc_attn_fwd4.cu")
+SOURCE = os.path.join(os.path.dirname(__file__), "..", "paper_2609_15810_b200", "csrc", "vc_nvfp4_codes.cuh")
 THRESHOLDS = np.array([0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.0])
 
 
