@@ -381,10 +381,10 @@ __device__ __forceinline__ void attn_2q_body(const CUtensorMap& tm_q, const CUte
     // my row of the row-sum operand: 32-byte rows, the two 16-byte chunks swap when (row / 4) is odd
     const uint32_t am_row = smem_u32(sAm + t * kAmBytes + row * 32 + 16 * ((row >> 2) & 1));
     const uint32_t alpha_at = smem_u32(&sh->alpha[0][row]), vs_at = smem_u32(sh->v_scale[t]);
-    // s_V of my channel, for everyone in the epilogue.  (Read from global memory there, eight dependent round trips:
-    // the epilogue took 2.8 us.
-    // B1 H2 N1024 d128 25.4 -> 24.0 us, B1 H6 N1955 d64 28.9 -> 28.1, B1 H12 N32760 d128 without smoothing 3.60 -> 3.55 ms.)
-    // (The barrier stands here, where every warp of the group comes by, and not where a wait may have given up.)
+    // s_V of my channel, for everyone in the epilogue: read from global memory there, its eight dependent round trips
+    // made the epilogue 2.8 us (B1 H2 N1024 d128 25.4 -> 24.0 us, B1 H6 N1955 d64 28.9 -> 28.1, B1 H12 N32760 d128 without
+    // smoothing 3.60 -> 3.55 ms).  The barrier stands here, where every warp of the group comes by, and not where a wait
+    // may have given up.
     if (row < D) sts32(vs_at + 4 * row, __ldg(&a.v_scale[(size_t)bh * D + row]));
     asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
     float l_resc = 0.f;       // l as it stands in column d after the latest rescale, before the tile's own sum

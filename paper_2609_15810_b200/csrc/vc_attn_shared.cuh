@@ -182,12 +182,11 @@ struct MeanRows {
   }
 };
 
-// Output rows leave through shared memory.  A thread of the epilogue holds one row, and storing it from there puts the lanes
-// of a warp on 32 lines at a time.  So a
-// warp writes its 32 rows, W columns at a time, into a tile of its own (16-byte chunk c at position c ^ swizzle: no bank
-// conflicts) and stores it in whole lines: B2 H16 N4096 d128 INT8 scores 267.3 -> 263.1 us, B1 H16 N4096 FP8 126.8 -> 124.9.
-// (The epilogue by the softmax warps, 64 columns at a time, is 0.2 us shorter, but what it keeps alive across their loop
-// costs more: the same calls 267 and 131 us.)
+// Output rows leave through shared memory.  A thread of the epilogue holds one row, and storing it from there puts the
+// lanes of a warp on 32 lines at a time.  So a warp writes its 32 rows, W columns at a time, into a tile of its own
+// (16-byte chunk c at position c ^ swizzle: no bank conflicts) and stores it in whole lines: B2 H16 N4096 d128 INT8 scores
+// 267.3 -> 263.1 us, B1 H16 N4096 FP8 126.8 -> 124.9.  (The epilogue by the softmax warps, 64 columns at a time, is 0.2 us
+// shorter, but what it keeps alive across their loop costs more: the same calls 267 and 131 us.)
 // The tile lies in stage (nb + t) % kStages2 of the ring: it held key tile nb - 4 + t, and what may still be read when tile t's
 // last product is complete are the last key tile and the block mean of the one before it.
 template <int W> struct OutTile {

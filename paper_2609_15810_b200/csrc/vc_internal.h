@@ -63,7 +63,7 @@ WorkLayout work_layout(const Problem& pr);
 
 // Launchers (each returns the CUDA error of its launches; all asynchronous on `stream`).
 // then_attention: the attention launch follows at once (vc_attn), and short heads may take the one launch made for that.
-// (vc_prep alone keeps its launches: their number, with and without supplied statistics, is part of what it reports.)
+// (vc_prep alone keeps a launch per phase: with supplied statistics it is two launches fewer, which callers can count.)
 cudaError_t launch_prep(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
                         const void* q, const void* k, const void* v, const int32_t* perm,
                         uint8_t* quant, uint8_t* work, cudaStream_t stream, const vc_prep_stats* stats, bool then_attention);

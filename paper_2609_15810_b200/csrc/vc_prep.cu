@@ -1427,14 +1427,18 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
 // launches: table, statistics, finalization, codes, at 4 bits one more, 0.8 to 1.5 us from the end of each to the start of
 // the next beside its own filling of a pipeline (13.2 us from the table's start to the attention's at B1 H2 N1024 d128).  Here
 //   - every CTA computes the RoPE tables it needs itself, in front of the wait for the kernel before it;
-//   - a CTA keeps its block in shared memory, so K and V are read once and the statistics of a head meet in distributed
-//     shared memory, behind one cluster barrier each;
-//   - K is staged twice when a permutation gathers it: in sequence order for the column sums (and the head maximum),
-//     gathered for the codes.  The sums run over the same blocks, in the same order, as in the launches above.
+//   - a CTA keeps its block in shared memory, so V is read once, and K once unless a permutation gathers it; the statistics
+//     of a head meet in distributed shared memory, behind one cluster barrier each;
+//   - gathered K is staged twice: in sequence order for the column sums (and the head maximum), gathered for the codes
+//     (from L2 as a rule).  The sums run over the same blocks, in the same order, as in the launches above.
 // The row and value transforms are the ones of the other launches, and the bundle is the same, byte for byte.
-// Whole calls (d128; four launches before): FP8 B1 H2 N1024 24.0 -> 19.5 us, H12 28.8 -> 25.9, N576 H12 25.6 -> 19.6, N200 H12
-// 21.7 -> 14.8; NVFP4 (six launches) N1024 H12 37.3 -> 30.7, N200 H12 27.9 -> 18.3.  What bounds it: latency. Tables 1.5 to
-// 2.5 us (hidden when calls follow one another), rows 1.5, column sums 2, barrier 0.8, fold 1, codes 2.
+// Whole calls, d128, a launch per phase -> this one: FP8 (four launches) B1 H1 N1024 23.1 -> 18.4 us, H12 25.9 -> 24.9, H9 N576
+// 21.8 -> 18.0, H4 N200 18.0 -> 13.9; NVFP4 (five) H12 N1024 35.3 -> 30.3, H4 N200 25.6 -> 18.3.  What bounds it: latency. Tables
+// 1.5 to 2.5 us, rows 1.5, column sums 2, barrier 0.8, fold 1, codes 2.
+// The tables are hidden when calls of the library follow one another.  Behind a caller's kernel, which lets nothing start early,
+// they are in the open: H1 N1024 20.4 us instead of 18.4, 1 x 1 x 64 tokens (1387 entries) 16.4 instead of 12.2 (a launch per phase
+// 23.1 and 18.5 to 19.2 either way).  And every CTA computes its own: where many streams fill the GPU with such calls the sum of the
+// work counts, NVFP4 H8 N1024 on eight streams 13.6 us a call (13.0 with a launch per phase; on two 16.1 against 18.7).
 struct Short {
   double theta, n;           // n: tokens
   unsigned int* status;
@@ -1454,8 +1458,11 @@ __device__ __forceinline__ uint32_t peer_word(const void* p, int rank) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
   return v;
 }
-// x / n, correctly rounded, with inv = 1 / n already at hand: a quotient within an ulp and one correction by its exact
-// remainder (Markstein's theorem), three operations in place of a division behind the sums.
+// x / n for an integer n <= 128 kShortCluster, correctly rounded, with inv = 1 / n (rounded) already at hand: a quotient and one
+// correction by its remainder, three operations in place of a division behind the sums.  q is within 1.5 ulp of x / n (two
+// roundings), so x - q n is a multiple of ulp(q) below 2^12 of them: exact.  What is added is then off by 2^-52 of an ulp, while
+// x / n lies at least 1 / (2 n) of an ulp from a number halfway between two doubles (n times such a number has more than 53 bits, so
+// no x reaches it): the sum rounds as x / n does.
 __device__ __forceinline__ double divided(double x, double n, double inv) {
   const double q = x * inv;
   return isfinite(q) ? fma(fma(-q, n, x), inv, q) : q;
@@ -1640,9 +1647,12 @@ __global__ void __launch_bounds__(kThreads, 2) prep_short_kernel(const PrepArgs 
 }
 
 // Which calls take it: heads of at most eight blocks whose CTAs are resident at once at 8 bits (two per SM), or in two
-// waves at 4 bits, where one more launch falls away.  Beyond, a launch per phase whose CTAs prefetch their next blocks
-// is faster: FP8 d128 N576 H24 (432 CTAs in clusters of 8) 31.9 us against 27.0, NVFP4 H40 55.9 against 50.1; N1024 NVFP4 H24
-// (576 CTAs) 43.3 against 48.8, FP8 H18 (432) 30.0 against 30.0.
+// waves at 4 bits, where one more launch falls away.  Up to there it is the faster form in every format, at both widths and behind a
+// caller's kernel too.  At the line and beyond, one launch / a launch per phase (us, whole calls, d128): FP8 N1024 H12 (288 CTAs)
+// 24.9 / 25.9, H15 (360) 26.6 / 27.6, H18 (432) 28.8 / 29.1 and behind a caller's kernel 30.0 / 29.0, H30 (720) 39.2 / 36.4; N576
+// H24 (360) 24.7 / 26.3, H28 (420) 31.6 / 31.3; NVFP4 N1024 H18 38.4 / 39.8, H24 (576) 42.2 / 47.6, H30 (720) 47.1 / 49.3; d64 H24
+// 32.4 / 37.2.  So at 8 bits the line is where heads of eight blocks still gain behind anything; shorter heads gain beyond it as well
+// (N100 H240, 720 CTAs, 30.1 / 37.6), which the rule leaves.
 inline bool short_heads(const Problem& pr, const PrepArgs& a) {
   return pr.nb <= kShortCluster && a.rd.entries <= kShortEntries && !(pr.flags & VC_FLAG_CHECK_PERM) && 3 * pr.BH * pr.nb <= (pr.bits == 8 ? 2 : 4) * sm_count();
 }
