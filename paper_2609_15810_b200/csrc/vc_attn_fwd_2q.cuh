@@ -25,16 +25,16 @@ using namespace attn;
 //     registers.  At d = 128 one score buffer serves both query tiles in turn (all that tensor memory
 //     has room for); at d = 64 each tile has its own, but for kSfu.  (An MMA with both operands in shared memory reads
 //     128 bytes a clock, all a shared-memory port gives.  With the codes there as well, 32 KB written and
-//     32 KB read per pair of tiles, every copy and store slowed the products down: B2 H16 N16384 d64
-//     1956 -> 1870 us, B1 H12 N32760 d128 without value smoothing 3677 -> 3604, B1 H40 12.49 -> 12.33 ms
-//     under the power cap, B1 H6 N1955 d64 29.8 -> 28.9 us.)
+//     32 KB read per pair of tiles, every copy and store slowed the products down; the port was busy for 78 percent of
+//     the launch at d = 128 and 69 at d = 64, now 53 and 39.  B2 H16 N16384 d64 1956 -> 1870 us, B1 H12 N32760 d128
+//     without value smoothing 3677 -> 3604, B1 H40 12.49 -> 12.33 ms under the power cap, B1 H6 N1955 d64 29.8 -> 28.9 us.)
 //   * The row sums of the decoded codes (Eq. 6: r_ij, and the normalizer l) come from the
 //     tensor core: the value operand carries 16 extra rows of ones, so columns d..d+15 of the
 //     accumulator hold l, rescaled by alpha together with the rest.  The softmax threads do
 //     nothing but the row maximum and five instructions per four codes.
 //
-// What bounds it: per key tile and pair of query tiles the kernel takes about 2070 cycles at d = 128
-// (1850 at d = 64).  The tensor pipe needs 1216 of them (704 at d = 64); two softmax warps per
+// What bounds it: per key tile and pair of query tiles the kernel takes about 2030 cycles at d = 128
+// (1680 at d = 64).  The tensor pipe needs 1216 of them (704 at d = 64); two softmax warps per
 // scheduler need about 1000 when nothing else runs on it and the correction warps and the hand-offs
 // of the shared score buffer (1500 cycles per pair when they are all that is timed) take the rest.
 // Above a few milliseconds at a stretch the power cap of the board bounds it as well.
