@@ -1087,17 +1087,21 @@ __device__ __forceinline__ void v_pass(const PrepArgs& a, unsigned char* smem, c
   }
 }
 
-// Per-head finalization.  which 0: K channel mean, V scale, at 4 bits the outer scale of Q; a block of 8 D threads per head, the
-// block partial sums are added in double, in eight interleaved slices that are then added in a fixed order.
-// which 1 (4 bits): the outer scale of K.
-template <int D, int BITS>
-__global__ void prep_finalize_kernel(const PrepArgs a, int which) {
+// Per-head finalization.  kMeans: K channel mean, V scale; a block of 8 D threads per head, the block partial sums are added in
+// double, in eight interleaved slices that are then added in a fixed order.  kOuter (4 bits): the outer scale of Q, or on its
+// own, behind the next launch, that of K.
+enum { kMeans = 1, kOuter = 2 };
+template <int D, int BITS, int WHAT>
+__global__ void prep_finalize_kernel(const PrepArgs a) {
   __shared__ double part[8][D];
   const int bh = a.bh0 + blockIdx.x, c = threadIdx.x % D, slice = threadIdx.x / D;
   pdl_wait();
   pdl_allow();
-  if (BITS == 4 && threadIdx.x == 0) (which == 0 ? a.q_scale : a.k_scale)[bh] = outer_scale(__uint_as_float(a.qk_amax[which * a.BH + bh]));
-  if (which) return;
+  if ((WHAT & kOuter) && threadIdx.x == 0) {
+    constexpr bool kOfK = !(WHAT & kMeans);
+    (kOfK ? a.k_scale : a.q_scale)[bh] = outer_scale(__uint_as_float(a.qk_amax[kOfK * a.BH + bh]));
+  }
+  if (!(WHAT & kMeans)) return;
   if (a.flags & VC_FLAG_K_SMOOTH) {
     double s = 0.0;
 #pragma unroll 8
@@ -1246,7 +1250,7 @@ struct Share {
 };
 
 // Pass PASS of a launch.  VARIANT: INT8 codes (8 bits), power-of-two value factors (4 bits, launch 1), outer scale formed from the
-// head maximum by every item (4 bits, launch 3).
+// head maximum by every item (4 bits, launches 2 and 3).
 template <int D, int BITS, int PHASE, bool FAST, int VARIANT, int PASS>
 __device__ __forceinline__ void one_pass(const PrepArgs& a, unsigned char* smem, const Slot sl, int nh, int z0) {
   constexpr int kQuant = BITS == 4 ? kStageQuant4 : (VARIANT ? kStageQuant8I : kStageQuant8);
@@ -1255,7 +1259,7 @@ __device__ __forceinline__ void one_pass(const PrepArgs& a, unsigned char* smem,
   else if constexpr (PHASE == kPhase1) v_pass<D, BITS == 8 ? kVStats : (VARIANT ? kVQuant4M : kVQuant4)>(a, smem, sl, nh);
   else if constexpr (BITS == 8 && PASS == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, z0);
   else if constexpr (BITS == 8) v_pass<D, kVQuant8>(a, smem, sl, nh);
-  else if constexpr (PHASE == kPhase2 && PASS == 0) qk_pass<D, kQuant, FAST>(a, smem, sl, nh, 0);
+  else if constexpr (PHASE == kPhase2 && PASS == 0) qk_pass<D, kQuant, FAST, VARIANT != 0>(a, smem, sl, nh, 0);
   else if constexpr (PHASE == kPhase2) qk_pass<D, kStageAmax, FAST>(a, smem, sl, nh, 1);
   else qk_pass<D, kQuant, FAST, VARIANT != 0>(a, smem, sl, nh, 1);
 }
@@ -1376,8 +1380,8 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     const int per = pr.nb * nh;
     a.bh0 = bh0;
     const int sums = a.flags & VC_FLAG_K_SMOOTH ? per : 0;
-    auto finalize = [&](int which, int threads) {
-      if (e == cudaSuccess) e = launch_overlapped(prep_finalize_kernel<D, BITS>, dim3((unsigned)nh), threads, 0, s, a, which);
+    auto finalize = [&](auto kernel, int threads) {
+      if (e == cudaSuccess) e = launch_overlapped(kernel, dim3((unsigned)nh), threads, 0, s, a);
       count_launches(1);
     };
     auto launch = [&](auto whole, auto in_turns, size_t bytes, Work w0, Work w1, Work w2, int z0) {
@@ -1392,7 +1396,7 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
                  second = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, false>>, second_turns = launch_phase<prep_kernel<D, 8, kPhase2, FAST, VARIANT, true>>;
       if (!ext) {
         launch(first, first_turns, wide ? rest_smem : smem, wide ? none : rows, k_sums, v_stats, 0);
-        finalize(0, 8 * D);
+        finalize(prep_finalize_kernel<D, 8, kMeans>, 8 * D);
       }
       // (with supplied statistics there is no first launch for Q to share; on a wide grid it does not share one)
       const bool q_too = ext || wide;
@@ -1401,21 +1405,27 @@ cudaError_t run_phases(const Problem& pr, PrepArgs a, cudaStream_t s) {
     } else {
       const auto first = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, false>>, first_turns = launch_phase<prep_kernel<D, 4, kPhase1, FAST, VARIANT, true>>,
                  second = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, false>>, second_turns = launch_phase<prep_kernel<D, 4, kPhase2, FAST, 0, true>>,
-                 third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>, third_outer = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 1, false>>;
+                 third = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 0, false>>, third_outer = launch_phase<prep_kernel<D, 4, kPhase3, FAST, 1, false>>,
+                 second_outer = launch_phase<prep_kernel<D, 4, kPhase2, FAST, FAST, false>>;
       launch(first, first_turns, wide ? rest_smem : smem, wide ? none : amax, k_sums, v_codes4, 0);
       if (wide) launch(first, first_turns, row_smem, amax, none, none, 0);
-      finalize(0, 8 * D);
-      launch(second, second_turns, smem, rows, amax, none, 0);
-      // The outer scale of K: a launch of its own is some 0.6 us of the chain, forming it in every item 1 percent of the K codes'
-      // pass, so the items form it while a CTA has few.  By items / by a launch, NVFP4: B1 H12 N4096 d64 29.0 / 29.5 us, d128
-      // 41.6 / 42.2; H12 N16384 d64 81.0 / 81.6; H12 N32760 (10 items per CTA) d64 146.5 / 146.4; H40 (35) d64 436.8 / 435.2;
-      // H24 N118800 (75) d64 904 / 899, d128 1468 / 1463.
-      if (per <= 16 * 2 * sm_count()) {
-        launch(third_outer, third_outer, smem, rows, none, none, 1);
+      // The outer scales.  K's in a launch of its own is some 0.6 us of the chain, Q's in the finalization 0.3; forming them in every
+      // item costs 1 percent of the codes' passes.  So the items form them while a CTA has few.  By items / by launches, NVFP4:
+      // B1 H12 N4096 d64 29.0 / 29.5 us, d128 41.6 / 42.2; H12 N16384 d64 81.0 / 81.6; H12 N32760 (10 items per CTA) d64 146.5 /
+      // 146.4; H40 (35) d64 438 / 435; H24 N118800 (75) d64 908 / 899, d128 without RoPE 1506 / 1434.
+      // Q's share a launch with another pass, which goes in turns beyond turns_from items per CTA of both (share_ctas): the items
+      // form them only where it does not.  (And not in the general row body, which has no registers left for it.)
+      const bool few = per <= 16 * 2 * sm_count(), q_too = FAST && 2 * per <= turns_from * 2 * sm_count();
+      if (q_too) {
+        finalize(prep_finalize_kernel<D, 4, kMeans>, 8 * D);
+        launch(second_outer, second_outer, smem, rows, amax, none, 0);
       } else {
-        finalize(1, 32);
-        launch(third, third, smem, rows, none, none, 1);
+        finalize(prep_finalize_kernel<D, 4, kMeans | kOuter>, 8 * D);
+        launch(second, second_turns, smem, rows, amax, none, 0);
       }
+      if (!few) finalize(prep_finalize_kernel<D, 4, kOuter>, 32);
+      const auto codes = few ? third_outer : third;
+      launch(codes, codes, smem, rows, none, none, 1);
     }
   }
   return e != cudaSuccess ? e : cudaGetLastError();

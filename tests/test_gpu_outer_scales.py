@@ -1,5 +1,6 @@
-"""The NVFP4 outer scale of K: formed by the items of the codes' pass up to 16 items per CTA, by a launch in front of it
-beyond.  A head's codes and scales are the same bytes either way, and the same as in a call of its own."""
+"""The NVFP4 outer scales: K's formed by the items of the codes' pass up to 16 items per CTA, by a launch in front of it
+beyond; Q's by the items where their launch does not go in turns, by the finalization beyond.  A head's codes and scales are
+the same bytes in every form, and the same as in a call of its own."""
 import pytest
 import torch
 
@@ -41,10 +42,12 @@ def test_both_forms_give_the_same_bundle(d, p_format, flags):
     by_items, n_items = _prep(q[:, :most].contiguous(), k[:, :most].contiguous(), v[:, :most].contiguous(), grid, p_format, flags)
     by_launch, n_launch = _prep(q, k, v, grid, p_format, flags)
     assert (n_items, n_launch) == (5, 6)
-    groups, _ = _prep(q, k, v, grid, p_format, flags, heads_per_pass=most // 2)
     for n in SECTIONS:
         assert torch.equal(by_launch[n][:most], by_items[n]), n
-        assert torch.equal(by_launch[n], groups[n]), n
+    for group in (most // 2, most // 2 + 1):                 # the most heads whose Q items form the scale, and one more
+        groups, _ = _prep(q, k, v, grid, p_format, flags, heads_per_pass=group)
+        for n in SECTIONS:
+            assert torch.equal(by_launch[n], groups[n]), (n, group)
     for h in (0, 1, 2, most):
         alone, _ = _prep(*[t[:, h:h + 1].contiguous() for t in (q, k, v)], grid, p_format, flags)
         for n in SECTIONS:
