@@ -24,9 +24,9 @@ def _inputs(H, grid, d, perm, token_major, B=1):
     return q, k, v, torch.argsort(torch.rand(B, H, N, generator=g, device="cuda"), dim=-1).int() if perm else None
 
 
-def _params(q, grid, bits, p_format, flags):
+def _params(q, grid, bits, p_format, flags, **kw):
     B, H, N, d = q.shape
-    return Params.make(B, H, N, d, grid, bits=bits, p_format=p_format, flags=flags, stride_b=q.stride(0), stride_h=q.stride(1), stride_n=q.stride(2))
+    return Params.make(B, H, N, d, grid, bits=bits, p_format=p_format, flags=flags, stride_b=q.stride(0), stride_h=q.stride(1), stride_n=q.stride(2), **kw)
 
 
 def _same_bundle_and_output(q, k, v, perm, p, short):
@@ -60,6 +60,22 @@ def _same_bundle_and_output(q, k, v, perm, p, short):
 def test_same_bundle_and_output(grid, bits, p_format, flags, d, perm, token_major):
     q, k, v, pm = _inputs(3, grid, d, perm, token_major, B=2)
     _same_bundle_and_output(q, k, v, pm, _params(q, grid, bits, p_format, flags), True)
+
+
+# rows wider than the head, heads and batches with gaps between them, other frequencies and another scale
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("order", ["bhn", "bnh", "hbn"])
+def test_other_strides_and_frequencies(bits, d, order):
+    grid, sizes = (3, 7, 17), {"b": 2, "h": 3, "n": 357 + 5}
+    g = torch.Generator(device="cuda").manual_seed(d)
+    views = []
+    for _ in range(3):
+        full = torch.randn(*[sizes[c] for c in order], d + 24, generator=g, device="cuda", dtype=torch.bfloat16)
+        views.append(full.permute(*[order.index(c) for c in "bhn"], 3)[:, :, :357, :d])
+    perm = torch.argsort(torch.rand(2, 3, 357, generator=g, device="cuda"), dim=-1).int()
+    p = _params(views[0], grid, bits, vc.VC_P_DEFAULT, ALL, rope_theta=500.0, softmax_scale=0.07)
+    _same_bundle_and_output(*views, perm, p, True)
 
 
 # RoPE tables of 1390 to 1408 entries, the largest that leave two CTAs on an SM (d128: 44 / 42 / 42 channels, d64: 24 / 20 / 20), and of
