@@ -306,14 +306,15 @@ vc_status vc_test_expcast_codes(const float *s, int64_t n, float cs, float m, fl
                                 uint8_t *codes, void *stream);
 
 /* Test hook: NVFP4 probabilities formed exactly as the softmax stage of the 4-bit attention kernel for
- * head dimension `d` (64 or 128) forms them, on their own.  Row r holds 128 scores s[128 r ...] (FP32,
+ * head dimension `d` (64 or 128) forms them, on their own: with some groups' codes by polynomial, as from six key
+ * tiles on, or with none (`polynomial` 0).  Row r holds 128 scores s[128 r ...] (FP32,
  * in units of the score product) under the factor `cs` (> 0) and the running maximum m[r] (log2
  * domain; s * cs <= m is the caller's business).  factors[8 r + g] is the E4M3 byte of
  * max 2^(s cs - m) * 2688 / 6 over keys 16 g .. 16 g + 15, codes[64 r + i] holds the E2M1 codes of keys 2 i
  * (low nibble) and 2 i + 1 divided by the factor of their group.  Device pointers, 16-byte aligned.
  * Asynchronous on `stream`; VC_ERR_INVALID_ARG for a bad argument.  Not for production. */
-vc_status vc_test_nvfp4_codes(const float *s, const float *m, int64_t rows, int32_t d, float cs, uint8_t *codes,
-                              uint8_t *factors, void *stream);
+vc_status vc_test_nvfp4_codes(const float *s, const float *m, int64_t rows, int32_t d, int32_t polynomial, float cs,
+                              uint8_t *codes, uint8_t *factors, void *stream);
 
 /* Measurement aid (Sec. 3.1 "The softmax bottleneck" compares the softmax stage with the time of
  * the two matrix products): the rate at which this GPU executes the products' MMAs with

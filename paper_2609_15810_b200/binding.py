@@ -107,7 +107,7 @@ def load_library():
     lib.vc_test_expcast_codes.restype = ctypes.c_int
     lib.vc_test_expcast_codes.argtypes = [vp, ctypes.c_int64, ctypes.c_float, ctypes.c_float, ctypes.c_float, vp, vp]
     lib.vc_test_nvfp4_codes.restype = ctypes.c_int
-    lib.vc_test_nvfp4_codes.argtypes = [vp, vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_float, vp, vp, vp]
+    lib.vc_test_nvfp4_codes.argtypes = [vp, vp, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_float, vp, vp, vp]
     lib.vc_mma_peak.restype = ctypes.c_int
     lib.vc_mma_peak.argtypes = [ctypes.c_int32, ctypes.c_int32, vp, ctypes.POINTER(ctypes.c_double),
                                 ctypes.POINTER(ctypes.c_double), vp]
@@ -239,13 +239,14 @@ def vc_test_expcast_codes(s, cs, m, beta=0.0):
     return out.view(s.shape)
 
 
-def vc_test_nvfp4_codes(s, m, d, cs):
+def vc_test_nvfp4_codes(s, m, d, cs, polynomial=True):
     """Test hook: (E2M1 codes [rows, 64], two a byte, E4M3 factors [rows, 8]) of the fp32 scores `s` [rows, 128] under the
-    factor cs and the running maxima `m` [rows], as the 4-bit attention kernel for head dimension d forms them."""
+    factor cs and the running maxima `m` [rows], as the 4-bit attention kernel for head dimension d forms them, with some groups'
+    codes by polynomial or with none."""
     assert s.dtype == m.dtype == torch.float32 and s.is_cuda and s.is_contiguous() and m.is_contiguous() and s.shape == (m.numel(), 128)
     codes = torch.empty(m.numel(), 64, dtype=torch.uint8, device=s.device)
     factors = torch.empty(m.numel(), 8, dtype=torch.uint8, device=s.device)
-    _check(load_library().vc_test_nvfp4_codes(_ptr(s), _ptr(m), m.numel(), int(d), float(cs), _ptr(codes), _ptr(factors), _stream()),
+    _check(load_library().vc_test_nvfp4_codes(_ptr(s), _ptr(m), m.numel(), int(d), int(polynomial), float(cs), _ptr(codes), _ptr(factors), _stream()),
            "vc_test_nvfp4_codes")
     return codes, factors
 

@@ -99,7 +99,7 @@ struct Attn4Args {
 // The codes are the A operand of the value product there.  Through shared memory, where the copies and both operands
 // of the score product meet, B1 H40 N32760 d128 took 11.69 ms instead of 11.20 (hybrid), B1 H24 N118800 83.3
 // instead of 80.1, and B1 H12 N32760 4.49 instead of 4.45 (NVFP4).
-template <int D, bool HYB, bool SMOOTH, bool TWO>
+template <int D, bool HYB, bool SMOOTH, bool POLY, bool TWO>
 __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                               const Attn4Args& a, const int q0, const int bh) {
   constexpr int kTmemCols = 512;
@@ -407,8 +407,8 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
         mbar_arrive(&sh->pc_full[slot(t, j)]);
         continue;
       }
-      // NVFP4 (see nvfp4::Row)
-      const nvfp4::Row<D> nv(cs, m_new, lg2_at);
+      // NVFP4 (see nvfp4::Row; POLY: some groups' codes by the polynomial)
+      const nvfp4::Row<D, POLY> nv(cs, m_new, lg2_at);
       uint32_t sfw[2] = {0u, 0u};
       float off[8];
       // Six factors in front of the wait, two behind it, where they overlap the first exponentials (four and
@@ -531,14 +531,14 @@ __device__ __forceinline__ void attn4_2q_body(const CUtensorMap& tm_q, const CUt
 }
 
 // CTAs with a pair of query tiles, and behind them CTAs with one (see split_tiles).
-template <int D, bool HYB, bool SMOOTH>
+template <int D, bool HYB, bool SMOOTH, bool POLY>
 __global__ void __launch_bounds__(640, 1)
 attn4_fwd_2q_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const Attn4Args a) {
   const TileOf w = tile_of(a.tiles, a.nb);
   if (w.q0 >= a.nb) return;                 // the missing second tile of a head's last pair
-  if (w.two) attn4_2q_body<D, HYB, SMOOTH, true>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
-  else attn4_2q_body<D, HYB, SMOOTH, false>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
+  if (w.two) attn4_2q_body<D, HYB, SMOOTH, POLY, true>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
+  else attn4_2q_body<D, HYB, SMOOTH, POLY, false>(tm_q, tm_k, tm_v, a, w.q0, w.bh);
 }
 
 template <int D, bool HYB>
@@ -568,14 +568,18 @@ cudaError_t run4(const Problem& pr, const QuantLayout& ql, const WorkLayout& wl,
   static_assert(smem <= 227 * 1024, "shared memory of the 4-bit kernel exceeds the SM");
   unsigned grid;
   a.tiles = split_tiles(pr, true, &grid);
-  cudaError_t e;
-  if (pr.flags & VC_FLAG_V_SMOOTH) {
-    if ((e = allow_smem<attn4_fwd_2q_kernel<D, HYB, true>>()) == cudaSuccess)
-      e = launch_overlapped(attn4_fwd_2q_kernel<D, HYB, true>, dim3(grid), 640, smem, s, tq, tk, tv, a);
-  } else {
-    if ((e = allow_smem<attn4_fwd_2q_kernel<D, HYB, false>>()) == cudaSuccess)
-      e = launch_overlapped(attn4_fwd_2q_kernel<D, HYB, false>, dim3(grid), 640, smem, s, tq, tk, tv, a);
-  }
+  // NVFP4 codes by polynomial from six key tiles on: the loop's longer code has to be fetched and the first tiles, with nothing
+  // to overlap, wait for it.  Whole calls, us, without / with: d64 N360 H80 40.3 / 42.3, N576 H48 41.1 / 42.3, N768 H40 36.5 / 35.9,
+  // N1024 H37 41.8 / 40.9; d128 N360 H80 54.6 / 55.2, N576 H48 52.9 / 53.5, N768 H40 46.0 / 45.7, N1024 H37 53.1 / 52.7.
+  const bool poly = !HYB && pr.nb >= 6;
+  cudaError_t e = cudaSuccess;
+#define VC_LAUNCH_4(...)                                                                                        \
+  ((e = allow_smem<attn4_fwd_2q_kernel<D, HYB, __VA_ARGS__>>()) == cudaSuccess                                  \
+       ? (e = launch_overlapped(attn4_fwd_2q_kernel<D, HYB, __VA_ARGS__>, dim3(grid), 640, smem, s, tq, tk, tv, a)) \
+       : e)
+  if (pr.flags & VC_FLAG_V_SMOOTH) poly ? VC_LAUNCH_4(true, !HYB) : VC_LAUNCH_4(true, false);
+  else poly ? VC_LAUNCH_4(false, !HYB) : VC_LAUNCH_4(false, false);
+#undef VC_LAUNCH_4
   if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();

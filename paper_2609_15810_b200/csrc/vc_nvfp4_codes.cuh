@@ -38,15 +38,15 @@ __device__ __forceinline__ uint64_t e2m1_poly2(uint64_t x) {
 // of the 128 codes, filled with what the instruction gives: decoding a code and taking its
 // logarithm eight times per row and key tile cost 14 percent of the kernel (B1 H12 N32760 d128
 // 5.25 -> 4.50 ms, B2 H16 N16384 d64 3.37 -> 2.83).
-// Groups whose codes come from the polynomial: two of the eight at d = 128, three at d = 64 (the
+// Groups whose codes come from the polynomial (POLY): two of the eight at d = 128, three at d = 64 (the
 // special-function unit is the longer queue there).  None 4.44 / 4.35 ms (B1 H12 N32760 d128 with / without value
 // smoothing) and 2.89 (B2 H16 N16384 d64); groups 2 and 4 4.29 / 4.09 and 2.79; 1, 4 and 7 4.47 / 4.33 and 2.74;
 // other pairs and threes lie between, four groups 4.43 / 4.37 and 2.89.
-template <int D> struct Row {
+template <int D, bool POLY> struct Row {
   float cs, c0, c0p;                                    // log2(2688) - m'; ... + 2, where the polynomial's argument starts
   uint32_t lg2_at;                                      // the table, in shared memory
   __device__ __forceinline__ Row(float cs_, float m, uint32_t table) : cs(cs_), c0(11.39231742277876f - m), c0p(13.39231742277876f - m), lg2_at(table) {}
-  static __device__ __forceinline__ constexpr bool by_poly(int g) { return ((D == 128 ? 0x14 : 0x92) >> g) & 1; }
+  static __device__ __forceinline__ constexpr bool by_poly(int g) { return POLY && (((D == 128 ? 0x14 : 0x92) >> g) & 1); }
   // factor bytes of groups g and g + 1 (maxima mx) into their words, and the exponents' offsets
   __device__ __forceinline__ void factors(int g, const float (&mx)[8], uint32_t (&sfw)[2], float (&off)[8]) const {
     const float p0 = ex2_approx(fmaf(mx[g], cs, c0)), p1 = ex2_approx(fmaf(mx[g + 1], cs, c0));

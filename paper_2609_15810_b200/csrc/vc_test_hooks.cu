@@ -21,14 +21,14 @@ __global__ void expcast_codes_kernel(const float* __restrict__ s, int64_t n4, fl
 }
 
 // NVFP4 probabilities of rows of 128 scores under their running maxima, one thread per row as in the softmax stage.
-template <int D>
+template <int D, bool POLY>
 __global__ void __launch_bounds__(128) nvfp4_codes_kernel(const float* __restrict__ s, const float* __restrict__ m, int64_t rows, float cs,
                                                           uint4* __restrict__ codes, uint2* __restrict__ factors) {
   __shared__ float table[128];
   table[threadIdx.x] = nvfp4::log2_entry(threadIdx.x);
   __syncthreads();
   for (int64_t r = (int64_t)blockIdx.x * 128 + threadIdx.x; r < rows; r += (int64_t)gridDim.x * 128) {
-    const nvfp4::Row<D> nv(cs, m[r], smem_u32(table));
+    const nvfp4::Row<D, POLY> nv(cs, m[r], smem_u32(table));
     const float4* src = reinterpret_cast<const float4*>(s + 128 * r);
     uint32_t sv[4][32], sfw[2] = {0u, 0u};
     float mx[8], off[8];
@@ -60,14 +60,15 @@ __global__ void __launch_bounds__(128) nvfp4_codes_kernel(const float* __restric
 }  // namespace
 }  // namespace vc
 
-extern "C" vc_status vc_test_nvfp4_codes(const float* s, const float* m, int64_t rows, int32_t d, float cs, uint8_t* codes,
-                                         uint8_t* factors, void* stream) {
+extern "C" vc_status vc_test_nvfp4_codes(const float* s, const float* m, int64_t rows, int32_t d, int32_t polynomial, float cs,
+                                         uint8_t* codes, uint8_t* factors, void* stream) {
   if (rows < 0 || (d != 64 && d != 128) || !(cs > 0.f)) return VC_ERR_INVALID_ARG;
   if (rows == 0) return VC_OK;
   if (!s || !m || !codes || !factors || (((uintptr_t)s | (uintptr_t)m | (uintptr_t)codes | (uintptr_t)factors) & 15)) return VC_ERR_INVALID_ARG;
   const int blocks = (int)((rows + 127) / 128 < 4096 ? (rows + 127) / 128 : 4096);
-  (d == 128 ? vc::nvfp4_codes_kernel<128> : vc::nvfp4_codes_kernel<64>)<<<blocks, 128, 0, (cudaStream_t)stream>>>(
-      s, m, rows, cs, reinterpret_cast<uint4*>(codes), reinterpret_cast<uint2*>(factors));
+  const auto kernel = polynomial ? (d == 128 ? vc::nvfp4_codes_kernel<128, true> : vc::nvfp4_codes_kernel<64, true>)
+                                 : (d == 128 ? vc::nvfp4_codes_kernel<128, false> : vc::nvfp4_codes_kernel<64, false>);
+  kernel<<<blocks, 128, 0, (cudaStream_t)stream>>>(s, m, rows, cs, reinterpret_cast<uint4*>(codes), reinterpret_cast<uint2*>(factors));
   vc::count_launches(1);
   return cudaGetLastError() == cudaSuccess ? VC_OK : VC_ERR_CUDA;
 }

@@ -11,7 +11,12 @@ import pytest
 import torch
 
 import paper_2609_15810_b200 as vc
+import vc_inputs
+from paper_2609_15810_b200.binding import Params, alloc_buffers
+from oracle import attention as OA
 from oracle import codecs as OC
+
+import helpers as Hh
 
 pytestmark = pytest.mark.gpu
 
@@ -35,12 +40,13 @@ def _rows(rows, cs, seed):
     return s, m
 
 
+@pytest.mark.parametrize("polynomial", [True, False])
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("cs", [3.1e-5, 0.37, 1.0 / 128.0, 7.7e-4])
-def test_codes_and_factors(d, cs):
+def test_codes_and_factors(d, cs, polynomial):
     rows = 4100                                              # (more than a block, a ragged last one)
     s, m = _rows(rows, cs, d)
-    codes, factors = [t.cpu().numpy() for t in vc.vc_test_nvfp4_codes(torch.from_numpy(s).cuda(), torch.from_numpy(m).cuda(), d, cs)]
+    codes, factors = [t.cpu().numpy() for t in vc.vc_test_nvfp4_codes(torch.from_numpy(s).cuda(), torch.from_numpy(m).cuda(), d, cs, polynomial)]
     codes = np.stack([codes & 15, codes >> 4], axis=2).reshape(rows, 8, 16)
     with np.errstate(divide="ignore", invalid="ignore", over="ignore"):
         z = (s.astype(np.float64) * float(np.float32(cs))).reshape(rows, 8, 16)
@@ -73,3 +79,20 @@ def test_hook_rejects_bad_arguments():
         with pytest.raises(vc.VcError):
             vc.vc_test_nvfp4_codes(s, m, d, cs)
     assert vc.vc_test_nvfp4_codes(s[:0], m[:0], 64, 1.0)[0].numel() == 0
+
+
+# five key tiles (no polynomial) and six (the sixth with one key)
+@pytest.mark.parametrize("grid", [(4, 10, 16), (1, 1, 641)])
+@pytest.mark.parametrize("v_smooth", [True, False])
+@pytest.mark.parametrize("d", [64, 128])
+def test_outputs_on_both_sides_of_the_line(grid, v_smooth, d):
+    H, N = 2, grid[0] * grid[1] * grid[2]
+    q, k, v = [t.cuda() for t in vc_inputs.make_qkv(vc_inputs.Workload("t", 1, H, N, d, grid, (8,), 91, "gauss"))]
+    p = Params.make(1, H, N, d, grid, bits=4, flags=vc.VC_FLAG_ALL if v_smooth else vc.VC_FLAG_ALL & ~vc.VC_FLAG_V_SMOOTH)
+    quant, work = alloc_buffers(p)
+    o = torch.empty(1, H, N, d, dtype=torch.bfloat16, device="cuda")
+    vc.vc_attn(p, q, k, v, None, o, quant, work)
+    vc.vc_poll_status(work)
+    for h in range(H):
+        bundle, cfg = Hh.oracle_prep(p, q, k, v, None, 0, h)
+        Hh.check_output(o[0, h].float().cpu().numpy(), OA.emulate_head(bundle, cfg), float(v[0, h].float().abs().max()))
